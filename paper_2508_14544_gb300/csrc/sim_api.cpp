@@ -327,8 +327,7 @@ int sim_load(sim_ctx *c, int32_t n, const int32_t *a, const int32_t *s, const in
 
 // One launch of the simulation kernel over n_work instances (all, or the device list work_dev).
 // smem: the active sets in shared memory (else a global-memory workspace of n_max slots);
-// dense: the 12-warps-per-SM configuration (blocks of 4 warps, 384 shared-memory slots); not with
-// the instrumented kernel, which keeps its own register budget.
+// dense: kDenseCa shared-memory slots per warp, as many warps per SM as then fit.
 static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int32_t n_work, bool smem,
                       int warps_per_sm, bool dense = false) {
     cudaError_t e;
@@ -336,29 +335,27 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
     int n_sm = 0, smem_optin = 0;
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    dense = dense && smem && !c->count_work && !c->batch_time;
+    dense = dense && smem;
     int wpb = dense ? simgb::kDenseWarps : c->wpb;
     // no more instances than SMs: one warp per block, so that each instance gets an SM to itself
     // (64 instances of 10^5 requests: 1.5-3.7 % faster than four to a block on 16 SMs)
     if (!dense && !c->wpb_set && n_work <= n_sm) wpb = 1;
-    int ca = smem ? (dense ? simgb::kDenseCa : c->smem_ca) : ((std::max(c->n_max, 128) + 127) / 128) * 128;
-    size_t per_warp = simgb::warp_ws_bytes(ca);
+    simgb::RunParams p;
+    p.ca = smem ? (dense ? simgb::kDenseCa : c->smem_ca) : ((std::max(c->n_max, 128) + 127) / 128) * 128;
+    p.dcap = simgb::delta_cap(c->n_max);
+    p.use_smem = smem ? 1 : 0;
+    p.work_count = c->count_work ? c->d_wc : nullptr;
+    p.batch_time = c->batch_time ? c->d_bt : nullptr;
+    const size_t per_warp = simgb::ws_bytes(c->policy == SIM_AMIN, p.ca, p.dcap);
     size_t smem_bytes = 0;
+    int per_sm = std::max(1, 16 / wpb);
     if (smem) {
         while (wpb > 1 && per_warp * wpb > size_t(smem_optin)) --wpb;
         if (per_warp * wpb > size_t(smem_optin)) return fail(c, SIM_E_INVAL, "workspace does not fit shared memory");
         smem_bytes = per_warp * wpb;
-        e = simgb::set_run_smem_limit(c->policy, smem_bytes);
-        if (e != cudaSuccess) return cuda_fail(c, e, "cudaFuncSetAttribute");
-    }
-    int per_sm = 1;
-    if (smem) {
-        int smem_sm = 0;
-        cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        per_sm = std::max(1, int(size_t(smem_sm) / (smem_bytes + 1024)));
-        per_sm = std::min(per_sm, dense ? 3 : 64 / wpb);
-    } else {
-        per_sm = std::max(1, 16 / wpb);
+        e = simgb::run_blocks_per_sm(c->policy, p, wpb, smem_bytes, &per_sm);
+        if (e != cudaSuccess) return cuda_fail(c, e, "sim_run: kernel set-up");
+        per_sm = std::max(per_sm, 1);
     }
     if (warps_per_sm > 0 && !dense) per_sm = std::max(1, std::min(per_sm, warps_per_sm / wpb));
     int64_t blocks = int64_t(n_sm) * per_sm;
@@ -384,7 +381,6 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
             c->gws_bytes = need;
         }
     }
-    simgb::RunParams p;
     p.M = c->M;
     p.n_work = n_work;
     p.work = work_dev;
@@ -396,10 +392,6 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
     p.completion = c->record_completions ? c->d_comp : nullptr;
     p.lu = c->d_lu;
     p.tie_seed = c->d_seed;
-    p.work_count = c->count_work ? c->d_wc : nullptr;
-    p.batch_time = c->batch_time ? c->d_bt : nullptr;
-    p.ca = ca;
-    p.use_smem = smem ? 1 : 0;
     p.debug = c->debug_checks;
     p.evict_index = c->evict_index;
     p.gws = c->d_gws;
@@ -408,7 +400,7 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
     p.main_cap = main_cap;
     if ((e = cudaMemsetAsync(c->d_counter, 0, sizeof(int32_t), st)) != cudaSuccess)
         return cuda_fail(c, e, "cudaMemsetAsync");
-    e = simgb::launch_run(c->policy, p, int(blocks), wpb, smem_bytes, dense, st);
+    e = simgb::launch_run(c->policy, p, int(blocks), wpb, smem_bytes, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "sim_run: kernel launch");
     ++c->launches;
     return SIM_OK;

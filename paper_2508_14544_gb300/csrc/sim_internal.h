@@ -34,8 +34,6 @@ struct InstInfo {
     int64_t cap;      // step cap
     int32_t n;        // number of requests
     int32_t status;   // 0 or a sim_status from validation
-    int32_t lmax;     // largest u_i or o_i of the instance (bounds every projected length)
-    int32_t pad;
 };
 
 struct DevResult {
@@ -76,7 +74,8 @@ struct RunParams {
                                // evaluations of the per-step method, global bytes moved by the queue
     int64_t *batch_time;       // optional, 6 per instance: the batch-time sums X0..X3, F2, F3
     // workspace
-    int32_t ca;                // active-set capacity per instance (multiple of 32)
+    int32_t ca;                // active-set capacity per instance (multiple of 64)
+    int32_t dcap;              // delta-queue capacity per warp slot (at most kDcap)
     int32_t use_smem;          // 1: active set + delta queue in shared memory; 0: global workspace
     int32_t debug;             // 1: check the simulation state's invariants every iteration (global kernel)
     int32_t evict_index;       // 1: A_min eviction ties by request index instead of the random tie key
@@ -86,20 +85,34 @@ struct RunParams {
     int64_t main_cap;
 };
 
-size_t warp_ws_bytes(int ca);  // workspace bytes per warp slot for ca active-set slots
-
-cudaError_t launch_stage(const StageParams &p, cudaStream_t st);
-// dense: the 12-warps-per-SM copy of the plain shared-memory kernel (blocks of 4 warps, kDenseCa slots)
-cudaError_t launch_run(int policy, const RunParams &p, int blocks, int warps_per_block, size_t smem_bytes, bool dense,
-                       cudaStream_t st);
 constexpr int kDenseCa = 384;      // active-set slots per warp of the dense configuration
 constexpr int kDenseWarps = 4;     // warps per block of the dense configuration
 constexpr int kSmemCaDefault = 512;  // active-set slots per warp in shared memory by default
-constexpr int kDcap = 256;         // delta-queue capacity per warp slot (multiple of 32)
+constexpr int kDcap = 256;         // largest delta-queue capacity (multiple of 32)
+constexpr int kMc = 64;            // cached entries of the main queue (two per lane)
+
+// Delta-queue entries used for an instance of n requests.
+__host__ __device__ constexpr int delta_cap(int64_t n) { return n <= 1024 ? 64 : (n <= 4096 ? 128 : kDcap); }
+
+// Workspace of one simulating warp: ca slots of {E, V, B, F} (16 bytes), the delta queue, the head
+// cache of the main queue (whose space also holds the merge histogram of dcap + 1 counters), {P, I} per
+// slot (8 bytes) and, under A_min, the estimate per slot (4 bytes).
+__host__ __device__ constexpr size_t ws_cache_bytes(int dcap) {
+    const size_t cache = size_t(kMc) * sizeof(QEnt), hist = (size_t(dcap + 1) * 4 + 15) & ~size_t(15);
+    return cache > hist ? cache : hist;
+}
+__host__ __device__ constexpr size_t ws_bytes(bool amin, int ca, int dcap) {
+    return size_t(ca) * (amin ? 28 : 24) + size_t(dcap) * sizeof(QEnt) + ws_cache_bytes(dcap);
+}
+
+cudaError_t launch_stage(const StageParams &p, cudaStream_t st);
+// Blocks of the kernel that p selects that one SM holds at a time; raises its shared-memory limit.
+cudaError_t run_blocks_per_sm(int policy, const RunParams &p, int warps_per_block, size_t smem_bytes, int *blocks);
+cudaError_t launch_run(int policy, const RunParams &p, int blocks, int warps_per_block, size_t smem_bytes,
+                       cudaStream_t st);
 cudaError_t launch_ratio(const DevResult *pol, const DevResult *ref, double *out, int32_t n, cudaStream_t st);
 cudaError_t launch_batch_time(const int64_t *sums, const DevResult *res, const double *coef, double *out, int32_t n,
                               cudaStream_t st);
-cudaError_t set_run_smem_limit(int policy, size_t bytes);
 cudaError_t launch_lemma(int32_t n_hist, int32_t len, int32_t l, double s, const double *x, double *out,
                          cudaStream_t st);
 cudaError_t launch_rho(int32_t n_u, const int32_t *us, double *out, double *scratch, int64_t stride,

@@ -36,20 +36,11 @@ constexpr int64_t kNaMaxPerInstance = 2048;       // requests per instance
 constexpr int kNaWarpsPerBlock = 4;
 constexpr int kNaBlocks = 32;
 constexpr int64_t kNaSlots = int64_t(kNaBlocks) * kNaWarpsPerBlock;  // simulating warps
-constexpr int kNaDeltaCap = simgb::kDcap;
 
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Workspace bytes per warp for an active-set capacity of kNaMaxPerInstance (same formula as the
-// simulation kernel's carve: 6 x ca + 2 x (ca + 4) int32, 16-byte aligned, then the delta queue
-// and the main-queue head cache, and the int32 scratch of the window and the merge histogram).
-// A run-time check compares it with the kernel's own size.
-constexpr size_t ws_bytes_max() {
-    size_t b = size_t(6) * kNaMaxPerInstance * 4 + size_t(2) * (kNaMaxPerInstance + 4) * 4;
-    b = (b + 15) & ~size_t(15);
-    b += size_t(kNaDeltaCap + 64) * sizeof(simgb::QEnt) + size_t(kNaDeltaCap + 4 + 68) * 4;
-    return (b + 15) & ~size_t(15);
-}
+// Workspace bytes per warp for an active-set capacity of kNaMaxPerInstance.
+constexpr size_t ws_bytes_max() { return simgb::ws_bytes(true, int(kNaMaxPerInstance), simgb::kDcap); }
 
 constexpr size_t kOffOff = 0;
 constexpr size_t kOffRec = align256(kOffOff + size_t(kNaMaxInstances + 1) * sizeof(int64_t));
@@ -97,8 +88,6 @@ extern "C" int sim_run_noalloc(int policy, int64_t M, int32_t n_instances, const
     if (nt > 0 && (!arrival_t || !prompt_s || !lower_l || !upper_u || !true_o))
         return fail(SIM_E_INVAL, "sim_run_noalloc: NULL input array");
 
-    if (simgb::warp_ws_bytes(int(kNaMaxPerInstance)) > ws_bytes_max())
-        return fail(SIM_E_STATE, "sim_run_noalloc: workspace layout mismatch");
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess || dev < 0 || dev >= kMaxDevices) return fail(SIM_E_CUDA, "sim_run_noalloc: cudaGetDevice failed");
@@ -163,6 +152,7 @@ extern "C" int sim_run_noalloc(int policy, int64_t M, int32_t n_instances, const
     p.work_count = nullptr;
     p.batch_time = nullptr;
     p.ca = int32_t(((std::max<int64_t>(n_max, 128) + 127) / 128) * 128);  // >= any active set: no fallback
+    p.dcap = simgb::kDcap;
     p.use_smem = 0;
     p.debug = 0;
     p.evict_index = 0;
@@ -171,7 +161,7 @@ extern "C" int sim_run_noalloc(int policy, int64_t M, int32_t n_instances, const
     p.mainbuf = reinterpret_cast<simgb::QEnt *>(base + kOffMain);
     p.main_cap = kNaMaxPerInstance;
     const int blocks = int(std::min<int64_t>(kNaBlocks, (n_instances + kNaWarpsPerBlock - 1) / kNaWarpsPerBlock));
-    e = simgb::launch_run(policy, p, blocks, kNaWarpsPerBlock, 0, false, st);
+    e = simgb::launch_run(policy, p, blocks, kNaWarpsPerBlock, 0, st);
     if (e != cudaSuccess) return fail(SIM_E_CUDA, "sim_run_noalloc: simulation kernel launch failed");
     return SIM_OK;
 }

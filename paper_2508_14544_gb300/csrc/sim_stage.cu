@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageParams S, int np) 
     // instance before anything is written: it is staged as empty with status INVAL
     const bool oob = base < 0 || n64 < 0 || n64 > S.max_n || base + n64 > S.max_total;
     const int n = oob ? 0 : int(n64);
-    int64_t bad_inval = oob ? 1 : 0, bad_inf = 0, sum_a = 0, sum_o = 0, lmax = 0, kmax = 0, amax = 0;
+    int64_t bad_inval = oob ? 1 : 0, bad_inf = 0, sum_a = 0, sum_o = 0, kmax = 0, amax = 0;
     const bool in_smem = n <= np;
     int32_t *kk = reinterpret_cast<int32_t *>(stage_smem);
     int32_t *ka = kk + np;
@@ -226,7 +226,6 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageParams S, int np) 
         }
         sum_a += a;
         sum_o += o;
-        lmax = max(lmax, int64_t(max(u, o)));
         kmax = max(kmax, int64_t(key));
         amax = max(amax, int64_t(a));
     }
@@ -234,7 +233,6 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageParams S, int np) 
     bad_inf = block_reduce<int64_t>(bad_inf, sh64, true);
     sum_a = block_reduce<int64_t>(sum_a, sh64, false);
     sum_o = block_reduce<int64_t>(sum_o, sh64, false);
-    lmax = block_reduce<int64_t>(lmax, sh64, true);
     if (in_smem) {
         kmax = block_reduce<int64_t>(kmax, sh64, true);
         amax = block_reduce<int64_t>(amax, sh64, true);
@@ -249,8 +247,6 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageParams S, int np) 
         in.status = status;
         in.sum_a = sum_a;
         in.cap = S.step_cap > 0 ? S.step_cap : 64 * (int64_t(n) + sum_o);
-        in.lmax = int32_t(lmax);
-        in.pad = 0;
         S.info[inst] = in;
     }
     __syncthreads();
