@@ -344,6 +344,7 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
     p.ca = smem ? (dense ? simgb::kDenseCa : c->smem_ca) : ((std::max(c->n_max, 128) + 127) / 128) * 128;
     p.dcap = simgb::delta_cap(c->n_max);
     p.use_smem = smem ? 1 : 0;
+    p.wide = dense ? 0 : 1;
     p.work_count = c->count_work ? c->d_wc : nullptr;
     p.batch_time = c->batch_time ? c->d_bt : nullptr;
     const size_t per_warp = simgb::ws_bytes(c->policy == SIM_AMIN, p.ca, p.dcap);

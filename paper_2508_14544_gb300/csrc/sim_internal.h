@@ -77,6 +77,7 @@ struct RunParams {
     int32_t ca;                // active-set capacity per instance (multiple of 64)
     int32_t dcap;              // delta-queue capacity per warp slot (at most kDcap)
     int32_t use_smem;          // 1: active set + delta queue in shared memory; 0: global workspace
+    int32_t wide;              // 1: the copy with more registers a thread and at most 12 warps per SM
     int32_t debug;             // 1: check the simulation state's invariants every iteration (global kernel)
     int32_t evict_index;       // 1: A_min eviction ties by request index instead of the random tie key
     unsigned char *gws;        // global workspace base (use_smem == 0)
@@ -95,11 +96,11 @@ constexpr int kMc = 64;            // cached entries of the main queue (two per 
 __host__ __device__ constexpr int delta_cap(int64_t n) { return n <= 1024 ? 64 : (n <= 4096 ? 128 : kDcap); }
 
 // Workspace of one simulating warp: ca slots of {E, V, B, F} (16 bytes), the delta queue, the head
-// cache of the main queue (whose space also holds the merge histogram of dcap + 1 counters), {P, I} per
+// cache of the main queue (whose space also holds the dcap positions of a merge), {P, I} per
 // slot (8 bytes) and, under A_min, the estimate per slot (4 bytes).
 __host__ __device__ constexpr size_t ws_cache_bytes(int dcap) {
-    const size_t cache = size_t(kMc) * sizeof(QEnt), hist = (size_t(dcap + 1) * 4 + 15) & ~size_t(15);
-    return cache > hist ? cache : hist;
+    const size_t cache = size_t(kMc) * sizeof(QEnt), pos = size_t(dcap) * 4;
+    return cache > pos ? cache : pos;
 }
 __host__ __device__ constexpr size_t ws_bytes(bool amin, int ca, int dcap) {
     return size_t(ca) * (amin ? 28 : 24) + size_t(dcap) * sizeof(QEnt) + ws_cache_bytes(dcap);

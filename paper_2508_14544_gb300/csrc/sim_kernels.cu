@@ -1,4 +1,4 @@
-// Simulation kernel of the batched scheduler simulator (sm_103a): k_run<policy, shared, instrumented>.
+// Simulation kernel of the batched scheduler simulator (sm_103a): k_run<policy, shared, instrumented, wide>.
 //
 // One warp simulates one instance at a time (persistent warps pull instance ids from a work
 // queue).  Each step follows the paper's algorithms:
@@ -20,8 +20,8 @@
 // Active set (per warp, shared memory; a global-memory workspace of the same layout serves
 // instances that outgrow it): an unordered array of slots, a job keeps its slot until it ends.
 //   E = p + Lhat - 1   projected last step (Lhat = u, o or the A_min estimate)
-//   V                  projected memory of the whole set at step E, kept up to date (valid while
-//                      E >= t)
+//   W = V(E) + E       V(E) the projected memory of the whole set at step E, kept up to date (valid
+//                      while E >= t)
 //   B = s - p + 1      the job's memory at step x is B + x
 //   F = p + o - 1      true last step (completion at step F, C = F + 1)
 //   P = p, I = request index, K = the estimate (A_min cancellation key)
@@ -30,15 +30,16 @@
 // (B_j + x) the projected memory of the set at step x (eq. Constraint restricted to S'), a
 // candidate (prompt s, estimate L) started at step t ends at y = t + L - 1 and fits iff
 //   (1) need + s + 1 <= M, need = sum of (B_j + t), the memory of the coming step,
-//   (2) V_i + s + 1 + (E_i - t) <= M for every active endpoint t <= E_i <= y,
+//   (2) V(E_i) + s + 1 + (E_i - t) <= M, i.e. W_i <= M - s - 1 + t, for every active endpoint
+//       t <= E_i <= y,
 //   (3) V(y) + s + L <= M at its own last step.
 // Between endpoints V(x) grows, so these points decide every future step.  (2) and (3) are one pass
 // over the slots and three warp reductions.  A job (E, B) that joins or leaves adds or subtracts
-// B + E_i at every endpoint E_i <= E: that update is left pending and applied by the next pass that
+// B + E_i in W_i at every endpoint E_i <= E: that update is left pending and applied by the next pass that
 // tests a candidate, so an admission costs one pass, and a job that leaves at or after its E
-// (every H-SF, A_r and A_min completion, every A_ell promotion) changes no V at all.  There are no
+// (every H-SF, A_r and A_min completion, every A_ell promotion) changes no W at all.  There are no
 // sorted arrays, prefix sums or moves; freed slots are reclaimed by a compaction once they outnumber
-// half of the live ones.  A candidate that fails also yields the first later step at which (2) and
+// half of the live ones.  A candidate that fails yields the first later step at which (2) and
 // (3) could hold with the set unchanged; the steps up to the next event (that step, a completion, an
 // arrival, an A_min overflow, an A_ell promotion) are processed in closed form.
 //
@@ -60,10 +61,14 @@ enum { ST_OK = 0, ST_INVAL = -1, ST_STEPCAP = -3, ST_STATE = -5 };
 // Loops whose trip count is known only at run time carry `#pragma unroll 1`: unrolled copies grow
 // the simulation loop, which the warps of a scheduler share through its instruction cache.
 constexpr int kPage = 128;  // active-set slots per pass iteration (four per lane)
+constexpr int kHalf = 64;   // sets whose slots end here are passed over in one half page (two per lane)
 // s of the entry that stands for the head of an empty queue: never fits, greater than every entry
 constexpr int kNoHead = 1 << 28;
 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
+__device__ __forceinline__ int64_t warp_slot() {
+    return int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+}
 
 // Random tie key of request i at step t for A_min's cancellation order: the high 32 bits of
 // output number t * 2^32 + i + 1 of the SplitMix64 generator seeded with `seed` (Steele, Lea and
@@ -87,6 +92,20 @@ __device__ __forceinline__ bool qless(const QEnt &a, const QEnt &b) {
     return a.key < b.key || (a.key == b.key && a.idx < b.idx);
 }
 
+// floor(a / b) for 0 <= a < 2^22, b >= 1, by a reciprocal and one correction each way (the estimate is
+// off by less than one); a lower bound of it for larger a (there the estimate is off by less than 40).
+// About half the latency of the integer division.
+__device__ __forceinline__ int quotient_lb(int a, int b) {
+    int q = __float2int_rz(__fdividef(float(a), float(b)));
+    if (a >= (1 << 22)) return max(q - 40, 0);
+    const int r = a - q * b;
+    if (r < 0) --q;
+    if (r >= b) ++q;
+    return q;
+}
+
+__device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
 // Projected length of a queue entry.  For A_max, A_min and H-SF the sort key is that length; A_r
 // projects the true length o and A_ell the current estimate (l before a promotion, u after:
 // promotions have odd keys).
@@ -100,51 +119,16 @@ __device__ __forceinline__ int proj_len(const RunParams &P, int64_t base, const 
     return e.key;
 }
 
-// Number of leading positions i in [0, len) with pred(i) true (pred true on a prefix); warp-wide.
-template <class Pred>
-__device__ __forceinline__ int warp_prefix_count(int len, Pred pred) {
-    if (len <= 0) return 0;
-    const int lane = lane_id();
-    const int c = (len + 31) >> 5;
-    const int pos = min((lane + 1) * c - 1, len - 1);
-    const int full = __popc(__ballot_sync(FULL, pred(pos)));
-    int cnt = full * c;
-    if (cnt >= len) return len;
-    const int end = min(cnt + c, len);
-    #pragma unroll 1
-    for (int off = cnt; off < end; off += 32) {
-        const int i = off + lane;
-        const unsigned b = __ballot_sync(FULL, i < end && pred(i));
-        const int k = __popc(b);
-        cnt += k;
-        if (k < 32) break;
-    }
-    return cnt;
-}
-
-// The same, computed by one lane alone (binary search).
-template <class Pred>
-__device__ __forceinline__ int lane_prefix_count(int len, Pred pred) {
-    int lo = 0, hi = len;
-    #pragma unroll 1
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (pred(mid)) lo = mid + 1; else hi = mid;
-    }
-    return lo;
-}
-
 // ---------------------------------------------------------------------------------------------
 // Per-warp workspace (layout: ws_bytes in sim_internal.h)
 // ---------------------------------------------------------------------------------------------
 struct Ws {
-    int4 *H;         // active-set slots {E, V, B, F}, capacity ca (a multiple of kPage)
+    int4 *H;         // active-set slots {E, W, B, F}, capacity ca (a multiple of kPage)
     QEnt *dq;        // delta queue, dcap entries, sorted DESCENDING (head = dq[dn-1])
     QEnt *mc;        // cached head of the main queue, kMc entries
-    int32_t *cnt;    // merge histogram, dcap + 1 entries: the cache's space (a merge invalidates it)
+    int32_t *cnt;    // merge positions, dcap entries: the cache's space (a merge invalidates it)
     int2 *C;         // {P, I} per slot
     unsigned *K;     // A_min: the estimate per slot, UINT_MAX in a free one
-    QEnt *mb0, *mb1;  // global ping-pong main-queue buffers
     int32_t ca, dcap;
 };
 
@@ -161,32 +145,27 @@ __device__ __forceinline__ Ws carve_ws(unsigned char *base, int ca, int dcap) {
     return w;
 }
 
-// Position of the job A_min cancels when several jobs share the smallest estimate mk: the smallest
-// (tie key, index) among them, the tie key drawn from `base` (tie_base of the step) or, under the
-// index rule, the index itself.  Warp-wide; every lane gets the position.  Out of line: ties are a
-// small share of the cancellations, and keeping the hashing out of the simulation loop keeps that
-// loop's code small.
-__device__ __noinline__ int tie_position(const unsigned *K, const int2 *C, int end, unsigned mk, uint64_t base,
-                                         int rnd) {
-    const int lane = lane_id();
+// Position of the job A_min cancels when several jobs share the smallest estimate mk, the first of them
+// at slot `first` and the last at `last`: the smallest (tie key, index) among them, the tie key drawn
+// from `base` (tie_base of the step) or, under the index rule, the index itself.  Warp-wide; every
+// lane gets the position.
+__device__ __forceinline__ int tie_position(const unsigned *K, const int2 *C, int first, int last, unsigned mk,
+                                            uint64_t base, int rnd) {
     unsigned br = UINT_MAX, bi = UINT_MAX;
-    int bp = -1;
+    int bp = 0;
     #pragma unroll 1
-    for (int i = lane; i < end; i += 32) {
-        if (K[i] == mk) {
-            const unsigned id = unsigned(C[i].y);
-            const unsigned r = rnd ? tie_key(base, int(id)) : id;
-            if (r < br || (r == br && id < bi)) {
-                br = r;
-                bi = id;
-                bp = i;
-            }
-        }
+    for (int b = first & ~31; b <= last; b += 32) {
+        const int i = b + lane_id();
+        const unsigned id = unsigned(C[i].y);
+        const unsigned r = rnd ? tie_key(base, int(id)) : id;
+        const bool less = K[i] == mk && (r < br || (r == br && id < bi));
+        br = less ? r : br;
+        bi = less ? id : bi;
+        bp = less ? i : bp;
     }
     const unsigned mr = __reduce_min_sync(FULL, br);
     const unsigned mi = __reduce_min_sync(FULL, br == mr ? bi : UINT_MAX);
-    const unsigned b = __ballot_sync(FULL, bp >= 0 && br == mr && bi == mi);
-    return b ? __shfl_sync(FULL, bp, __ffs(b) - 1) : -1;
+    return int(__reduce_min_sync(FULL, br == mr && bi == mi ? unsigned(bp) : UINT_MAX));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -223,10 +202,14 @@ __device__ __forceinline__ void main_cache_at_head(const Ws &w, Queue &q, int64_
 }
 
 // Merge the delta into the main array (into the other ping-pong buffer).  Rare (a full delta, or
-// a long arrival run), so it is kept out of line: the simulation loop stays small enough for the
-// instruction cache when two warps share a scheduler.  Takes the few workspace pointers it needs
-// by value and the queue by pointer; gb (null in the plain kernel) counts the global bytes moved.
-__device__ __noinline__ void merge_delta(int32_t *cnt, const QEnt *dq, QEnt *mb0, QEnt *mb1, Queue *qp, int64_t *gb) {
+// a long arrival run), so it is kept out of line.  Takes the few workspace pointers it needs by value and
+// the queue by pointer; gb (null in the plain kernel) counts the global bytes moved.
+// The delta is short and the main array long (up to the instance's requests): each delta entry finds
+// its place in the main array by binary search, two searches per lane in flight, and the main array is
+// then copied in coalesced runs of 128 entries, shifted by the number of delta entries before each.
+// (More in flight costs registers, which count toward the simulation loop's: eight loads instead of four
+// made the loop spill and every policy 25-60 % slower.)
+__device__ __noinline__ void merge_delta(int32_t *pos, const QEnt *dq, QEnt *mb0, QEnt *mb1, Queue *qp, int64_t *gb) {
     const int lane = lane_id();
     Queue q = *qp;
     const int dn = q.dn;
@@ -234,45 +217,53 @@ __device__ __noinline__ void merge_delta(int32_t *cnt, const QEnt *dq, QEnt *mb0
     QEnt *out = (q.mbuf == 0) ? mb1 : mb0;
     const QEnt *X = q.mq + q.mh;
     #pragma unroll 1
-    for (int j = lane; j <= dn; j += 32) cnt[j] = 0;
-    __syncwarp();
-    const int c = (nx + 31) >> 5;
-    const int s0 = lane * c;
-    const int s1 = min(s0 + c, nx);
-    if (s0 < s1) {
-        const QEnt x0 = X[s0];
-        int r = lane_prefix_count(dn, [&](int m) { return qless(dq[dn - 1 - m], x0); });
-        int run_r = r, run_len = 0;
+    for (int j0 = lane; j0 < dn; j0 += 64) {
+        const int j1 = j0 + 32;
+        const int2 d0 = *reinterpret_cast<const int2 *>(&dq[dn - 1 - j0]);
+        const int2 d1 = *reinterpret_cast<const int2 *>(&dq[j1 < dn ? dn - 1 - j1 : 0]);
+        int lo0 = 0, hi0 = nx, lo1 = 0, hi1 = nx;
         #pragma unroll 1
-        for (int i = s0; i < s1; ++i) {
-            const QEnt x = X[i];
-            #pragma unroll 1
-            while (r < dn && qless(dq[dn - 1 - r], x)) ++r;
-            out[i + r] = x;
-            if (r != run_r) {
-                if (run_len) atomicAdd(&cnt[run_r], run_len);
-                run_r = r;
-                run_len = 0;
+        while (lo0 < hi0 || lo1 < hi1) {
+            const int m0 = (lo0 + hi0) >> 1, m1 = (lo1 + hi1) >> 1;
+            const int2 x0 = *reinterpret_cast<const int2 *>(&X[min(m0, nx - 1)]);
+            const int2 x1 = *reinterpret_cast<const int2 *>(&X[min(m1, nx - 1)]);
+            const bool l0 = x0.x < d0.x || (x0.x == d0.x && x0.y < d0.y);
+            const bool l1 = x1.x < d1.x || (x1.x == d1.x && x1.y < d1.y);
+            if (lo0 < hi0) {
+                if (l0) lo0 = m0 + 1; else hi0 = m0;
             }
-            ++run_len;
+            if (lo1 < hi1) {
+                if (l1) lo1 = m1 + 1; else hi1 = m1;
+            }
         }
-        if (run_len) atomicAdd(&cnt[run_r], run_len);
+        pos[j0] = lo0;  // main entries before delta entry j (ascending)
+        out[lo0 + j0] = dq[dn - 1 - j0];
+        if (j1 < dn) {
+            pos[j1] = lo1;
+            out[lo1 + j1] = dq[dn - 1 - j1];
+        }
     }
     __syncwarp();
-    // delta element j (ascending) goes to j + #{main entries smaller} = j + sum_{r <= j} cnt[r]
-    int carry = 0;
+    int r = 0;  // delta entries before main entry b
     #pragma unroll 1
-    for (int c0 = 0; c0 < dn; c0 += 32) {
-        const int j = c0 + lane;
-        int v = (j < dn) ? cnt[j] : 0;
+    for (int b = 0; b < nx; b += 128) {
+        QEnt x[4];
+        int sh[4];
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int y = __shfl_up_sync(FULL, v, d);
-            if (lane >= d) v += y;
+        for (int k = 0; k < 4; ++k) {
+            const int i = b + 32 * k + lane;
+            if (i < nx) x[k] = X[i];
+            sh[k] = i + r;
         }
-        v += carry;
-        if (j < dn) out[j + v] = dq[dn - 1 - j];
-        carry = __shfl_sync(FULL, v, 31);
+        #pragma unroll 1
+        for (; r < dn && pos[r] < b + 128; ++r) {
+            const int p = pos[r];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sh[k] += p <= b + 32 * k + lane ? 1 : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (b + 32 * k + lane < nx) out[sh[k]] = x[k];
     }
     __syncwarp();
     __threadfence_block();
@@ -287,46 +278,56 @@ __device__ __noinline__ void merge_delta(int32_t *cnt, const QEnt *dq, QEnt *mb0
     *qp = q;
 }
 
-__device__ __forceinline__ void merge_delta(const Ws &w, Queue &q, int64_t *gb) {
+// The warp's ping-pong buffers are found from its slot here, not held in registers.
+__device__ __forceinline__ void merge_delta(const RunParams &P, const Ws &w, Queue &q, int64_t *gb) {
     Queue qq = q;
-    merge_delta(w.cnt, w.dq, w.mb0, w.mb1, &qq, gb);
+    QEnt *mb = P.mainbuf + warp_slot() * 2 * P.main_cap;
+    merge_delta(w.cnt, w.dq, mb, mb + P.main_cap, &qq, gb);
     q = qq;
 }
 
-// Insert one entry into the delta (merging the delta into main first if it is full: returns true).
-__device__ __forceinline__ bool delta_insert(const Ws &w, Queue &q, const QEnt &e, int64_t *gb) {
+// Insert one entry into the delta, which is not full.
+__device__ __forceinline__ void delta_put(const Ws &w, Queue &q, const QEnt &e) {
     const int lane = lane_id();
-    const bool full = q.dn == w.dcap;
-    if (full) merge_delta(w, q, gb);
     const int dn = q.dn;
     // the smaller entries move one place right: usually all of them are among the last 32
     const int base = max(dn - 32, 0), i0 = base + lane;
     const QEnt d = w.dq[i0];
     const bool in = i0 < dn;
     const unsigned gt = __ballot_sync(FULL, in && qless(e, d));
-    if (__reduce_max_sync(FULL, gt != 0u || base == 0)) {
+    if (gt != 0u || base == 0) {
         if (in && lane >= __popc(gt)) w.dq[i0 + 1] = d;
         w.dq[base + __popc(gt)] = e;
         __syncwarp();
         q.dn = dn + 1;
-        return full;
+        return;
     }
-    const int pos = warp_prefix_count(dn, [&](int i) { return qless(e, w.dq[i]); });  // #entries > e
+    // otherwise: its place by one count over the keys, and the entries behind it moved from the back
+    int greater = 0;
+    #pragma unroll 2
+    for (int i = lane; i < dn; i += 32) {
+        const int2 k = *reinterpret_cast<const int2 *>(&w.dq[i]);
+        greater += e.key < k.x || (e.key == k.x && e.idx < k.y) ? 1 : 0;
+    }
+    const int pos = int(__reduce_add_sync(FULL, unsigned(greater)));
     #pragma unroll 1
     for (int hi = dn; hi > pos; hi -= 32) {
-        const int lo = max(pos, hi - 32);
-        const int i = lo + lane;
+        const int i = hi - 32 + lane;
         QEnt v;
-        const bool act = i < hi;
-        if (act) v = w.dq[i];
+        if (i >= pos) v = w.dq[i];
         __syncwarp();
-        if (act) w.dq[i + 1] = v;
+        if (i >= pos) w.dq[i + 1] = v;
         __syncwarp();
     }
     w.dq[pos] = e;
     __syncwarp();
     q.dn = dn + 1;
-    return full;
+}
+
+// The same, merging the delta into main first if it is full.
+__device__ __forceinline__ void delta_insert(const RunParams &P, const Ws &w, Queue &q, const QEnt &e, int64_t *gb) {
+    if (q.dn == w.dcap) merge_delta(P, w, q, gb);
+    delta_put(w, q, e);
 }
 
 // Head of R_t (smallest (key, idx)) and which part holds it (src 0: main, 1: delta), or the kNoHead entry
@@ -352,8 +353,8 @@ __device__ __forceinline__ QEnt queue_head(const Ws &w, const Queue &q, int &src
 // is empty and extends it under A_ell when it follows it in the staged records (FIFO keys); a few
 // entries go into the delta one by one; a long batch is copied into the emptied delta in chunks.
 template <int POL>
-__device__ __forceinline__ void insert_run(const Ws &w, Queue &q, const QEnt *rec, int n, int ap, int ae, int64_t &gb,
-                                           int64_t *gbp) {
+__device__ __forceinline__ void insert_run(const RunParams &P, const Ws &w, Queue &q, const QEnt *rec, int n, int ap,
+                                           int ae, int64_t &gb, int64_t *gbp) {
     const int lane = lane_id();
     const int len = ae - ap;
     gb += int64_t(len) * int64_t(sizeof(QEnt));
@@ -379,10 +380,10 @@ __device__ __forceinline__ void insert_run(const Ws &w, Queue &q, const QEnt *re
         const int rem = len - done;
         if (rem <= 8) {
             #pragma unroll 1
-            for (int j = 0; j < rem; ++j) delta_insert(w, q, run[done + j], gbp);
+            for (int j = 0; j < rem; ++j) delta_insert(P, w, q, run[done + j], gbp);
             break;
         }
-        if (q.dn > 0) merge_delta(w, q, gbp);
+        if (q.dn > 0) merge_delta(P, w, q, gbp);
         const int k = min(rem, w.dcap);
         #pragma unroll 1
         for (int j = lane; j < k; j += 32) w.dq[j] = run[done + k - 1 - j];  // descending
@@ -392,20 +393,40 @@ __device__ __forceinline__ void insert_run(const Ws &w, Queue &q, const QEnt *re
     }
 }
 
-// A job (e, b) leaves the set: V loses b + E at the endpoints E <= e (free slots compare greater).
+template <int N>
+struct Slots {
+    static constexpr int value = N;
+};
+
+// body(Slots<N>, p) for the slots p + 32 j + lane, j < N, of every page in [0, end) (a half page when
+// the caller knows, as a warp-uniform condition, that end <= kHalf).
+template <class Body>
+__device__ __forceinline__ void over_slots(bool half, int end, Body body) {
+    if (half) {
+        body(Slots<kHalf / 32>(), 0);
+    } else {
+        #pragma unroll 1
+        for (int p = 0; p < end; p += kPage) body(Slots<kPage / 32>(), p);
+    }
+}
+
+// Passes (half pages) that over_slots makes over n slots.
+__device__ __forceinline__ int slot_pages(int n) { return n <= kHalf ? 1 : 2 * ((n + kPage - 1) / kPage); }
+
+// A job (e, b) leaves the set: W loses b + E at the endpoints E <= e (free slots compare greater).
 __device__ __forceinline__ void subtract_job(const Ws &w, int end, int e, int b) {
     #pragma unroll 1
     for (int p = 0; p < end; p += kPage) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int i = p + 32 * j + lane_id();
-            const int2 ev = *reinterpret_cast<const int2 *>(&w.H[i]);
-            if (unsigned(ev.x) <= unsigned(e)) w.H[i].y = ev.y - b - ev.x;
+            const int2 ew = *reinterpret_cast<const int2 *>(&w.H[i]);
+            if (unsigned(ew.x) <= unsigned(e)) w.H[i].y = ew.y - b - ew.x;
         }
     }
 }
 
-// Free slots [from, from + kPage).
+// Free the slots [from, from + kPage).
 template <int POL>
 __device__ __forceinline__ void free_page(const Ws &w, int from) {
 #pragma unroll
@@ -423,22 +444,30 @@ __device__ __forceinline__ void compact(const Ws &w, int &end) {
     const unsigned lt = (1u << lane) - 1u;
     int wpos = 0;
     #pragma unroll 1
-    for (int b = 0; b < end; b += 32) {
-        const int i = b + lane;
-        const int4 h = w.H[i];
-        const int2 c = w.C[i];
-        const unsigned k = POL == P_AMIN ? w.K[i] : 0u;
-        const bool live = i < end && h.w >= 0;
-        const unsigned m = __ballot_sync(FULL, live);
-        __syncwarp();
-        if (live) {
-            const int d = wpos + __popc(m & lt);
-            w.H[d] = h;
-            w.C[d] = c;
-            if (POL == P_AMIN) w.K[d] = k;
+    for (int b = 0; b < end; b += kHalf) {
+        int4 h[2];
+        int2 c[2];
+        unsigned k[2], m[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int i = b + 32 * j + lane;
+            h[j] = w.H[i];
+            c[j] = w.C[i];
+            k[j] = POL == P_AMIN ? w.K[i] : 0u;
+            m[j] = __ballot_sync(FULL, h[j].w >= 0);
         }
         __syncwarp();
-        wpos += __popc(m);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int d = wpos + __popc(m[j] & lt);
+            if (h[j].w >= 0) {
+                w.H[d] = h[j];
+                w.C[d] = c[j];
+                if (POL == P_AMIN) w.K[d] = k[j];
+            }
+            wpos += __popc(m[j]);
+        }
+        __syncwarp();
     }
     #pragma unroll 1
     for (int i = wpos + lane; i < end; i += 32) {
@@ -450,13 +479,13 @@ __device__ __forceinline__ void compact(const Ws &w, int &end) {
 }
 
 // Invariants of the simulation state between events (SIM_OPT_DEBUG_CHECKS; global-memory kernel
-// only): the live slots number A and sum to need; nextF is their smallest F; V is the projected memory
-// at every endpoint not yet passed (with the pending update); under A_max, H-SF and A_r no job runs
+// only): the live slots number A and sum to need; nextF is their smallest F; W is the projected memory
+// plus E at every endpoint not yet passed (with the pending updates); under A_max, H-SF and A_r no job runs
 // past its projected last step; free slots are free; the delta queue is strictly descending and the
 // cached head of the main array ascending.  Returns false on the first violation.
 template <int POL>
-__device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int need, int nextF, int py, int pm,
-                         int pc, int filled) {
+__device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int need, int nextF, int py, int pc,
+                         int qy, int qc, int filled) {
     const int lane = lane_id();
     bool bad = false;
     unsigned fmin = UINT_MAX;
@@ -475,11 +504,11 @@ __device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int
         if ((POL == P_AMAX || POL == P_HSF || POL == P_AR) && h.w > h.x) bad = true;
         if (POL == P_AMIN && w.K[i] != unsigned(h.x - w.C[i].x + 1)) bad = true;
         if (h.x < t) continue;
-        int v = 0;
+        int v = h.x;
         #pragma unroll 1
         for (int j = 0; j < end; ++j)
             if (w.H[j].x >= h.x) v += w.H[j].z + h.x;
-        if (v != h.y + (unsigned(h.x) <= unsigned(py) ? pm * h.x + pc : 0)) bad = true;
+        if (v != h.y + (h.x <= py ? h.x + pc : 0) - (h.x <= qy ? h.x + qc : 0)) bad = true;
     }
     if (int(__reduce_add_sync(FULL, unsigned(cnt))) != A || int(__reduce_add_sync(FULL, unsigned(sum))) != need) bad = true;
     #pragma unroll 1
@@ -499,8 +528,8 @@ __device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int
 // INS: the instrumented copy, which also keeps the work counters of the per-step method and the
 // batch-time sums; the plain copy has neither.
 // All memory sums are at most M <= 2^26 where they are compared (V, need and a candidate's points
-// belong to feasible schedules, a violated one exceeds M by one job's memory at most), so 32 bits
-// hold them; steps stay below kMaxStep + 2^26.
+// belong to feasible schedules, a violated one exceeds M by one job's memory at most) and a projected
+// step at most kMaxStep + 2^26, so 32 bits hold them and W <= 2^31 - 1.
 // ---------------------------------------------------------------------------------------------
 template <int POL, bool SMEM, bool INS>
 __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, int inst) {
@@ -520,14 +549,12 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
         return;
     }
     const int n = info.n;
-    const QEnt *rec = P.rec + info.base;
-    const int32_t *ra = P.rec_a + info.base;
+    const int64_t base = info.base;
     const uint64_t tie_seed = (POL == P_AMIN && P.tie_seed) ? P.tie_seed[inst] : 0ull;
     const int M = int(P.M);
-    const int64_t cap = info.cap;
 
     Queue q;
-    q.mq = rec;
+    q.mq = P.rec + base;
     q.mh = q.me = 0;
     q.lim = n;
     q.mbuf = -1;
@@ -541,7 +568,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
     // (A ceil(log2 A)^2), S5 endpoint evaluations of a binary-search admission
     // ((A' + k) ceil(log2(Q + 1))); k_step / ev_step: admitted / removed at the current step
     int64_t cS2 = 0, cS3 = 0, cS5 = 0;
-    int k_step = 0, ev_step = 0;
+    int k_step = 0, ev_step = 0, ovf_t = -1;
 
     // Batch time (Section 6's linear batch-time model, coefficients given later): bx0..bx3 =
     // X0..X3, the sums over requests of the processed steps, batch sizes, step memories and
@@ -552,20 +579,21 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
     int64_t bx0 = 0, bx1 = 0, bx2 = 0, bx3 = 0, bmem = 0, bpf = 0;
 
     // A live jobs in the slots [0, end), the slots [0, filled) initialised; need: the memory of step
-    // t; nextF, nextE: the smallest F and (A_ell) E; py, pm, pc: the pending update V += pm E + pc at
-    // the endpoints E <= py (pm = 0: none)
+    // t; nextF, nextE: the smallest F and (A_ell) E; pending updates: W += E + pc at the endpoints
+    // E <= py (the last job admitted) and W -= E + qc at those E <= qy (a job removed); -2: none
     int A = 0, end = 0, filled = kPage, need = 0;
     unsigned nextF = UINT_MAX, nextE = UINT_MAX;
-    int py = 0, pm = 0, pc = 0;
+    int py = -2, pc = 0, qy = -2, qc = 0;
+    constexpr bool kSub = POL != P_HSF && POL != P_AR;
     free_page<POL>(w, 0);
     // steps processed = t - tb (tb moves with every idle gap); the instance stops at step tstop (the
     // step cap or kMaxStep); trare = min(tstop, next arrival)
-    int t = ra[0], tb = t;
-    const auto stop_at = [&]() { return int(min(int64_t(tb) + min(cap, int64_t(INT_MAX)), int64_t(kMaxStep) + 1)); };
+    int t = P.rec_a[base], tb = t;
+    const auto stop_at = [&]() { return int(min(int64_t(tb) + min(P.info[inst].cap, int64_t(INT_MAX)), int64_t(kMaxStep) + 1)); };
     int tstop = stop_at();
     // arrival steps of the records [apb, apb + 32), one per lane
     int ap = 0, apb = 0, next_a = t, trare = t;
-    int pa = lane < n ? ra[lane] : INT_MAX;
+    int pa = lane < n ? P.rec_a[base + lane] : INT_MAX;
     int64_t sumC = 0, rsteps = 0, nev = 0;
     // 32 bits suffice (fewer live registers): makespan <= t + 1 with t <= kMaxStep + 1, and the peak
     // is a step's memory, <= M <= 2^26
@@ -581,13 +609,13 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
     h.o = 0;
     int hL = 1, hsrc = 0, fit_lb = 0;
     // what the next iteration has to look at first
-    enum { HEAD = 1, NEXTF = 2, SLOTS = 4, IDLE = 8 };
+    enum { HEAD = 1, NEXTF = 2, SLOTS = 4, IDLE = 8, MERGE = 16 };
     int attn = 0;
 
     const auto load_head = [&](bool cached) {  // cached: w.mc covers q.mh (else h is reloaded before use)
         h = queue_head(w, q, hsrc);
         hL = h.key;
-        if (POL == P_AR || POL == P_AELL) hL = cached && h.s != kNoHead ? proj_len<POL>(P, info.base, h) : 1;
+        if (POL == P_AR || POL == P_AELL) hL = cached && h.s != kNoHead ? proj_len<POL>(P, base, h) : 1;
     };
 
     // The conditions of all warp-uniform branches below are warp reductions: the compiler then knows
@@ -595,7 +623,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
     // (about 45, measured), and one reduction (29) decides several of them.  Single-value stores are
     // made by all lanes alike, for the same reason.
     for (;;) {
-        if (!SMEM && P.debug && attn == 0 && !state_ok<POL>(w, q, A, end, t, need, int(nextF), py, pm, pc, filled)) {
+        if (!SMEM && P.debug && attn == 0 && !state_ok<POL>(w, q, A, end, t, need, int(nextF), py, pc, qy, qc, filled)) {
             status = ST_STATE;  // a consistency check of SIM_OPT_DEBUG_CHECKS failed
             break;
         }
@@ -604,9 +632,11 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
         if (POL == P_AMIN && need > M) fl |= 2u;
         if (t >= fit_lb && need + h.s < M) fl |= 4u;
         if (unsigned(t) == nextF) fl |= 8u;
+        if (end <= kHalf) fl |= 16u;
         fl = __reduce_or_sync(FULL, fl);
+        const bool half = (fl & 16u) != 0;
         if (fl & 1u) {
-            if (end >= min(filled, w.ca) || (attn & SLOTS)) {  // reclaim free slots, or take a new page
+            if (attn & SLOTS) {  // reclaim free slots, or take a new page
                 if (end - A >= max(16, A >> 3) || (end >= w.ca && A < end)) {
                     compact<POL>(w, end);
                 } else if (end >= w.ca) {
@@ -628,12 +658,13 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 for (int i = lane; i < end; i += 32) f = min(f, unsigned(w.H[i].w));
                 nextF = __reduce_min_sync(FULL, f);
             }
-            bool dirty = (attn & HEAD) != 0;
+            bool dirty = (attn & (HEAD | MERGE)) != 0;
+            if (POL == P_AMIN && (attn & MERGE)) merge_delta(P, w, q, gbp);
             attn = 0;
             // ---- S1: arrivals with a <= t join R_t (a sorted run of the staged records)
             if (next_a <= t) {
                 int ae;
-                if (__ldg(ra + n - 1) <= t) {
+                if (ap == 0 && P.rec_a[base + n - 1] <= t) {  // all at once
                     ae = n;
                     next_a = INT_MAX;
                 } else {
@@ -648,10 +679,10 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                         }
                         apb += 32;
                         ae = apb;
-                        pa = apb + lane < n ? ra[apb + lane] : INT_MAX;
+                        pa = apb + lane < n ? P.rec_a[base + apb + lane] : INT_MAX;
                     }
                 }
-                insert_run<POL>(w, q, rec, n, ap, ae, gbq, gbp);
+                insert_run<POL>(P, w, q, P.rec + base, n, ap, ae, gbq, gbp);
                 if (INS) gbq += int64_t(ae - ap) * 4;  // their arrival steps
                 if (bt) {
                     const int64_t m = ae - ap;
@@ -663,6 +694,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 ap = ae;
                 trare = min(tstop, next_a);
                 dirty = true;
+                if (ap < n) prefetch_l1(P.rec + base + min(ap + 8, n - 1));  // a line ahead of the next arrivals
             }
             // ---- A_ell: jobs that used up their estimate unfinished (E < t) leave the batch and
             // re-enter the queue at its end with the estimate u (the delta orders their equal keys by
@@ -700,7 +732,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                         --A;
                         ++nev;
                         if (INS) ++ev_step;
-                        delta_insert(w, q, e, gbp);
+                        delta_insert(P, w, q, e, gbp);
                     }
                 }
                 nextF = __reduce_min_sync(FULL, f);
@@ -728,9 +760,10 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
         }
         // ---- S2/S3: A_min overflow of the next step -> cancel in ascending (estimate, tie key, index)
         if (POL == P_AMIN && (fl & 2u)) {
-            if (INS) {
+            if (INS && t != ovf_t) {  // (a full delta may interrupt the step's cancellations)
                 const int lg = A > 1 ? 32 - __clz(A - 1) : 0;
                 cS3 += int64_t(A) * lg * lg;
+                ovf_t = t;
             }
             // Cancellation order (estimate, r, index), r the step's tie key (SplitMix64 of the seed
             // and t * 2^32 + index; under the index rule r = index, the same order).  A round
@@ -738,20 +771,26 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             // differ does tie_position draw and compare the tied jobs' keys.  (On the 40960 x 2000
             // workload 1.3 % of the overflow steps have a tie at the smallest estimate.)
             #pragma unroll 1
-            while (need > M) {
+            while (need > M && q.dn < w.dcap) {
                 unsigned bk = UINT_MAX;
                 int lo = 0, hi = 0;
-                #pragma unroll 1
-                for (int p = 0; p < end; p += kPage) {
-                    const int i = p + 4 * lane;
-                    const uint4 k = *reinterpret_cast<const uint4 *>(w.K + i);
-                    const unsigned m = min(min(k.x, k.y), min(k.z, k.w));
-                    const int first = i + (k.x == m ? 0 : (k.y == m ? 1 : (k.z == m ? 2 : 3)));
-                    const int last = i + (k.w == m ? 3 : (k.z == m ? 2 : (k.y == m ? 1 : 0)));
-                    if (m < bk) lo = first;
-                    if (m <= bk) hi = last;
+                over_slots(half, end, [&](auto slots, int p) {
+                    constexpr int N = decltype(slots)::value;
+                    unsigned k[N], m = UINT_MAX;
+#pragma unroll
+                    for (int j = 0; j < N; ++j) {
+                        k[j] = w.K[p + 32 * j + lane];
+                        m = min(m, k[j]);
+                    }
+                    int first = 0, last = 0;
+#pragma unroll
+                    for (int j = 1; j < N; ++j) last = k[j] == m ? j : last;
+#pragma unroll
+                    for (int j = N - 1; j > 0; --j) first = k[j - 1] == m ? j - 1 : (j == N - 1 ? j : first);
+                    if (m < bk) lo = p + 32 * first + lane;
+                    if (m <= bk) hi = p + 32 * last + lane;
                     bk = min(bk, m);
-                }
+                });
                 const unsigned mk = __reduce_min_sync(FULL, bk);
                 int pos = int(__reduce_min_sync(FULL, bk == mk ? unsigned(lo) : UINT_MAX));
                 const int pos2 = int(__reduce_max_sync(FULL, bk == mk ? unsigned(hi) : 0u));
@@ -759,7 +798,8 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                     status = ST_STATE;
                     break;
                 }
-                if (pos != pos2) pos = tie_position(w.K, w.C, end, mk, tie_base(tie_seed, t), P.evict_index == 0);
+                if (pos != pos2)
+                    pos = tie_position(w.K, w.C, pos, pos2, mk, tie_base(tie_seed, t), P.evict_index == 0);
                 const int4 j = w.H[pos];
                 const int2 pi = w.C[pos];
                 __syncwarp();
@@ -777,15 +817,14 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 if (INS) ++ev_step;
                 if (unsigned(j.w) == nextF) attn |= NEXTF;
                 // endpoints before t need no update, and the update is left pending if none is
-                const int do_sub = j.x < t ? 0 : (pm == 0 ? 1 : 2);
+                const int do_sub = j.x < t ? 0 : (qy < 0 ? 1 : 2);
                 if (__reduce_max_sync(FULL, do_sub) == 2) {
                     subtract_job(w, end, j.x, j.z);
                 } else if (do_sub) {
-                    py = j.x;
-                    pm = -1;
-                    pc = -j.z;
+                    qy = j.x;
+                    qc = j.z;
                 }
-                if (delta_insert(w, q, e, gbp)) attn |= HEAD;
+                delta_put(w, q, e);
                 if (qless(e, h)) {  // the head of R_t is the smaller of the two
                     h = e;
                     hL = e.key;
@@ -795,51 +834,63 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             if (status != ST_OK) break;
             fit_lb = 0;
             if (A == 0) attn |= IDLE;
-            if (end - A >= max(16, A >> 3) && ((end - 1) ^ max(A - 1, 0)) >= kPage) attn |= SLOTS;
+            if (q.dn == w.dcap) attn |= MERGE;
+            if (end - A >= max(16, A >> 3) && slot_pages(end) > slot_pages(A)) attn |= SLOTS;
             continue;
         }
         // ---- S4/S5: admit the largest feasible prefix of R_t, one candidate at a time ((1) holds)
         if (fl & 4u) {
             const int y = t + hL - 1;
-            const int c1 = h.s + 1 - M;
-            int vy = 0, r2 = INT_MIN;
-            unsigned em = UINT_MAX;
-            #pragma unroll 1
-            for (int p = 0; p < end; p += kPage) {
-                int4 a[4];
+            const int lim = M - h.s - 1 + t;
+            int vy = 0, wm = INT_MIN;
+            const int pq = kSub ? max(py, qy) : py;
+            over_slots(half, end, [&](auto slots, int p) {
+                constexpr int N = decltype(slots)::value;
+                int4 a[N];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) a[j] = w.H[p + 32 * j + lane];
+                for (int j = 0; j < N; ++j) a[j] = w.H[p + 32 * j + lane];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (unsigned(a[j].x) <= unsigned(py)) {
-                        a[j].y += pm * a[j].x + pc;
-                        w.H[p + 32 * j + lane].y = a[j].y;
-                    }
+                for (int j = 0; j < N; ++j) {
+                    if (a[j].x <= py) a[j].y += a[j].x + pc;
+                    if (kSub && a[j].x <= qy) a[j].y -= a[j].x + qc;
+                    if (a[j].x <= pq) w.H[p + 32 * j + lane].y = a[j].y;
                     if (a[j].x >= y) vy += a[j].z + y;
-                    em = min(em, unsigned(a[j].x - y));
-                    // d = E - t: (2) asks V + d + s + 1 <= M; it holds from step t + (V + d + s + 1 - M)
-                    // on, or once the endpoint has passed (t + d + 1)
-                    const int d = a[j].x - t;
-                    if (unsigned(d) < unsigned(hL)) r2 = max(r2, min(a[j].y + d + c1, d + 1));
+                    if (unsigned(a[j].x - t) < unsigned(hL)) wm = max(wm, a[j].y);
                 }
-            }
-            pm = pc = 0;
+            });
+            py = qy = -2;
             vy = int(__reduce_add_sync(FULL, unsigned(vy)));
-            em = __reduce_min_sync(FULL, em);
-            // (3) at y; if it fails it cannot hold before y passes the next endpoint y + em
-            if (vy + h.s + hL > M) r2 = max(r2, int(em) + 1);
-            const int d = __reduce_max_sync(FULL, r2);
+            int d = max(wm, lim) - lim;      // > 0: (2) fails
+            if (vy + h.s + hL > M) d = 1;    // (3) fails
+            d = __reduce_max_sync(FULL, d);
             if (d > 0) {
-                // no fit before step t + d, and none at all if (1) fails there
-                fit_lb = int64_t(need) + int64_t(A) * d + h.s + 1 > M ? INT_MAX : t + d;
+                // A second pass finds the first later step that could fit: W_i > lim violates (2) at
+                // endpoint i until the overlap has shrunk (W_i <= lim + tau - t) or the endpoint has
+                // passed, and (3) cannot hold before y has passed the next endpoint after it.  (In the
+                // same pass as the test it cost more than it saved, also where half of the tests fail.)
+                int r2 = 1;
+                unsigned em = UINT_MAX;
+                over_slots(half, end, [&](auto slots, int p) {
+                    constexpr int N = decltype(slots)::value;
+#pragma unroll
+                    for (int j = 0; j < N; ++j) {
+                        const int2 ew = *reinterpret_cast<const int2 *>(&w.H[p + 32 * j + lane]);
+                        em = min(em, unsigned(ew.x - y));
+                        if (unsigned(ew.x - t) < unsigned(hL)) r2 = max(r2, min(max(ew.y, lim) - lim, ew.x - t + 1));
+                    }
+                });
+                em = __reduce_min_sync(FULL, em);
+                r2 = __reduce_max_sync(FULL, r2);
+                if (vy + h.s + hL > M) r2 = max(r2, int(em) + 1);
+                // no fit before step t + r2, and none at all if (1) fails there
+                fit_lb = int64_t(need) + int64_t(A) * r2 + h.s + 1 > M ? INT_MAX : t + r2;
             } else {
-                // the pending update of its own admission adds the job's memory at y to its V
+                // the pending update of its own admission adds the job's memory at y to its W
                 __syncwarp();
-                w.H[end] = make_int4(y, vy, h.s - t + 1, t + h.o - 1);
+                w.H[end] = make_int4(y, vy + y, h.s - t + 1, t + h.o - 1);
                 w.C[end] = make_int2(t, h.idx);
                 if (POL == P_AMIN) w.K[end] = unsigned(h.key);
                 py = y;
-                pm = 1;
                 pc = h.s - t + 1;
                 ++end;
                 ++A;
@@ -852,7 +903,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 q.mh += 1 - hsrc;
                 const bool miss = q.mh < q.me && unsigned(q.mh - q.mcb) >= unsigned(kMc);
                 if (miss) attn |= HEAD;
-                if (end >= min(filled, w.ca)) attn |= SLOTS;
+                if (end == kHalf || (end & (kPage - 1)) == 0) attn |= SLOTS;
                 load_head(!miss);
                 fit_lb = 0;
                 __syncwarp();
@@ -875,55 +926,62 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             if (P.completion) {
                 #pragma unroll 1
                 for (int i = lane; i < end; i += 32)
-                    if (w.H[i].w == t) P.completion[info.base + w.C[i].y] = int64_t(t) + 1;
+                    if (w.H[i].w == t) P.completion[base + w.C[i].y] = int64_t(t) + 1;
             }
-            // A job that ends before its projected last step changes V: its slot keeps E (in place of
-            // V) and B, and F = -2 - t tells it from the slots freed at other steps.
+            // A job that ends before its projected last step changes W: its slot keeps E (in place of
+            // W) and B, and F = -2 - t tells it from the slots freed at other steps.
             constexpr bool kEarly = POL == P_AMAX || POL == P_AELL;
             int c = 0, sm = 0, ne = 0, ek = -1, bk = INT_MIN;
             unsigned f = UINT_MAX, e1 = UINT_MAX;
-            #pragma unroll 1
-            for (int p = 0; p < end; p += kPage) {
-                int4 a[4];
+            over_slots(half, end, [&](auto slots, int p) {
+                constexpr int N = decltype(slots)::value;
+                int4 a[N];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) a[j] = w.H[p + 32 * j + lane];
+                for (int j = 0; j < N; ++j) a[j] = w.H[p + 32 * j + lane];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < N; ++j) {
                     const bool done = a[j].w == t, early = kEarly && done && a[j].x > t;
-                    if (done) {
-                        w.H[p + 32 * j + lane] = make_int4(-1, a[j].x, a[j].z, early ? -2 - t : -1);
-                        if (POL == P_AMIN) w.K[p + 32 * j + lane] = UINT_MAX;
-                        sm += a[j].z + t;
-                        ++c;
-                    } else {
-                        f = min(f, unsigned(a[j].w));
-                        if (POL == P_AELL) e1 = min(e1, unsigned(a[j].x));
+                    sm += done ? a[j].z + t : 0;
+                    c += done ? 1 : 0;
+                    f = min(f, done ? UINT_MAX : unsigned(a[j].w));
+                    if (POL == P_AELL) e1 = min(e1, done ? UINT_MAX : unsigned(a[j].x));
+                    if (kEarly) {
+                        ne += early ? 1 : 0;
+                        ek = early ? a[j].x : ek;
+                        bk = early ? a[j].z : bk;
                     }
-                    if (early) {
-                        ++ne;
-                        ek = a[j].x;
-                        bk = a[j].z;
-                    }
+                    a[j] = make_int4(-1, a[j].x, a[j].z, kEarly ? -2 - t : -1);
+                    if (done) w.H[p + 32 * j + lane] = a[j];  // nothing else in the branch: one predicated store
+                    if (POL == P_AMIN)
+                        if (done) w.K[p + 32 * j + lane] = UINT_MAX;
                 }
-            }
+            });
             c = int(__reduce_add_sync(FULL, unsigned(c)));
             sm = int(__reduce_add_sync(FULL, unsigned(sm)));
             nextF = __reduce_min_sync(FULL, f);
             if (POL == P_AELL) nextE = __reduce_min_sync(FULL, e1);
             if (kEarly) {
-                ne = int(__reduce_add_sync(FULL, unsigned(ne + (lane == 0 && pm != 0 ? 1 : 0))));
-                ek = __reduce_max_sync(FULL, ek);
-                bk = __reduce_max_sync(FULL, bk);
-                if (ne == 1 && ek >= 0) {  // one such job, and no update pending: leave this one pending
-                    py = ek;
-                    pm = -1;
-                    pc = -bk;
-                }
-                if (ne > 1 && ek >= 0) {
+                // the lanes that hold such a job (several on one lane: found again by their mark)
+                const int most = __reduce_max_sync(FULL, ne);
+                if (most == 1) {
+                    unsigned m = __ballot_sync(FULL, ne > 0);
+                    if (qy < 0) {
+                        const int src = __ffs(m) - 1;
+                        m &= m - 1;
+                        qy = __shfl_sync(FULL, ek, src);
+                        qc = __shfl_sync(FULL, bk, src);
+                    }
+                    #pragma unroll 1
+                    while (m) {
+                        const int src = __ffs(m) - 1;
+                        m &= m - 1;
+                        subtract_job(w, end, __shfl_sync(FULL, ek, src), __shfl_sync(FULL, bk, src));
+                    }
+                } else if (most > 1) {
                     #pragma unroll 1
                     for (int b = 0; b < end; b += 32) {
                         const int4 x = w.H[b + lane];
-                        unsigned m = __ballot_sync(FULL, x.w == -2 - t);
+                        unsigned m = __ballot_sync(FULL, x.w == -2 - t && x.y > t);
                         #pragma unroll 1
                         while (m) {
                             const int src = __ffs(m) - 1;
@@ -947,7 +1005,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             ndone += c;
             fit_lb = 0;
             if (A == 0) attn |= IDLE;
-            if (end - A >= max(16, A >> 3) && ((end - 1) ^ max(A - 1, 0)) >= kPage) attn |= SLOTS;
+            if (end - A >= max(16, A >> 3) && slot_pages(end) > slot_pages(A)) attn |= SLOTS;
             if (ndone >= n) break;
         } else {
             // steps t .. tau-1 change nothing: no completion before nextF, no arrival before
@@ -956,11 +1014,11 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             int tau = min(min(int(nextF), trare), need + h.s < M ? fit_lb : INT_MAX);
             if (POL == P_AELL) tau = min(tau, int(nextE) + 1);
             // the first step whose memory exceeds M
-            if (POL == P_AMIN) tau = min(tau, t + int(unsigned(M - need) / unsigned(max(A, 1))) + 1);
+            if (POL == P_AMIN) tau = min(tau, t + quotient_lb(M - need, max(A, 1)) + 1);
             const int c = max(tau - t, 1);
-            const int64_t mem = int64_t(need) + int64_t(A) * (c - 1);
-            if (mem > M) status = ST_STATE;  // an internal error, reported at the end
-            peak = max(peak, int(mem));
+            const int mem = need + A * (c - 1);  // of step tau - 1: feasible, so at most M
+            if (mem > M) status = ST_STATE;      // an internal error, reported at the end
+            peak = max(peak, mem);
             rsteps += int64_t(A) * c;
             if (bt)  // steps t .. t+c-1 have memory need + A (x - t)
                 bmem += c * int64_t(need) + int64_t(A) * (int64_t(c) * (c - 1) / 2);
@@ -970,13 +1028,13 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 cS5 += int64_t(A) * (32 - __clz(Qa + k_step)) + int64_t(A) * (c - 1) * (32 - __clz(Qa));
                 k_step = ev_step = 0;
             }
-            need = int(mem) + A;
+            need = mem + A;
             t += c;
         }
     }
     if (lane == 0) {
         r.status = status;
-        r.total_latency = sumC - info.sum_a;
+        r.total_latency = sumC - P.info[inst].sum_a;
         r.makespan = makespan;
         r.peak_memory = peak;
         r.evictions = nev;
@@ -1004,18 +1062,18 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
     __syncwarp();
 }
 
-template <int POL, bool SMEM, bool INS>
-__global__ void __launch_bounds__(256, 2) k_run(RunParams P) {
+// WIDE: up to 168 registers a thread (12 warps per SM), for launches whose time is one instance's serial
+// chain; otherwise 128 (16 warps per SM), for launches with more instances than that.  A_min at 128
+// registers spills 9 of them: the 256 x 10^4 online workload takes 28.5 ms against 26.9, the 40960 x 2000
+// one 111 ms at 16 warps per SM against 133 at 12.
+template <int POL, bool SMEM, bool INS, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? 128 : 256, WIDE ? 3 : 2) k_run(RunParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = lane_id();
-    const int wib = threadIdx.x >> 5;
-    const int64_t slot = int64_t(blockIdx.x) * (blockDim.x >> 5) + wib;
     unsigned char *base;
-    if (SMEM) base = smem_raw + size_t(wib) * ws_bytes(POL == P_AMIN, P.ca, P.dcap);
-    else base = P.gws + slot * P.gws_stride;
+    if (SMEM) base = smem_raw + size_t(threadIdx.x >> 5) * ws_bytes(POL == P_AMIN, P.ca, P.dcap);
+    else base = P.gws + warp_slot() * P.gws_stride;
     Ws w = carve_ws(base, P.ca, P.dcap);
-    w.mb0 = P.mainbuf + slot * 2 * P.main_cap;
-    w.mb1 = w.mb0 + P.main_cap;
     for (;;) {
         int k = 0;
         if (lane == 0) k = atomicAdd(P.counter, 1);
@@ -1029,26 +1087,28 @@ __global__ void __launch_bounds__(256, 2) k_run(RunParams P) {
 using KernelFn = void (*)(RunParams);
 
 template <int POL>
-KernelFn pick(bool smem, bool ins) {
-    if (smem) return ins ? k_run<POL, true, true> : k_run<POL, true, false>;
-    return ins ? k_run<POL, false, true> : k_run<POL, false, false>;
+KernelFn pick(bool smem, bool ins, bool wide) {
+    if (smem && ins) return wide ? k_run<POL, true, true, true> : k_run<POL, true, true, false>;
+    if (smem) return wide ? k_run<POL, true, false, true> : k_run<POL, true, false, false>;
+    return ins ? k_run<POL, false, true, false> : k_run<POL, false, false, false>;
 }
 
-KernelFn run_fn(int policy, const RunParams &p) {
+KernelFn run_fn(int policy, const RunParams &p, int warps_per_block) {
     const bool smem = p.use_smem != 0, ins = p.work_count != nullptr || p.batch_time != nullptr;
+    const bool wide = p.wide != 0 && warps_per_block <= 4;
     switch (policy) {
-        case P_AMAX: return pick<P_AMAX>(smem, ins);
-        case P_AMIN: return pick<P_AMIN>(smem, ins);
-        case P_HSF: return pick<P_HSF>(smem, ins);
-        case P_AR: return pick<P_AR>(smem, ins);
-        default: return pick<P_AELL>(smem, ins);
+        case P_AMAX: return pick<P_AMAX>(smem, ins, wide);
+        case P_AMIN: return pick<P_AMIN>(smem, ins, wide);
+        case P_HSF: return pick<P_HSF>(smem, ins, wide);
+        case P_AR: return pick<P_AR>(smem, ins, wide);
+        default: return pick<P_AELL>(smem, ins, wide);
     }
 }
 
 }  // namespace
 
 cudaError_t run_blocks_per_sm(int policy, const RunParams &p, int warps_per_block, size_t smem_bytes, int *blocks) {
-    const KernelFn fn = run_fn(policy, p);
+    const KernelFn fn = run_fn(policy, p, warps_per_block);
     if (smem_bytes > 48 * 1024) {
         const cudaError_t e =
             cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem_bytes));
@@ -1059,7 +1119,7 @@ cudaError_t run_blocks_per_sm(int policy, const RunParams &p, int warps_per_bloc
 
 cudaError_t launch_run(int policy, const RunParams &p, int blocks, int warps_per_block, size_t smem_bytes,
                        cudaStream_t st) {
-    run_fn(policy, p)<<<dim3(blocks), dim3(32 * warps_per_block), smem_bytes, st>>>(p);
+    run_fn(policy, p, warps_per_block)<<<dim3(blocks), dim3(32 * warps_per_block), smem_bytes, st>>>(p);
     return cudaGetLastError();
 }
 

@@ -154,6 +154,7 @@ extern "C" int sim_run_noalloc(int policy, int64_t M, int32_t n_instances, const
     p.ca = int32_t(((std::max<int64_t>(n_max, 128) + 127) / 128) * 128);  // >= any active set: no fallback
     p.dcap = simgb::kDcap;
     p.use_smem = 0;
+    p.wide = 0;
     p.debug = 0;
     p.evict_index = 0;
     p.gws = base + kOffWs;
