@@ -1,16 +1,40 @@
 // Analytic competitive-ratio evaluators of A_min (double precision, sm_103a).
 //
-//   k_lemma   - Lemma thm:Amin for a batch of length histograms: one thread per histogram walks it
-//               from the longest length down with the four running sums the lemma needs
-//               (sum i x_i, sum x_i/(s+i), sum i x_i/(s+i), sum x_i over i >= k), about ten FP64
-//               operations per length, with 1/(s+k) and k(s+k) from a shared-memory table.  The
-//               histogram is read once; GB300's FP64 rate, not HBM, bounds the kernel.
+//   k_lemma   - Lemma thm:Amin for a batch of length histograms, walked from the longest length down.
+//               With X_k, S1_k, S2_k the sums over i >= k of x_i, i x_i, x_i / (s + i) and
+//               G_k = sum over i > k of (i - k) x_i / (s + i) = G_{k+1} + S2_{k+1},
+//                 numerator   = sum_k d_k S1_k (2 G_k + d_k S2_k)   (d_k = 1, and s + l at k = l),
+//                 denominator = sum_k k (s + k) x_k (x_k + 2 X_{k+1}) = sum_k D_k X_k^2,
+//               D_k = k (s + k) - (k - 1)(s + k - 1) = s + 2 k - 1 above l and l (s + l) at l
+//               (x_k (x_k + 2 X_{k+1}) = X_k^2 - X_{k+1}^2, summed by parts): eight FP64 operations
+//               per length and, for a histogram of counts, sums of positive terms only.
+//               GB300's FP64 rate (two lanes per SM and cycle) bounds it, not HBM.  A group of T
+//               lanes shares a histogram: T = 1 when there are enough histograms to fill the FP64
+//               pipes; otherwise each lane first sums its segment of lengths (four operations per
+//               length), the lanes' sums are scanned and each lane walks its segment with the sums of
+//               the segments above it.  2^20 histograms of 64 lengths take 0.97 ms (14 operations per
+//               length and a cancelling T - k S2 in place of G: 1.72 ms); 333 of 1999 lengths 0.05 ms
+//               (one lane each: 1.96 ms).  RMS error against 128-bit sums 1.0e-16 and 1.4e-16 (before:
+//               1.3e-16 and 1.1e-15).
 //   k_rho     - spectral radius of B_u^{-1} A_u (Corollary A/B; s = 0, l = 1), the bound on the
-//               Rayleigh quotient of Section 4.1, by power iteration.  A_u v is O(u) from prefix
-//               and suffix sums (for j <= i, a_ij = ij/2 + j^2 - j^3/(2i); symmetric), B_u^{-1} is
-//               the tridiagonal matrix printed in Section 4.1, and the estimate is the Rayleigh
-//               quotient v'Av / v'Bv with (Bv)_i = sum_{j<=i} j^2 v_j + i^2 sum_{j>i} v_j.  One
-//               warp per u; the vectors live in a global scratch of 3 u doubles per warp.
+//               Rayleigh quotient of Section 4.1, by power iteration from v = (1, .., 1).
+//               b_ij = min(i, j)^2, so with the suffix sums S_i = sum_{j >= i} v_j,
+//                 v' B v = sum_i (2 i - 1) S_i^2,
+//               and one step v <- B^{-1} A v reads, in the suffix sums (w_i = 3 i^2 - 3 i + 1),
+//                 S_i <- [ (3 - 2 / i) S_i + sum_k S_k + (sum_{k < i} w_k S_k) / (i (i - 1))
+//                          + w_i sum_{k > i} S_k / (k (k - 1)) ] / (2 (2 i - 1))
+//               (a_ij = i j / 2 + j^2 - j^3 / (2 i) for j <= i; differences of A v in i, summed by
+//               parts).  Every term is positive, so nothing cancels, and v' A v = sum_i (2 i - 1) S_i S'_i.
+//               A thread-block cluster works on one u, each thread on a run of consecutive i: sums of
+//               its run, a scan over the block and the cluster (one cluster barrier per step), then its
+//               run again.  The arrays stay in shared memory when they fit.  About 18 FP64 operations
+//               per index and step; FP64 rate and the serial steps (about 15) bound it.  u = 20,000:
+//               0.47 ms, 10^5: 1.4 ms, 2^20: 11.5 ms; 25 values up to 20,000: 0.56 ms.  (One warp per u,
+//               with four scans of totals minus prefixes, seven divisions per index and the tridiagonal
+//               B^{-1} applied to A v: 573 ms for the 25 values, relative error 2e-9 at u = 20,000 against
+//               4e-16 now.)
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -29,145 +53,222 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Inclusive prefix sum over lanes.
-__device__ __forceinline__ double prefix_incl(double v) {
+// Sum over the lanes below this one (up) or above it (down).
+__device__ __forceinline__ double excl_up(double v, double &total) {
     const int lane = threadIdx.x & 31;
+    double x = v;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const double y = __shfl_up_sync(FULL, v, d);
-        if (lane >= d) v += y;
+        const double y = __shfl_up_sync(FULL, x, d);
+        if (lane >= d) x += y;
     }
-    return v;
+    total = __shfl_sync(FULL, x, 31);
+    const double e = __shfl_up_sync(FULL, x, 1);
+    return lane == 0 ? 0.0 : e;
 }
 
+__device__ __forceinline__ double excl_down(double v, double &total) {
+    const int lane = threadIdx.x & 31;
+    double x = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const double y = __shfl_down_sync(FULL, x, d);
+        if (lane + d < 32) x += y;
+    }
+    total = __shfl_sync(FULL, x, 0);
+    const double e = __shfl_down_sync(FULL, x, 1);
+    return lane == 31 ? 0.0 : e;
+}
+
+// The running sums of a walk that has passed n lengths.
+struct LemmaSums {
+    double X, S1, S2, G;
+    int n;
+};
+
+// The sums after the segment b follows the lengths summed in a.
+__device__ __forceinline__ LemmaSums then(const LemmaSums &a, const LemmaSums &b) {
+    return {a.X + b.X, a.S1 + b.S1, a.S2 + b.S2, fma(double(b.n), a.S2, a.G) + b.G, a.n + b.n};
+}
+
+template <int T>
 __global__ void __launch_bounds__(256) k_lemma(int32_t n_hist, int32_t len, int32_t l, double s,
                                                 const double *__restrict__ x, double *__restrict__ out) {
-    // per-length constants shared by every histogram: 1/(s+k) and k(s+k)
+    // per-length constants shared by every histogram: 1/(s+k), k, D_k
     extern __shared__ double tab[];
-    double *rinv = tab, *ck = tab + len;
+    double *rinv = tab, *kk = tab + len, *dk = tab + 2 * len;
     for (int j = threadIdx.x; j < len; j += blockDim.x) {
         const double k = double(l + j);
         rinv[j] = 1.0 / (s + k);
-        ck[j] = k * (s + k);
+        kk[j] = k;
+        dk[j] = j == 0 ? k * (s + k) : s + 2.0 * k - 1.0;
     }
     __syncthreads();
-    const int64_t h = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (h >= n_hist) return;
-    const double *xh = x + h * int64_t(len);
-    // running sums over lengths > k (before the update) and >= k (after it)
-    double S1 = 0.0, S2 = 0.0, T = 0.0, X = 0.0;
-    double num = 0.0, den = 0.0;
-    for (int j = len - 1; j >= 0; --j) {
-        const double k = double(l + j);
-        const double xk = __ldg(xh + j);
-        // values over i > k
-        const double gap = fma(-k, S2, T);      // sum_{i>k} (i-k) x_i/(s+i)
-        const double twoXn = 2.0 * X;           // 2 sum_{i>k} x_i
-        const double fr = xk * rinv[j];
-        S1 = fma(k, xk, S1);                    // sum_{i>=k} i x_i
-        S2 += fr;                               // sum_{i>=k} x_i/(s+i)
-        T = fma(k, fr, T);                      // sum_{i>=k} i x_i/(s+i)
-        X += xk;
-        const double delta = (j == 0) ? (s + double(l)) : 1.0;
-        num = fma(delta * S1, fma(2.0, gap, delta * S2), num);
-        den = fma(ck[j] * xk, xk + twoXn, den);
-    }
-    out[h] = num / den;
-}
-
-// (A v)_i and (B v)_i for i = 1..u from prefix/suffix sums; v, av, bv in global scratch.
-__device__ void rho_products(int u, const double *v, double *av, double *bv, double &vav, double &vbv) {
-    const int lane = threadIdx.x & 31;
-    // totals first: P1 = sum j v_j
-    double p1 = 0.0;
-    for (int b = 0; b < u; b += 32) {
-        const int j = b + lane + 1;
-        if (j <= u) p1 += double(j) * v[j - 1];
-    }
-    p1 = warp_sum(p1);
-    // prefix sums Q2 = sum_{j<=i} j^2 v_j, Q3 = sum_{j<=i} j^3 v_j; suffix sums R0 = sum_{j>i} v_j,
-    // R1 = sum_{j>i} v_j / j, obtained as totals minus prefixes
-    double t0 = 0.0, t1 = 0.0;
-    for (int b = 0; b < u; b += 32) {
-        const int j = b + lane + 1;
-        if (j <= u) {
-            t0 += v[j - 1];
-            t1 += v[j - 1] / double(j);
+    const int64_t h = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / T;
+    if (T == 1 && h >= n_hist) return;
+    const int g = threadIdx.x % T;
+    const double *xh = x + min(h, int64_t(n_hist) - 1) * int64_t(len);
+    // lane g of the group takes the lengths [lo, hi), lane 0 the longest ones; an odd number per
+    // lane keeps the lanes' table reads on different banks
+    const int m = T == 1 ? len : ((len + T - 1) / T) | 1;
+    const int hi = max(len - g * m, 0), lo = T == 1 ? 0 : max(hi - m, 0);
+    LemmaSums p = {0.0, 0.0, 0.0, 0.0, 0};
+    if (T > 1) {
+        for (int j = hi - 1; j >= lo; --j) {
+            const double xk = __ldg(xh + j);
+            p.X += xk;
+            p.S1 = fma(kk[j], xk, p.S1);
+            p.S2 = fma(rinv[j], xk, p.S2);
+            p.G += p.S2;
         }
-    }
-    t0 = warp_sum(t0);
-    t1 = warp_sum(t1);
-    double q2c = 0.0, q3c = 0.0, r0c = 0.0, r1c = 0.0;  // running prefixes of the four sums
-    double sa = 0.0, sb = 0.0;
-    for (int b = 0; b < u; b += 32) {
-        const int i = b + lane + 1;
-        const double di = double(i);
-        const double vi = (i <= u) ? v[i - 1] : 0.0;
-        const double q2 = prefix_incl(di * di * vi) + q2c;
-        const double q3 = prefix_incl(di * di * di * vi) + q3c;
-        const double p0 = prefix_incl(vi) + r0c;         // sum_{j<=i} v_j
-        const double p1i = prefix_incl(vi / di) + r1c;   // sum_{j<=i} v_j / j
-        if (i <= u) {
-            const double R0 = t0 - p0, R1 = t1 - p1i;
-            const double a = 0.5 * di * p1 + q2 - q3 / (2.0 * di) + di * di * R0 - 0.5 * di * di * di * R1;
-            const double bb = q2 + di * di * R0;
-            av[i - 1] = a;
-            bv[i - 1] = bb;
-            sa += vi * a;
-            sb += vi * bb;
-        }
-        q2c = __shfl_sync(FULL, q2, 31);
-        q3c = __shfl_sync(FULL, q3, 31);
-        r0c = __shfl_sync(FULL, p0, 31);
-        r1c = __shfl_sync(FULL, p1i, 31);
-    }
-    vav = warp_sum(sa);
-    vbv = warp_sum(sb);
-    __syncwarp();
-}
-
-__global__ void k_rho(int32_t n_u, const int32_t *__restrict__ us, double *__restrict__ out, double *scratch,
-                      int64_t stride, int32_t max_iter) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    if (warp >= n_u) return;
-    const int u = us[warp];
-    double *v = scratch + warp * stride;
-    double *av = v + u;
-    double *bv = av + u;
-    for (int i = lane; i < u; i += 32) v[i] = 1.0;
-    __syncwarp();
-    double lam = 0.0;
-    for (int it = 0; it < max_iter; ++it) {
-        double vav, vbv;
-        rho_products(u, v, av, bv, vav, vbv);
-        const double nl = vav / vbv;  // generalized Rayleigh quotient of the current vector
-        // next vector: B^{-1} (A v), tridiagonal, then scale by its largest entry
-        double mx = 0.0;
-        for (int b = 0; b < u; b += 32) {
-            const int i = b + lane + 1;
-            double z = 0.0;
-            if (i <= u) {
-                const double di = double(i);
-                const double d = (i < u) ? 4.0 * di / (4.0 * di * di - 1.0) : 1.0 / (2.0 * di - 1.0);
-                z = d * av[i - 1];
-                if (i > 1) z -= av[i - 2] / (2.0 * (di - 1.0) + 1.0);
-                if (i < u) z -= av[i] / (2.0 * di + 1.0);
-            }
-            __syncwarp();
-            if (i <= u) bv[i - 1] = z;  // bv is free until the next products
-            mx = fmax(mx, fabs(z));
-        }
+        p.n = hi - lo;
+        // inclusive scan over the group, then shift by one lane
 #pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) mx = fmax(mx, __shfl_xor_sync(FULL, mx, d));
-        __syncwarp();
-        for (int i = lane; i < u; i += 32) v[i] = bv[i] / mx;
-        __syncwarp();
-        const bool done = it > 0 && fabs(nl - lam) <= 1e-15 * nl;
-        lam = nl;
-        if (done) break;
+        for (int d = 1; d < T; d <<= 1) {
+            const LemmaSums q = {__shfl_up_sync(FULL, p.X, d, T), __shfl_up_sync(FULL, p.S1, d, T),
+                                 __shfl_up_sync(FULL, p.S2, d, T), __shfl_up_sync(FULL, p.G, d, T),
+                                 __shfl_up_sync(FULL, p.n, d, T)};
+            if (g >= d) p = then(q, p);
+        }
+        p = {__shfl_up_sync(FULL, p.X, 1, T), __shfl_up_sync(FULL, p.S1, 1, T), __shfl_up_sync(FULL, p.S2, 1, T),
+             __shfl_up_sync(FULL, p.G, 1, T), 0};
+        if (g == 0) p = {0.0, 0.0, 0.0, 0.0, 0};
     }
-    if (lane == 0) out[warp] = lam;
+    double num = 0.0, den = 0.0;
+#pragma unroll 4
+    for (int j = hi - 1; j >= max(lo, 1); --j) {
+        const double xk = __ldg(xh + j);
+        p.X += xk;                                      // sum_{i>=k} x_i
+        p.S1 = fma(kk[j], xk, p.S1);                    // sum_{i>=k} i x_i
+        p.S2 = fma(rinv[j], xk, p.S2);                  // sum_{i>=k} x_i/(s+i)
+        num = fma(p.S1, fma(2.0, p.G, p.S2), num);      // G: sum_{i>k} (i-k) x_i/(s+i)
+        den = fma(dk[j], p.X * p.X, den);
+        p.G += p.S2;
+    }
+    if (lo == 0 && hi > 0) {  // k = l
+        const double xk = __ldg(xh);
+        const double delta = s + double(l);
+        p.X += xk;
+        p.S1 = fma(kk[0], xk, p.S1);
+        p.S2 = fma(rinv[0], xk, p.S2);
+        num = fma(delta * p.S1, fma(2.0, p.G, delta * p.S2), num);
+        den = fma(dk[0], p.X * p.X, den);
+    }
+    if (T > 1) {
+#pragma unroll
+        for (int d = T / 2; d >= 1; d >>= 1) {
+            num += __shfl_xor_sync(FULL, num, d, T);
+            den += __shfl_xor_sync(FULL, den, d, T);
+        }
+    }
+    if (g == 0 && h < n_hist) out[h] = num / den;
+}
+
+constexpr int kRhoThreads = 256;
+constexpr int kRhoArrays = 4;  // S, T, 1/(i(i-1)), 1/(8(2i-1)) per i
+
+__global__ void __launch_bounds__(kRhoThreads) k_rho(const int32_t *__restrict__ us, double *__restrict__ out,
+                                                      double *scratch, int64_t stride, int32_t max_iter) {
+    namespace cg = cooperative_groups;
+    constexpr int kW = kRhoThreads / 32;
+    extern __shared__ double rho_smem[];
+    __shared__ double wsum[5][kW];  // per warp: p1, Q, T, numerator, denominator
+    __shared__ double part[2][5];   // per block, double-buffered over steps, read by the cluster
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = int(cl.num_blocks()), rank = int(cl.block_rank());
+    const int64_t id = blockIdx.x / C;
+    const int u = us[id];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    // this block's indices [lo, hi) (0-based: entry e is i = e + 1), this thread's [a, b)
+    const int R = (u + C - 1) / C;
+    const int lo = min(rank * R, u), hi = min(lo + R, u);
+    const int m = ((hi - lo + kRhoThreads - 1) / kRhoThreads) | 1;  // odd: the runs start on different banks
+    const int a = min(lo + tid * m, hi), b = min(a + m, hi);
+    // arrays over the block's indices, in shared memory or in the scratch of this u
+    double *S = scratch ? scratch + id * stride + int64_t(kRhoArrays) * lo : rho_smem;
+    double *tv = S + (hi - lo), *rk = tv + (hi - lo), *bb = rk + (hi - lo);
+    S -= lo;
+    tv -= lo;
+    rk -= lo;
+    bb -= lo;
+    for (int e = a; e < b; ++e) {
+        const double i = double(e + 1);
+        S[e] = double(u - e);
+        rk[e] = e == 0 ? 0.0 : 1.0 / (i * (i - 1.0));
+        bb[e] = 0.125 / (2.0 * i - 1.0);  // a quarter of 1 / (2 (2 i - 1)): S neither grows nor vanishes
+    }
+    double lam = 0.0, num = 0.0, den = 0.0;
+    for (int it = 0; it <= max_iter; ++it) {
+        // sums over this thread's run
+        double p1 = 0.0, Q = 0.0, T = 0.0;
+        double im = double(a);  // i - 1
+        for (int e = a; e < b; ++e) {
+            const double v = S[e];
+            p1 += v;
+            Q = fma(fma(3.0 * im, im + 1.0, 1.0), v, Q);
+            T = fma(rk[e], v, T);
+            im += 1.0;
+        }
+        // exclusive prefix of Q, suffix of T, and totals, over the warp, the block and the cluster
+        double tq, tt;
+        double q = excl_up(Q, tq), tl = excl_down(T, tt);
+        p1 = warp_sum(p1);
+        num = warp_sum(num);
+        den = warp_sum(den);
+        if (lane == 0) {
+            wsum[0][wid] = p1;
+            wsum[1][wid] = tq;
+            wsum[2][wid] = tt;
+            wsum[3][wid] = num;
+            wsum[4][wid] = den;
+        }
+        __syncthreads();
+        double *mine = part[it & 1];
+        if (tid < 5) {
+            double acc = 0.0;
+            for (int k = 0; k < kW; ++k) acc += wsum[tid][k];
+            mine[tid] = acc;
+        }
+        for (int k = 0; k < wid; ++k) q += wsum[1][k];
+        for (int k = kW - 1; k > wid; --k) tl += wsum[2][k];
+        cl.sync();
+        double tot[3] = {0.0, 0.0, 0.0};  // p1, numerator, denominator over the cluster
+        for (int k = 0; k < C; ++k) {
+            const double *pk = cl.map_shared_rank(mine, k);
+            tot[0] += pk[0];
+            if (k < rank) q += pk[1];
+            if (k > rank) tl += pk[2];
+            tot[1] += pk[3];
+            tot[2] += pk[4];
+        }
+        if (it > 0) {  // the Rayleigh quotient of the vector of step it - 1
+            const double nl = 0.5 * tot[1] / tot[2];
+            const bool done = it > 1 && fabs(nl - lam) <= 1e-15 * nl;
+            lam = nl;
+            if (done) break;
+        }
+        // T_i = sum over k > i, from the end of the run
+        for (int e = b - 1; e >= a; --e) {
+            tv[e] = tl;
+            tl = fma(rk[e], S[e], tl);
+        }
+        // the step, from its start
+        num = den = 0.0;
+        im = double(a);
+        for (int e = a; e < b; ++e) {
+            const double v = S[e], r = rk[e];
+            const double w = fma(3.0 * im, im + 1.0, 1.0);
+            const double c = e == 0 ? 1.0 : fma(-2.0 * im, r, 3.0);  // 3 - 2 / i
+            const double br = fma(w, tv[e], fma(r, q, fma(c, v, tot[0])));
+            num = fma(v, br, num);
+            den = fma(fma(2.0, im, 1.0) * v, v, den);
+            q = fma(w, v, q);
+            S[e] = bb[e] * br;
+            im += 1.0;
+        }
+    }
+    if (rank == 0 && tid == 0) out[id] = lam;
+    cl.sync();  // no block leaves while another may still read its sums
 }
 
 }  // namespace
@@ -175,20 +276,73 @@ __global__ void k_rho(int32_t n_u, const int32_t *__restrict__ us, double *__res
 cudaError_t launch_lemma(int32_t n_hist, int32_t len, int32_t l, double s, const double *x, double *out,
                          cudaStream_t st) {
     if (n_hist <= 0) return cudaSuccess;
-    const size_t smem = size_t(2) * len * sizeof(double);
+    int dev = 0, n_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    // Lanes per histogram: the least (rounds of one warp per scheduler) x (operations of a lane's
+    // walk, 8 per length alone and 12 shared); a scheduler's FP64 pipe is busy with one warp.
+    const auto cost = [&](int T) {
+        const int64_t warps = (int64_t(n_hist) * T + 31) / 32, rounds = (warps + 4 * n_sm - 1) / (4 * n_sm);
+        return rounds * ((len + T - 1) / T) * (T == 1 ? 8 : 12);
+    };
+    int T = 1;
+    for (int c = 2; c <= 32 && c <= len; c <<= 1)
+        if (cost(c) < cost(T)) T = c;
+    // blocks small enough that every SM gets one
+    const int64_t lanes = int64_t(n_hist) * T;
+    int threads = 256;
+    while (threads > 64 && (lanes + threads - 1) / threads < n_sm) threads >>= 1;
+    const unsigned blocks = unsigned((lanes + threads - 1) / threads);
+    const size_t smem = size_t(3) * len * sizeof(double);
+    using Fn = void (*)(int32_t, int32_t, int32_t, double, const double *, double *);
+    const Fn fn = T == 1 ? k_lemma<1> : T == 2 ? k_lemma<2> : T == 4 ? k_lemma<4> : T == 8 ? k_lemma<8>
+                  : T == 16 ? k_lemma<16> : k_lemma<32>;
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_lemma, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
     }
-    k_lemma<<<(n_hist + 255) / 256, 256, smem, st>>>(n_hist, len, l, s, x, out);
+    fn<<<blocks, threads, smem, st>>>(n_hist, len, l, s, x, out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_rho(int32_t n_u, const int32_t *us, double *out, double *scratch, int64_t stride,
-                       int32_t max_iter, cudaStream_t st) {
+// Blocks per cluster: about 512 indices of the largest u each, at most 8 blocks.
+static int rho_cluster(int32_t u_max) {
+    int c = 1;
+    while (c < 8 && 512 * c < u_max) c <<= 1;
+    return c;
+}
+
+static size_t rho_smem_bytes(int32_t u_max) {
+    const int c = rho_cluster(u_max);
+    return size_t((u_max + c - 1) / c) * kRhoArrays * sizeof(double);
+}
+
+int64_t rho_scratch_doubles(int32_t u_max) {
+    return rho_smem_bytes(u_max) <= size_t(200) * 1024 ? 0 : int64_t(kRhoArrays) * u_max;
+}
+
+cudaError_t launch_rho(int32_t n_u, int32_t u_max, const int32_t *us, double *out, double *scratch, int32_t max_iter,
+                       cudaStream_t st) {
     if (n_u <= 0) return cudaSuccess;
-    k_rho<<<(n_u + 3) / 4, 128, 0, st>>>(n_u, us, out, scratch, stride, max_iter);
-    return cudaGetLastError();
+    const int64_t stride = rho_scratch_doubles(u_max);
+    const size_t smem = stride ? 0 : rho_smem_bytes(u_max);
+    cudaError_t e =
+        cudaFuncSetAttribute((const void *)k_rho, cudaFuncAttributeMaxDynamicSharedMemorySize, int(size_t(200) * 1024));
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    const int c = rho_cluster(u_max);
+    cfg.gridDim = dim3(unsigned(n_u) * unsigned(c));
+    cfg.blockDim = dim3(kRhoThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = unsigned(c);
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_rho, us, out, stride ? scratch : static_cast<double *>(nullptr), stride, max_iter);
 }
 
 }  // namespace simgb

@@ -716,32 +716,27 @@ int sim_cr_amin_rho(int32_t n_u, const int32_t *u_values, double *rho_out) {
             return fail(nullptr, SIM_E_INVAL, "sim_cr_amin_rho: u_values[%d]=%d outside [1, 2^20]", k, u_values[k]);
         umax = std::max(umax, u_values[k]);
     }
-    // batches of at most 256 MB of vectors (3 u doubles per value)
-    const int64_t stride = 3 * int64_t(umax);
-    const int64_t per_batch = std::max<int64_t>(1, (int64_t(256) << 20) / (stride * int64_t(sizeof(double))));
+    // batches of at most 1 GB of scratch, 2^20 values; one allocation: scratch, results, values
+    const int64_t stride = simgb::rho_scratch_doubles(umax);
+    const int64_t per_batch = stride ? std::max<int64_t>(1, (int64_t(1) << 30) / (stride * int64_t(sizeof(double)))) : 1 << 20;
     const int32_t nb = int32_t(std::min<int64_t>(per_batch, n_u));
-    double *scratch = nullptr, *dout = nullptr;
-    int32_t *dus = nullptr;
+    double *scratch = nullptr;
     cudaError_t e;
-    if ((e = cudaMalloc(&scratch, size_t(nb) * size_t(stride) * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&dout, size_t(nb) * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&dus, size_t(nb) * sizeof(int32_t))) != cudaSuccess) {
-        cudaFree(scratch);
-        cudaFree(dout);
+    const size_t bytes = size_t(nb) * (size_t(stride + 1) * sizeof(double) + sizeof(int32_t));
+    if ((e = cudaMalloc(&scratch, bytes)) != cudaSuccess)
         return e == cudaErrorMemoryAllocation ? fail(nullptr, SIM_E_NOMEM, "sim_cr_amin_rho: device allocation")
                                               : cuda_fail(nullptr, e, "sim_cr_amin_rho: cudaMalloc");
-    }
+    double *dout = scratch + size_t(nb) * size_t(stride);
+    int32_t *dus = reinterpret_cast<int32_t *>(dout + nb);
     int rc = SIM_OK;
     for (int32_t b = 0; b < n_u && rc == SIM_OK; b += nb) {
         const int32_t m = std::min(nb, n_u - b);
         if ((e = cudaMemcpy(dus, u_values + b, size_t(m) * sizeof(int32_t), cudaMemcpyHostToDevice)) != cudaSuccess ||
-            (e = simgb::launch_rho(m, dus, dout, scratch, stride, 200, nullptr)) != cudaSuccess ||
+            (e = simgb::launch_rho(m, umax, dus, dout, scratch, 200, nullptr)) != cudaSuccess ||
             (e = cudaMemcpy(rho_out + b, dout, size_t(m) * sizeof(double), cudaMemcpyDeviceToHost)) != cudaSuccess)
             rc = cuda_fail(nullptr, e, "sim_cr_amin_rho");
     }
     cudaFree(scratch);
-    cudaFree(dout);
-    cudaFree(dus);
     return rc;
 }
 

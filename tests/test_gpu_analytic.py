@@ -97,3 +97,35 @@ def test_invalid_arguments():
         cr_amin_lemma(np.ones((2, 3)), 0, 0.0)
     with pytest.raises(SimError):
         cr_amin_lemma(np.ones((2, 3)), 1, -1.0)
+
+
+@pytest.mark.parametrize("n,length", [(1, 1), (1, 2), (3, 31), (333, 63), (5, 1999), (700, 257), (2500, 130), (9000, 40),
+                                      (20000, 9), (2, 8192)])
+def test_lemma_shared_histograms(n, length):
+    """From one lane per histogram to 32: lane segments that are empty, ragged or end at the first
+    length.  Sums of up to 8192 positive terms: 1e-13 relative (about 1e-16 per operation)."""
+    from oracle import analytic as an
+    from paper_2508_14544_gb300 import cr_amin_lemma
+    rng = np.random.default_rng([n, length])
+    x = rng.random((n, length))
+    x[:, 1::5] = 0.0
+    got = cr_amin_lemma(x, 3, 2.5)
+    rows = np.unique(np.concatenate([np.arange(min(n, 20)), rng.integers(0, n, 20), [n - 1]]))
+    ref = np.array([an.lemma_amin_cr(x[i], 3, 2.5) for i in rows])
+    assert np.all(np.abs(got[rows] - ref) <= 1e-13 * ref)
+
+
+def test_rho_cluster_sizes_and_scratch():
+    """Values around the cluster sizes (512 indices per block), blocks without indices, and one above
+    the shared-memory limit (global scratch), alone and next to a larger one: the value does not
+    depend on the launch (sums in another order: 1e-13), and equals the dense eigensolver."""
+    from oracle import analytic as an
+    from paper_2508_14544_gb300 import cr_amin_rho
+    us = [1, 2, 5, 511, 512, 513, 1024, 1025, 2049, 4097]
+    alone = np.array([cr_amin_rho([u])[0] for u in us])
+    for big in (5000, 51200, 51300):
+        got = cr_amin_rho(us + [big])
+        assert np.all(np.abs(got[:-1] - alone) <= 1e-13 * alone)
+        assert got[-1] > got[-2]
+    for u, r in zip(us[:8], alone):
+        assert abs(r - an.rho(u)) <= 1e-10 * r, u
