@@ -298,15 +298,15 @@ int64_t sim_kernel_launches(const sim_ctx *ctx);
  *   results     DEVICE, n_instances sim_result, written by the kernels.
  *   cuda_stream a cudaStream_t or NULL.  The call only enqueues work: read `results` after
  *               synchronising the stream.  Per-instance statuses are in results[i].status.
- * Everything except the inputs and outputs lives in one fixed array of about 23 MB that every GPU
+ * Everything except the inputs and outputs lives in one fixed array of about 21 MB that every GPU
  * loading the library holds until the process exits.  Limits: at most 2048 requests per instance
  * and 262,144 requests per call; larger inputs are rejected with SIM_E_INVAL and a message in
  * sim_last_error(NULL).  The staging kernel checks the offsets it reads against the same limits
  * again: an instance that reaches past them gets status SIM_E_INVAL in its result and nothing of
- * it is staged.  The fixed array holds the workspaces of 128 simulating warps (32 blocks of 4),
- * so on a 152-SM GPU most SMs stay idle: with many instances expect several times the time of
- * sim_run, which sizes its launch to the whole GPU.  All calls share that array and it keeps the last call's contents: calls
- * that overlap on the GPU (different streams or threads) race; calls on one stream are safe.
+ * it is staged.  Active sets of up to 512 jobs are simulated in shared memory on the whole GPU, as
+ * by sim_run; the instances that outgrow it run afterwards on the array's global-memory workspaces,
+ * 128 at a time.  All calls share that array and it keeps the last call's contents: calls that
+ * overlap on the GPU (different streams or threads) race; calls on one stream are safe.
  * The first call on each device looks up the array's device address (cudaGetSymbolAddress) with
  * that device current.  Allocates nothing.
  * Returns SIM_OK, SIM_E_INVAL, SIM_E_CUDA or SIM_E_STATE.

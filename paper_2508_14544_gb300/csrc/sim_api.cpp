@@ -341,7 +341,8 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
     // (64 instances of 10^5 requests: 1.5-3.7 % faster than four to a block on 16 SMs)
     if (!dense && !c->wpb_set && n_work <= n_sm) wpb = 1;
     simgb::RunParams p;
-    p.ca = smem ? (dense ? simgb::kDenseCa : c->smem_ca) : ((std::max(c->n_max, 128) + 127) / 128) * 128;
+    const int all = ((std::max(c->n_max, 128) + 127) / 128) * 128;  // >= any active set
+    p.ca = smem ? std::min(dense ? simgb::kDenseCa : c->smem_ca, all) : all;
     p.dcap = simgb::delta_cap(c->n_max);
     p.use_smem = smem ? 1 : 0;
     p.wide = dense ? 0 : 1;
@@ -384,6 +385,8 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
     }
     p.M = c->M;
     p.n_work = n_work;
+    p.n_work_dev = nullptr;
+    p.redo = p.redo_count = nullptr;
     p.work = work_dev;
     p.counter = c->d_counter;
     p.rec = c->d_rec;

@@ -61,8 +61,11 @@ struct StageParams {
 struct RunParams {
     int64_t M;
     int32_t n_work;            // instances to run in this launch
+    const int32_t *n_work_dev; // optional: their number on the device (the redo count of an earlier launch)
     const int32_t *work;       // instance ids (n_work)
     int32_t *counter;          // work-queue cursor (zeroed before launch)
+    int32_t *redo;             // optional: ids of the instances that outgrew the capacity are listed here
+    int32_t *redo_count;       // their number (zeroed before launch)
     const QEnt *rec;
     const int32_t *rec_a;
     const InstInfo *info;
@@ -83,7 +86,7 @@ struct RunParams {
     unsigned char *gws;        // global workspace base (use_smem == 0)
     int64_t gws_stride;        // bytes per warp slot
     QEnt *mainbuf;             // ping-pong main-queue buffers, 2 * main_cap per warp slot
-    int64_t main_cap;
+    int64_t main_cap;          // 0: two buffers of n entries per instance, at twice its first request
 };
 
 constexpr int kDenseCa = 384;      // active-set slots per warp of the dense configuration

@@ -278,11 +278,13 @@ __device__ __noinline__ void merge_delta(int32_t *pos, const QEnt *dq, QEnt *mb0
     *qp = q;
 }
 
-// The warp's ping-pong buffers are found from its slot here, not held in registers.
-__device__ __forceinline__ void merge_delta(const RunParams &P, const Ws &w, Queue &q, int64_t *gb) {
+// The ping-pong buffers (of the warp's slot, or of the instance at its first request `base`) are found
+// here, not held in registers.
+__device__ __forceinline__ void merge_delta(const RunParams &P, const Ws &w, Queue &q, int64_t base, int n, int64_t *gb) {
     Queue qq = q;
-    QEnt *mb = P.mainbuf + warp_slot() * 2 * P.main_cap;
-    merge_delta(w.cnt, w.dq, mb, mb + P.main_cap, &qq, gb);
+    const bool slots = P.main_cap > 0;
+    QEnt *mb = P.mainbuf + 2 * (slots ? warp_slot() * P.main_cap : base);
+    merge_delta(w.cnt, w.dq, mb, mb + (slots ? P.main_cap : n), &qq, gb);
     q = qq;
 }
 
@@ -325,8 +327,9 @@ __device__ __forceinline__ void delta_put(const Ws &w, Queue &q, const QEnt &e) 
 }
 
 // The same, merging the delta into main first if it is full.
-__device__ __forceinline__ void delta_insert(const RunParams &P, const Ws &w, Queue &q, const QEnt &e, int64_t *gb) {
-    if (q.dn == w.dcap) merge_delta(P, w, q, gb);
+__device__ __forceinline__ void delta_insert(const RunParams &P, const Ws &w, Queue &q, const QEnt &e, int64_t base, int n,
+                                             int64_t *gb) {
+    if (q.dn == w.dcap) merge_delta(P, w, q, base, n, gb);
     delta_put(w, q, e);
 }
 
@@ -353,8 +356,9 @@ __device__ __forceinline__ QEnt queue_head(const Ws &w, const Queue &q, int &src
 // is empty and extends it under A_ell when it follows it in the staged records (FIFO keys); a few
 // entries go into the delta one by one; a long batch is copied into the emptied delta in chunks.
 template <int POL>
-__device__ __forceinline__ void insert_run(const RunParams &P, const Ws &w, Queue &q, const QEnt *rec, int n, int ap,
+__device__ __forceinline__ void insert_run(const RunParams &P, const Ws &w, Queue &q, int64_t base, int n, int ap,
                                            int ae, int64_t &gb, int64_t *gbp) {
+    const QEnt *rec = P.rec + base;
     const int lane = lane_id();
     const int len = ae - ap;
     gb += int64_t(len) * int64_t(sizeof(QEnt));
@@ -380,10 +384,10 @@ __device__ __forceinline__ void insert_run(const RunParams &P, const Ws &w, Queu
         const int rem = len - done;
         if (rem <= 8) {
             #pragma unroll 1
-            for (int j = 0; j < rem; ++j) delta_insert(P, w, q, run[done + j], gbp);
+            for (int j = 0; j < rem; ++j) delta_insert(P, w, q, run[done + j], base, n, gbp);
             break;
         }
-        if (q.dn > 0) merge_delta(P, w, q, gbp);
+        if (q.dn > 0) merge_delta(P, w, q, base, n, gbp);
         const int k = min(rem, w.dcap);
         #pragma unroll 1
         for (int j = lane; j < k; j += 32) w.dq[j] = run[done + k - 1 - j];  // descending
@@ -543,7 +547,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
     r.total_latency = r.makespan = r.peak_memory = r.evictions = r.steps = r.request_steps = 0;
     r.status = info.status;
     r.pad = 0;
-    if (info.status == ST_OK && int64_t(info.n) > P.main_cap) r.status = ST_INVAL;  // larger than the queue buffers
+    if (info.status == ST_OK && P.main_cap > 0 && int64_t(info.n) > P.main_cap) r.status = ST_INVAL;  // larger than the queue buffers
     if (r.status != ST_OK || info.n == 0) {
         if (lane == 0) P.res[inst] = r;
         return;
@@ -659,7 +663,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 nextF = __reduce_min_sync(FULL, f);
             }
             bool dirty = (attn & (HEAD | MERGE)) != 0;
-            if (POL == P_AMIN && (attn & MERGE)) merge_delta(P, w, q, gbp);
+            if (POL == P_AMIN && (attn & MERGE)) merge_delta(P, w, q, base, n, gbp);
             attn = 0;
             // ---- S1: arrivals with a <= t join R_t (a sorted run of the staged records)
             if (next_a <= t) {
@@ -682,7 +686,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                         pa = apb + lane < n ? P.rec_a[base + apb + lane] : INT_MAX;
                     }
                 }
-                insert_run<POL>(P, w, q, P.rec + base, n, ap, ae, gbq, gbp);
+                insert_run<POL>(P, w, q, base, n, ap, ae, gbq, gbp);
                 if (INS) gbq += int64_t(ae - ap) * 4;  // their arrival steps
                 if (bt) {
                     const int64_t m = ae - ap;
@@ -732,7 +736,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                         --A;
                         ++nev;
                         if (INS) ++ev_step;
-                        delta_insert(P, w, q, e, gbp);
+                        delta_insert(P, w, q, e, base, n, gbp);
                     }
                 }
                 nextF = __reduce_min_sync(FULL, f);
@@ -1041,6 +1045,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
         r.steps = t - tb;
         r.request_steps = rsteps;
         P.res[inst] = r;
+        if (status == kStatusCapacity && P.redo) P.redo[atomicAdd(P.redo_count, 1)] = inst;
         if (bt) {
             int64_t *o = P.batch_time + 6 * int64_t(inst);
             const bool ok = status == ST_OK;
@@ -1074,11 +1079,12 @@ __global__ void __launch_bounds__(WIDE ? 128 : 256, WIDE ? 3 : 2) k_run(RunParam
     if (SMEM) base = smem_raw + size_t(threadIdx.x >> 5) * ws_bytes(POL == P_AMIN, P.ca, P.dcap);
     else base = P.gws + warp_slot() * P.gws_stride;
     Ws w = carve_ws(base, P.ca, P.dcap);
+    const int n_work = P.n_work_dev ? *P.n_work_dev : P.n_work;
     for (;;) {
         int k = 0;
         if (lane == 0) k = atomicAdd(P.counter, 1);
         k = __shfl_sync(FULL, k, 0);
-        if (k >= P.n_work) break;
+        if (k >= n_work) break;
         const int inst = P.work ? P.work[k] : k;
         sim_instance<POL, SMEM, INS>(P, w, inst);
     }

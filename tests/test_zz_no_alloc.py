@@ -112,3 +112,43 @@ def test_noalloc_rejects_oversize_inputs():
     rc = L.sim_run_noalloc(L.SIM_AMIN, 10_000, off, *dev, out)
     assert rc == L.SIM_E_INVAL
     assert "262144" in L.sim_last_error(None)
+
+
+@pytest.mark.parametrize("pol", [0, 1, 2])
+def test_noalloc_sets_beyond_shared_memory(pol):
+    """Instances whose active set outgrows the shared-memory slots (one-token prompts, up to 2000 jobs at
+    once) between small ones: the second launch simulates exactly those."""
+    import torch
+
+    from paper_2508_14544_gb300 import workloads as W
+    from paper_2508_14544_gb300 import _lib as L
+    rng = np.random.default_rng(17)
+    parts = []
+    for n in (2000, 30, 513, 512, 511, 1, 2048, 0, 700, 64):
+        o = rng.integers(1, 6, n)
+        a = np.sort(rng.integers(0, 3, n))
+        parts.append(dict(a=a, s=np.ones(n, np.int64), l=np.ones(n, np.int64), u=o + 2, o=o))
+    w = W.concat_instances("wide", 6000, parts)
+    out = torch.zeros(w.n_instances * L.RESULT_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+    dev = _dev(w)
+    for _ in range(2):
+        _check(_noalloc(pol, w, dev, out), _oracle(pol, w), f"wide pol={pol}")
+
+
+def test_noalloc_more_instances_than_warps():
+    """16384 instances (the limit), several per simulating warp, with queues that spill to their own
+    buffers."""
+    import torch
+
+    from paper_2508_14544_gb300 import workloads as W
+    from paper_2508_14544_gb300 import _lib as L
+    rng = np.random.default_rng(18)
+    parts = []
+    for i in range(16384):
+        n = 300 if i % 64 == 0 else int(rng.integers(0, 12))
+        o = rng.integers(1, 30, n)
+        l = rng.integers(1, o + 1)
+        parts.append(dict(a=np.sort(rng.integers(0, 40, n)), s=rng.integers(1, 9, n), l=l, u=o + 5, o=o))
+    w = W.concat_instances("many", 120, parts)
+    out = torch.zeros(w.n_instances * L.RESULT_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+    _check(_noalloc(L.SIM_AMIN, w, _dev(w), out), _oracle(L.SIM_AMIN, w), "many")
