@@ -8,6 +8,10 @@
 //              Algorithms milb / milbrevise, o for Algorithm off, the given permutation rank for
 //              Algorithm random, and the FIFO position 2 a for Algorithm promote_l, which also
 //              gets its (l, u) table).
+//   k_stage_large - the same for instances of more than kStageSmemN requests, one CTA of 1024 threads
+//              each.  When the requests come in arrival order in groups of at most 32 per step, every
+//              request finds its place by comparing itself with its group; otherwise an LSD radix sort in
+//              global memory on 8-bit digits.
 //   k_ratio  - per instance TEL(pi) / TEL(H-SF) in IEEE double (Definition cr).
 //   k_batch_time - per instance total latency and makespan in time units under a linear
 //              batch-time model (Section 6), from the integer sums the simulation recorded.
@@ -28,10 +32,37 @@ struct BtCoef {
     double k[5];
 };
 
-__device__ __forceinline__ bool stage_less(int aa, const QEnt &x, int ab, const QEnt &y) {
-    if (aa != ab) return aa < ab;
-    if (x.key != y.key) return x.key < y.key;
-    return x.idx < y.idx;
+// Policy key of the request at g (validity is checked by stage_check).
+__device__ __forceinline__ int stage_key(const StageParams &S, int64_t g) {
+    switch (S.policy) {
+        case P_AMAX: return S.u[g];
+        case P_HSF: return S.o[g];
+        case P_AR: return S.rank[g];
+        case P_AELL: return 2 * min(S.a[g], kAellMaxStep);
+        default: return S.l[g];
+    }
+}
+
+// Validates the request at g, fills A_ell's (l, u) table and adds to the instance's sums.
+struct StageSums {
+    int64_t bad_inval, bad_inf, sum_a, sum_o;
+    int kmax, amax;
+};
+
+__device__ __forceinline__ void stage_check(const StageParams &S, int64_t g, int a, int s, int o, int key, StageSums &z) {
+    const int l = S.l[g], u = S.u[g];
+    if (s < 1 || a < 0 || l < 1 || l > o || o > u) z.bad_inval = 1;
+    if (int64_t(s) + o > S.M) z.bad_inf = 1;
+    if ((S.policy == P_AMAX || S.policy == P_AELL) && int64_t(s) + u > S.M) z.bad_inf = 1;
+    if (S.policy == P_AR && key < 0) z.bad_inval = 1;
+    if (S.policy == P_AELL) {
+        if (a > kAellMaxStep) z.bad_inval = 1;
+        S.lu[g] = make_int2(l, u);
+    }
+    z.sum_a += a;
+    z.sum_o += o;
+    z.kmax = max(z.kmax, key);
+    z.amax = max(z.amax, a);
 }
 
 template <typename T>
@@ -50,30 +81,26 @@ __device__ T block_reduce(T v, T *sh, bool is_max) {
     return acc;
 }
 
-// Bitonic sort of n records by (a, key, idx) in place in global memory, padded virtually to a
-// power of two (positions >= n take no part): instances too large for shared memory.
-__device__ void bitonic_sort(QEnt *R, int32_t *RA, int n) {
-    int N = 1;
-    while (N < n) N <<= 1;
-    for (int k = 2; k <= N; k <<= 1) {
-        for (int d = k >> 1, ld = __ffs(d) - 1; d >= 1; d >>= 1, --ld) {
-            for (int p = threadIdx.x; p < N / 2; p += blockDim.x) {
-                const int i = ((p >> ld) << (ld + 1)) | (p & (d - 1));  // d is a power of two
-                const int j = (d == (k >> 1)) ? (i | (k - 1)) - (i & (k - 1)) : i + d;  // first pass: mirror
-                if (j < n) {
-                    const QEnt x = R[i], y = R[j];
-                    const int ax = RA[i], ay = RA[j];
-                    if (stage_less(ay, y, ax, x)) {
-                        R[i] = y;
-                        R[j] = x;
-                        RA[i] = ay;
-                        RA[j] = ax;
-                    }
-                }
-            }
-            __syncthreads();
-        }
+// Block-wide sums of z (kmax and amax are replaced by the block's), the instance's constants and status.
+__device__ int stage_finish(const StageParams &S, int inst, int64_t base, int n, StageSums &z, int64_t *sh64) {
+    const int64_t bad_inval = block_reduce<int64_t>(z.bad_inval, sh64, true);
+    const int64_t bad_inf = block_reduce<int64_t>(z.bad_inf, sh64, true);
+    const int64_t sum_a = block_reduce<int64_t>(z.sum_a, sh64, false);
+    const int64_t sum_o = block_reduce<int64_t>(z.sum_o, sh64, false);
+    z.kmax = int(block_reduce<int64_t>(z.kmax, sh64, true));
+    z.amax = int(block_reduce<int64_t>(z.amax, sh64, true));
+    const int status = bad_inval ? ST_INVAL : bad_inf ? ST_INFEASIBLE : ST_OK;
+    if (threadIdx.x == 0) {
+        InstInfo in;
+        in.base = base;
+        in.n = n;
+        in.status = status;
+        in.sum_a = sum_a;
+        in.cap = S.step_cap > 0 ? S.step_cap : 64 * (int64_t(n) + sum_o);
+        S.info[inst] = in;
     }
+    __syncthreads();
+    return status;
 }
 
 // Instances of up to this many requests are sorted in shared memory: per request its key, arrival,
@@ -181,8 +208,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageParams S, int np) 
     // instance before anything is written: it is staged as empty with status INVAL
     const bool oob = base < 0 || n64 < 0 || n64 > S.max_n || base + n64 > S.max_total;
     const int n = oob ? 0 : int(n64);
-    int64_t bad_inval = oob ? 1 : 0, bad_inf = 0, sum_a = 0, sum_o = 0, kmax = 0, amax = 0;
-    const bool in_smem = n <= np;
+    if (n > np) return;  // k_stage_large
     int32_t *kk = reinterpret_cast<int32_t *>(stage_smem);
     int32_t *ka = kk + np;
     int32_t *ss = ka + np;
@@ -190,72 +216,20 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageParams S, int np) 
     int32_t *i0 = so + np;
     int32_t *i1 = i0 + np;
     uint16_t *cnt = reinterpret_cast<uint16_t *>(i1 + np);
+    StageSums z = {oob ? 1 : 0, 0, 0, 0, 0, 0};
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
         const int64_t g = base + j;
-        const int a = S.a[g], s = S.s[g], l = S.l[g], u = S.u[g], o = S.o[g];
-        if (s < 1 || a < 0 || l < 1 || l > o || o > u) bad_inval = 1;
-        if (int64_t(s) + o > S.M) bad_inf = 1;
-        if ((S.policy == P_AMAX || S.policy == P_AELL) && int64_t(s) + u > S.M) bad_inf = 1;
-        int key;
-        switch (S.policy) {
-            case P_AMAX: key = u; break;
-            case P_HSF: key = o; break;
-            case P_AR: key = S.rank[g]; break;
-            case P_AELL: key = 2 * min(a, kAellMaxStep); break;
-            default: key = l; break;
-        }
-        if (S.policy == P_AR && key < 0) bad_inval = 1;
-        if (S.policy == P_AELL) {
-            if (a > kAellMaxStep) bad_inval = 1;
-            S.lu[g] = make_int2(l, u);  // indexed by request: j == idx below
-        }
-        if (in_smem) {
-            kk[j] = key;
-            ka[j] = a;
-            ss[j] = s;
-            so[j] = o;
-            i0[j] = j;
-        } else {
-            QEnt e;
-            e.key = key;
-            e.idx = j;
-            e.s = s;
-            e.o = o;
-            S.rec[g] = e;
-            S.rec_a[g] = a;
-        }
-        sum_a += a;
-        sum_o += o;
-        kmax = max(kmax, int64_t(key));
-        amax = max(amax, int64_t(a));
+        const int a = S.a[g], s = S.s[g], o = S.o[g], key = stage_key(S, g);
+        stage_check(S, g, a, s, o, key, z);
+        kk[j] = key;
+        ka[j] = a;
+        ss[j] = s;
+        so[j] = o;
+        i0[j] = j;
     }
-    bad_inval = block_reduce<int64_t>(bad_inval, sh64, true);
-    bad_inf = block_reduce<int64_t>(bad_inf, sh64, true);
-    sum_a = block_reduce<int64_t>(sum_a, sh64, false);
-    sum_o = block_reduce<int64_t>(sum_o, sh64, false);
-    if (in_smem) {
-        kmax = block_reduce<int64_t>(kmax, sh64, true);
-        amax = block_reduce<int64_t>(amax, sh64, true);
-    }
-    int status = ST_OK;
-    if (bad_inval) status = ST_INVAL;
-    else if (bad_inf) status = ST_INFEASIBLE;
-    if (threadIdx.x == 0) {
-        InstInfo in;
-        in.base = oob ? 0 : base;
-        in.n = n;
-        in.status = status;
-        in.sum_a = sum_a;
-        in.cap = S.step_cap > 0 ? S.step_cap : 64 * (int64_t(n) + sum_o);
-        S.info[inst] = in;
-    }
-    __syncthreads();
-    if (!in_smem) {
-        if (status == ST_OK && n > 1) bitonic_sort(S.rec + base, S.rec_a + base, n);
-        return;
-    }
+    const int status = stage_finish(S, inst, oob ? 0 : base, n, z, sh64);
     const int32_t *ord = i0;
-    if (status == ST_OK && n > 1) ord = radix_sort_idx(kk, ka, i0, i1, cnt, wsum, n, int(kmax), int(amax));
+    if (status == ST_OK && n > 1) ord = radix_sort_idx(kk, ka, i0, i1, cnt, wsum, n, z.kmax, z.amax);
     // write the (sorted, or for a rejected instance unsorted) records out
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
         const int idx = ord[j];
@@ -266,6 +240,166 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageParams S, int np) 
         e.o = so[idx];
         S.rec[base + j] = e;
         S.rec_a[base + j] = ka[idx];
+    }
+}
+
+// ---- instances of more than kStageSmemN requests ----------------------------------------------
+
+constexpr int kLargeThreads = 1024;
+constexpr int kLargeWarps = kLargeThreads / 32;
+constexpr int kLargeGroup = 32;  // longest run of equal arrival steps that is ranked directly
+
+// One stable pass of the LSD radix sort over n (value, index) pairs by the 8 bits of the value at
+// `shift`, value replaced by a[index] first if a is given.  Per tile of 4096 pairs a warp takes 128
+// consecutive ones: ranks within the warp by match_any and per-warp counters, whose sums over the
+// warps (one thread per digit) on top of the digit's running position are the output positions.
+__device__ void large_radix_pass(const int2 *in, int2 *out, const int32_t *a, int n, int shift, int32_t *cnt,
+                                 int32_t *pos) {
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    if (t < 256) pos[t] = 0;
+    __syncthreads();
+    for (int b = 0; b < n; b += kLargeThreads) {
+        const int e = b + t;
+        int d = 256;
+        if (e < n) {
+            const int2 x = in[e];
+            d = ((a ? a[x.y] : x.x) >> shift) & 255;
+        }
+        const unsigned peers = __match_any_sync(FULL, d);
+        if (d < 256 && (peers & lt) == 0) atomicAdd(&pos[d], __popc(peers));
+    }
+    __syncthreads();
+    if (t < 32) {  // exclusive prefix sums of the 256 digit counts
+        int v[8], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[k] = pos[8 * t + k];
+            sum += v[k];
+        }
+        int x = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(FULL, x, d);
+            if (lane >= d) x += y;
+        }
+        int run = x - sum;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            pos[8 * t + k] = run;
+            run += v[k];
+        }
+    }
+    __syncthreads();
+    for (int b = 0; b < n; b += 4 * kLargeThreads) {
+        for (int k = t; k < 256 * kLargeWarps; k += kLargeThreads) cnt[k] = 0;
+        __syncthreads();
+        int2 x[4];
+        int d[4], rk[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int e = b + w * 128 + r * 32 + lane;
+            d[r] = 256;
+            if (e < n) {
+                x[r] = in[e];
+                if (a) x[r].x = a[x[r].y];
+                d[r] = (x[r].x >> shift) & 255;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const unsigned peers = __match_any_sync(FULL, d[r]);
+            int32_t *c = cnt + w * 256 + (d[r] & 255);
+            rk[r] = d[r] < 256 ? *c + __popc(peers & lt) : 0;
+            __syncwarp();
+            if (d[r] < 256 && (peers & lt) == 0) *c += __popc(peers);
+            __syncwarp();
+        }
+        __syncthreads();
+        if (t < 256) {
+            int run = pos[t];
+            for (int k = 0; k < kLargeWarps; ++k) {
+                const int c = cnt[k * 256 + t];
+                cnt[k * 256 + t] = run;
+                run += c;
+            }
+            pos[t] = run;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (d[r] < 256) out[cnt[w * 256 + d[r]] + rk[r]] = x[r];
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kLargeThreads) k_stage_large(StageParams S, int np) {
+    __shared__ int64_t sh64[32];
+    __shared__ int32_t pos[256];
+    extern __shared__ __align__(16) unsigned char stage_smem[];
+    const int inst = blockIdx.x;
+    const int64_t base = S.off[inst];
+    const int64_t n64 = S.off[inst + 1] - base;
+    if (base < 0 || n64 <= np || n64 > S.max_n || base + n64 > S.max_total) return;  // k_stage
+    const int n = int(n64);
+    StageSums z = {0, 0, 0, 0, 0, 0};
+    int far = 0;  // requests not in arrival order, or more than kLargeGroup of them in one step
+    for (int j = threadIdx.x; j < n; j += kLargeThreads) {
+        const int64_t g = base + j;
+        const int a = S.a[g];
+        stage_check(S, g, a, S.s[g], S.o[g], stage_key(S, g), z);
+        if (j > 0 && S.a[g - 1] > a) far = 1;
+        if (j >= kLargeGroup && S.a[g - kLargeGroup] >= a) far = 1;
+    }
+    const int status = stage_finish(S, inst, base, n, z, sh64);
+    if (status != ST_OK) return;
+    if (!__syncthreads_or(far)) {
+        // place = the group's first place + the group's smaller (key, index)
+        for (int j = threadIdx.x; j < n; j += kLargeThreads) {
+            const int64_t g = base + j;
+            QEnt e;
+            e.key = stage_key(S, g);
+            e.idx = j;
+            e.s = S.s[g];
+            e.o = S.o[g];
+            const int a = S.a[g];
+            int place = j;
+            for (int k = j - 1; k >= 0 && S.a[base + k] == a; --k)
+                if (stage_key(S, base + k) > e.key) --place;
+            for (int k = j + 1; k < n && S.a[base + k] == a; ++k)
+                if (stage_key(S, base + k) < e.key) ++place;
+            S.rec[base + place] = e;
+            S.rec_a[base + place] = a;
+        }
+        return;
+    }
+    // the pairs live in the instance's record space (two buffers of n pairs), the final order in rec_a
+    int2 *in = reinterpret_cast<int2 *>(S.rec + base), *out = in + n;
+    int32_t *cnt = reinterpret_cast<int32_t *>(stage_smem);
+    for (int j = threadIdx.x; j < n; j += kLargeThreads) in[j] = make_int2(stage_key(S, base + j), j);
+    __syncthreads();
+    const int kbits = z.kmax > 0 ? 32 - __clz(z.kmax) : 0, abits = z.amax > 0 ? 32 - __clz(z.amax) : 0;
+    for (int p = 0; p < kbits + abits + 14; p += 8) {
+        const bool arr = p >= ((kbits + 7) & ~7);
+        const int shift = arr ? p - ((kbits + 7) & ~7) : p;
+        if (arr && shift >= abits) break;
+        large_radix_pass(in, out, arr && shift == 0 ? S.a + base : nullptr, n, shift, cnt, pos);
+        int2 *tmp = in;
+        in = out;
+        out = tmp;
+    }
+    for (int j = threadIdx.x; j < n; j += kLargeThreads) S.rec_a[base + j] = in[j].y;
+    __syncthreads();
+    for (int j = threadIdx.x; j < n; j += kLargeThreads) {
+        const int idx = S.rec_a[base + j];
+        const int64_t g = base + idx;
+        QEnt e;
+        e.key = stage_key(S, g);
+        e.idx = idx;
+        e.s = S.s[g];
+        e.o = S.o[g];
+        S.rec[base + j] = e;
+        S.rec_a[base + j] = S.a[g];
     }
 }
 
@@ -329,6 +463,7 @@ cudaError_t launch_stage(const StageParams &p, cudaStream_t st) {
         if (e != cudaSuccess) return e;
     }
     k_stage<<<p.n_inst, kStageThreads, smem, st>>>(p, np);
+    if (p.n_max > np) k_stage_large<<<p.n_inst, kLargeThreads, 256 * kLargeWarps * sizeof(int32_t), st>>>(p, np);
     return cudaGetLastError();
 }
 

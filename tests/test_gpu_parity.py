@@ -183,3 +183,29 @@ def test_c3_full(pol):
     got, _ = gpu_run(pol, w)
     ref = oracle_run(pol, w)
     assert_same(got, ref, tag=f"c3 pol={pol}")
+
+
+@pytest.mark.parametrize("pol", [1, 3, 4])
+def test_staging_large_instances(pol):
+    """Instances above the shared-memory staging limit next to small ones: sorted arrivals in groups of
+    32 (ranked directly) and 33 (radix sort), one burst, unsorted arrivals over one to three 8-bit
+    digits, sizes around the radix tile (4096 pairs), keys of one and of three digits, and long ties."""
+    from fractions import Fraction
+
+    from paper_2508_14544_gb300 import workloads as W
+    rng = np.random.default_rng(23)
+    parts = []
+    sizes = [2049, 4095, 4096, 4097, 3000, 8193, 5000, 2048, 7, 12289]
+    for i, n in enumerate(sizes):
+        big = i % 4 == 3  # a few lengths of 17 bits
+        o = np.where(rng.random(n) < 0.002, 70000, 3) if big else rng.choice([1, 2, 3, 17, 40], n)
+        l, u = W.interval_for(o, Fraction(1), rng) if big else W.interval_for(o, Fraction(1, 3), rng)
+        a = [np.sort(rng.integers(0, 4 * n, n)), np.repeat(np.arange(-(-n // 32)), 32)[:n] * 3,
+             np.repeat(np.arange(-(-n // 33)), 33)[:n], rng.integers(0, 1 << 18, n), np.zeros(n, np.int64),
+             rng.integers(0, 200, n), rng.integers(0, 70000, n)][i % 7]
+        parts.append(dict(a=a, s=rng.integers(1, 9, n), l=l, u=u, o=o))
+    w = W.concat_instances("staging-large", 90000, parts)
+    got, comp = gpu_run(pol, w, completions=True)
+    ref, rcomp = oracle_run(pol, w, completions=True)
+    assert_same(got, ref, tag=f"staging pol={pol}")
+    assert np.array_equal(comp, rcomp)
