@@ -98,15 +98,13 @@ constexpr int kMc = 64;            // cached entries of the main queue (two per 
 // Delta-queue entries used for an instance of n requests.
 __host__ __device__ constexpr int delta_cap(int64_t n) { return n <= 1024 ? 64 : (n <= 4096 ? 128 : kDcap); }
 
-// Workspace of one simulating warp: ca slots of {E, V, B, F} (16 bytes), the delta queue, the head
-// cache of the main queue (whose space also holds the dcap positions of a merge), {P, I} per
-// slot (8 bytes) and, under A_min, the estimate per slot (4 bytes).
-__host__ __device__ constexpr size_t ws_cache_bytes(int dcap) {
-    const size_t cache = size_t(kMc) * sizeof(QEnt), pos = size_t(dcap) * 4;
-    return cache > pos ? cache : pos;
-}
-__host__ __device__ constexpr size_t ws_bytes(bool amin, int ca, int dcap) {
-    return size_t(ca) * (amin ? 28 : 24) + size_t(dcap) * sizeof(QEnt) + ws_cache_bytes(dcap);
+// Workspace of one simulating warp, in this order: ca slots of {E, W, B, F} (16 bytes) and {P, I} (8), the
+// head cache of the main queue (whose space also holds the positions of a merge), the A_min estimate per
+// slot (4) and the delta queue.
+constexpr size_t kWsCacheBytes = size_t(kMc) * sizeof(QEnt);
+static_assert(size_t(kDcap) * 4 <= kWsCacheBytes, "merge positions");
+__host__ __device__ constexpr size_t ws_bytes(int ca, int dcap) {
+    return size_t(ca) * 28 + kWsCacheBytes + size_t(dcap) * sizeof(QEnt);
 }
 
 cudaError_t launch_stage(const StageParams &p, cudaStream_t st);

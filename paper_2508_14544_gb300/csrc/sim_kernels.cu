@@ -132,14 +132,16 @@ struct Ws {
     int32_t ca, dcap;
 };
 
+// The slot arrays and the head cache come first: with a capacity known at compile time they are constant
+// offsets from one address.
 __device__ __forceinline__ Ws carve_ws(unsigned char *base, int ca, int dcap) {
     Ws w;
     w.H = reinterpret_cast<int4 *>(base);
-    w.dq = reinterpret_cast<QEnt *>(w.H + ca);
-    w.mc = w.dq + dcap;
+    w.C = reinterpret_cast<int2 *>(w.H + ca);
+    w.mc = reinterpret_cast<QEnt *>(w.C + ca);
     w.cnt = reinterpret_cast<int32_t *>(w.mc);
-    w.C = reinterpret_cast<int2 *>(reinterpret_cast<unsigned char *>(w.mc) + ws_cache_bytes(dcap));
-    w.K = reinterpret_cast<unsigned *>(w.C + ca);
+    w.K = reinterpret_cast<unsigned *>(reinterpret_cast<unsigned char *>(w.mc) + kWsCacheBytes);
+    w.dq = reinterpret_cast<QEnt *>(w.K + ca);
     w.ca = ca;
     w.dcap = dcap;
     return w;
@@ -409,8 +411,12 @@ __device__ __forceinline__ void over_slots(bool half, int end, Body body) {
     if (half) {
         body(Slots<kHalf / 32>(), 0);
     } else {
+        int p = 0;
         #pragma unroll 1
-        for (int p = 0; p < end; p += kPage) body(Slots<kPage / 32>(), p);
+        do {
+            body(Slots<kPage / 32>(), p);
+            p += kPage;
+        } while (p < end);
     }
 }
 
@@ -954,10 +960,14 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                         ek = early ? a[j].x : ek;
                         bk = early ? a[j].z : bk;
                     }
-                    a[j] = make_int4(-1, a[j].x, a[j].z, kEarly ? -2 - t : -1);
-                    if (done) w.H[p + 32 * j + lane] = a[j];  // nothing else in the branch: one predicated store
-                    if (POL == P_AMIN)
-                        if (done) w.K[p + 32 * j + lane] = UINT_MAX;
+                    if (kEarly) {
+                        a[j] = make_int4(-1, a[j].x, a[j].z, -2 - t);
+                        if (done) w.H[p + 32 * j + lane] = a[j];  // nothing else in the branch: one predicated store
+                    } else if (done) {
+                        w.H[p + 32 * j + lane].x = -1;
+                        w.H[p + 32 * j + lane].w = -1;
+                        if (POL == P_AMIN) w.K[p + 32 * j + lane] = UINT_MAX;
+                    }
                 }
             });
             c = int(__reduce_add_sync(FULL, unsigned(c)));
@@ -1068,17 +1078,20 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
 }
 
 // WIDE: up to 168 registers a thread (12 warps per SM), for launches whose time is one instance's serial
-// chain; otherwise 128 (16 warps per SM), for launches with more instances than that.  A_min at 128
-// registers spills 9 of them: the 256 x 10^4 online workload takes 28.5 ms against 26.9, the 40960 x 2000
-// one 111 ms at 16 warps per SM against 133 at 12.
-template <int POL, bool SMEM, bool INS, bool WIDE>
+// chain; otherwise 128 (16 warps per SM), for launches with more instances than that.  On the
+// 40960 x 2000 workload A_min takes 111 ms at 16 warps per SM and 133 at 12; the 256 x 10^4 online
+// workload 26.2 ms with 168 registers and 28.5 with 128 (spills).
+// CA: the slots per warp when fixed at compile time (the workspace arrays are then constant offsets from
+// one address: 2-5 % on every policy), or 0 for P.ca (the global-memory kernel and other capacities).
+template <int POL, bool SMEM, bool INS, bool WIDE, int CA>
 __global__ void __launch_bounds__(WIDE ? 128 : 256, WIDE ? 3 : 2) k_run(RunParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = lane_id();
+    const int ca = CA ? CA : P.ca;
     unsigned char *base;
-    if (SMEM) base = smem_raw + size_t(threadIdx.x >> 5) * ws_bytes(POL == P_AMIN, P.ca, P.dcap);
+    if (SMEM) base = smem_raw + size_t(threadIdx.x >> 5) * ws_bytes(ca, P.dcap);
     else base = P.gws + warp_slot() * P.gws_stride;
-    Ws w = carve_ws(base, P.ca, P.dcap);
+    Ws w = carve_ws(base, ca, P.dcap);
     const int n_work = P.n_work_dev ? *P.n_work_dev : P.n_work;
     for (;;) {
         int k = 0;
@@ -1093,21 +1106,24 @@ __global__ void __launch_bounds__(WIDE ? 128 : 256, WIDE ? 3 : 2) k_run(RunParam
 using KernelFn = void (*)(RunParams);
 
 template <int POL>
-KernelFn pick(bool smem, bool ins, bool wide) {
-    if (smem && ins) return wide ? k_run<POL, true, true, true> : k_run<POL, true, true, false>;
-    if (smem) return wide ? k_run<POL, true, false, true> : k_run<POL, true, false, false>;
-    return ins ? k_run<POL, false, true, false> : k_run<POL, false, false, false>;
+KernelFn pick(bool smem, bool ins, bool wide, int ca) {
+    if (!smem) return ins ? k_run<POL, false, true, false, 0> : k_run<POL, false, false, false, 0>;
+    if (wide && ca == kSmemCaDefault)
+        return ins ? k_run<POL, true, true, true, kSmemCaDefault> : k_run<POL, true, false, true, kSmemCaDefault>;
+    if (ins) return k_run<POL, true, true, false, 0>;
+    if (!wide && ca == kDenseCa) return k_run<POL, true, false, false, kDenseCa>;
+    return k_run<POL, true, false, false, 0>;
 }
 
 KernelFn run_fn(int policy, const RunParams &p, int warps_per_block) {
     const bool smem = p.use_smem != 0, ins = p.work_count != nullptr || p.batch_time != nullptr;
     const bool wide = p.wide != 0 && warps_per_block <= 4;
     switch (policy) {
-        case P_AMAX: return pick<P_AMAX>(smem, ins, wide);
-        case P_AMIN: return pick<P_AMIN>(smem, ins, wide);
-        case P_HSF: return pick<P_HSF>(smem, ins, wide);
-        case P_AR: return pick<P_AR>(smem, ins, wide);
-        default: return pick<P_AELL>(smem, ins, wide);
+        case P_AMAX: return pick<P_AMAX>(smem, ins, wide, p.ca);
+        case P_AMIN: return pick<P_AMIN>(smem, ins, wide, p.ca);
+        case P_HSF: return pick<P_HSF>(smem, ins, wide, p.ca);
+        case P_AR: return pick<P_AR>(smem, ins, wide, p.ca);
+        default: return pick<P_AELL>(smem, ins, wide, p.ca);
     }
 }
 

@@ -47,7 +47,7 @@ constexpr int64_t kNaSlots = int64_t(kNaBlocks) * kNaWarpsPerBlock;  // warps of
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // Workspace bytes per warp for an active-set capacity of kNaMaxPerInstance.
-constexpr size_t ws_bytes_max() { return simgb::ws_bytes(true, int(kNaMaxPerInstance), simgb::kDcap); }
+constexpr size_t ws_bytes_max() { return simgb::ws_bytes(int(kNaMaxPerInstance), simgb::kDcap); }
 
 constexpr size_t kOffOff = 0;
 constexpr size_t kOffRec = align256(kOffOff + size_t(kNaMaxInstances + 1) * sizeof(int64_t));
@@ -172,11 +172,15 @@ extern "C" int sim_run_noalloc(int policy, int64_t M, int32_t n_instances, const
     int n_sm = 0, per_sm = 1;
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     const int all = int(((std::max<int64_t>(n_max, 128) + 127) / 128) * 128);  // >= any active set
-    p.ca = std::min(all, simgb::kSmemCaDefault);
+    p.ca = simgb::kSmemCaDefault;
     p.dcap = simgb::delta_cap(n_max);
     p.use_smem = 1;
-    p.wide = n_instances <= 12 * n_sm ? 1 : 0;  // all instances at once, else more warps per SM
-    const size_t smem = simgb::ws_bytes(policy == SIM_AMIN, p.ca, p.dcap);
+    p.wide = 1;
+    if (n_instances > 12 * n_sm && all <= simgb::kDenseCa) {  // as in sim_run
+        p.ca = simgb::kDenseCa;
+        p.wide = 0;
+    }
+    const size_t smem = simgb::ws_bytes(p.ca, p.dcap);
     e = simgb::run_blocks_per_sm(policy, p, 1, smem, &per_sm);
     if (e != cudaSuccess) return fail(SIM_E_CUDA, "sim_run_noalloc: kernel set-up failed");
     const int blocks = int(std::min<int64_t>(int64_t(n_sm) * std::max(per_sm, 1), n_instances));
