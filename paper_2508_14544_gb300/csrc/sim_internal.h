@@ -98,7 +98,7 @@ constexpr int kMc = 64;            // cached entries of the main queue (two per 
 // Delta-queue entries used for an instance of n requests.
 __host__ __device__ constexpr int delta_cap(int64_t n) { return n <= 1024 ? 64 : (n <= 4096 ? 128 : kDcap); }
 
-// Workspace of one simulating warp, in this order: ca slots of {E, W, B, F} (16 bytes) and {P, I} (8), the
+// Workspace of one simulating warp, in this order: ca slots of {E, W}, B, F (16 bytes) and {P, I} (8), the
 // head cache of the main queue (whose space also holds the positions of a merge), the A_min estimate per
 // slot (4) and the delta queue.
 constexpr size_t kWsCacheBytes = size_t(kMc) * sizeof(QEnt);

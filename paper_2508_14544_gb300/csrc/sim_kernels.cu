@@ -123,7 +123,8 @@ __device__ __forceinline__ int proj_len(const RunParams &P, int64_t base, const 
 // Per-warp workspace (layout: ws_bytes in sim_internal.h)
 // ---------------------------------------------------------------------------------------------
 struct Ws {
-    int4 *H;         // active-set slots {E, W, B, F}, capacity ca (a multiple of kPage)
+    int2 *EW;        // active-set slots {E, W}, capacity ca (a multiple of kPage)
+    int32_t *B, *F;  // and their B and F
     QEnt *dq;        // delta queue, dcap entries, sorted DESCENDING (head = dq[dn-1])
     QEnt *mc;        // cached head of the main queue, kMc entries
     int32_t *cnt;    // merge positions, dcap entries: the cache's space (a merge invalidates it)
@@ -136,8 +137,10 @@ struct Ws {
 // offsets from one address.
 __device__ __forceinline__ Ws carve_ws(unsigned char *base, int ca, int dcap) {
     Ws w;
-    w.H = reinterpret_cast<int4 *>(base);
-    w.C = reinterpret_cast<int2 *>(w.H + ca);
+    w.EW = reinterpret_cast<int2 *>(base);
+    w.B = reinterpret_cast<int32_t *>(w.EW + ca);
+    w.F = w.B + ca;
+    w.C = reinterpret_cast<int2 *>(w.F + ca);
     w.mc = reinterpret_cast<QEnt *>(w.C + ca);
     w.cnt = reinterpret_cast<int32_t *>(w.mc);
     w.K = reinterpret_cast<unsigned *>(reinterpret_cast<unsigned char *>(w.mc) + kWsCacheBytes);
@@ -430,10 +433,17 @@ __device__ __forceinline__ void subtract_job(const Ws &w, int end, int e, int b)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int i = p + 32 * j + lane_id();
-            const int2 ew = *reinterpret_cast<const int2 *>(&w.H[i]);
-            if (unsigned(ew.x) <= unsigned(e)) w.H[i].y = ew.y - b - ew.x;
+            const int2 ew = w.EW[i];
+            if (unsigned(ew.x) <= unsigned(e)) w.EW[i].y = ew.y - b - ew.x;
         }
     }
+}
+
+template <int POL>
+__device__ __forceinline__ void free_slot(const Ws &w, int i) {
+    w.EW[i].x = -1;
+    w.F[i] = -1;
+    if (POL == P_AMIN) w.K[i] = UINT_MAX;
 }
 
 // Free the slots [from, from + kPage).
@@ -442,8 +452,7 @@ __device__ __forceinline__ void free_page(const Ws &w, int from) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int i = from + 32 * j + lane_id();
-        w.H[i] = make_int4(-1, 0, 0, -1);
-        if (POL == P_AMIN) w.K[i] = UINT_MAX;
+        free_slot<POL>(w, i);
     }
 }
 
@@ -455,23 +464,27 @@ __device__ __forceinline__ void compact(const Ws &w, int &end) {
     int wpos = 0;
     #pragma unroll 1
     for (int b = 0; b < end; b += kHalf) {
-        int4 h[2];
-        int2 c[2];
+        int2 e[2], c[2];
+        int bb[2], f[2];
         unsigned k[2], m[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int i = b + 32 * j + lane;
-            h[j] = w.H[i];
+            e[j] = w.EW[i];
+            bb[j] = w.B[i];
+            f[j] = w.F[i];
             c[j] = w.C[i];
             k[j] = POL == P_AMIN ? w.K[i] : 0u;
-            m[j] = __ballot_sync(FULL, h[j].w >= 0);
+            m[j] = __ballot_sync(FULL, f[j] >= 0);
         }
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int d = wpos + __popc(m[j] & lt);
-            if (h[j].w >= 0) {
-                w.H[d] = h[j];
+            if (f[j] >= 0) {
+                w.EW[d] = e[j];
+                w.B[d] = bb[j];
+                w.F[d] = f[j];
                 w.C[d] = c[j];
                 if (POL == P_AMIN) w.K[d] = k[j];
             }
@@ -481,8 +494,7 @@ __device__ __forceinline__ void compact(const Ws &w, int &end) {
     }
     #pragma unroll 1
     for (int i = wpos + lane; i < end; i += 32) {
-        w.H[i] = make_int4(-1, 0, 0, -1);
-        if (POL == P_AMIN) w.K[i] = UINT_MAX;
+        free_slot<POL>(w, i);
     }
     end = wpos;
     __syncwarp();
@@ -502,7 +514,7 @@ __device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int
     int cnt = 0, sum = 0;
     #pragma unroll 1
     for (int i = lane; i < filled; i += 32) {
-        const int4 h = w.H[i];
+        const int4 h = make_int4(w.EW[i].x, w.EW[i].y, w.B[i], w.F[i]);
         if (h.w < 0) {
             if (h.x != -1 || (POL == P_AMIN && w.K[i] != UINT_MAX)) bad = true;
             continue;
@@ -517,7 +529,7 @@ __device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int
         int v = h.x;
         #pragma unroll 1
         for (int j = 0; j < end; ++j)
-            if (w.H[j].x >= h.x) v += w.H[j].z + h.x;
+            if (w.EW[j].x >= h.x) v += w.B[j] + h.x;
         if (v != h.y + (h.x <= py ? h.x + pc : 0) - (h.x <= qy ? h.x + qc : 0)) bad = true;
     }
     if (int(__reduce_add_sync(FULL, unsigned(cnt))) != A || int(__reduce_add_sync(FULL, unsigned(sum))) != need) bad = true;
@@ -665,7 +677,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             if (POL == P_AMIN && (attn & NEXTF)) {
                 unsigned f = UINT_MAX;
                 #pragma unroll 1
-                for (int i = lane; i < end; i += 32) f = min(f, unsigned(w.H[i].w));
+                for (int i = lane; i < end; i += 32) f = min(f, unsigned(w.F[i]));
                 nextF = __reduce_min_sync(FULL, f);
             }
             bool dirty = (attn & (HEAD | MERGE)) != 0;
@@ -717,28 +729,28 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 unsigned f = UINT_MAX, e1 = UINT_MAX;
                 #pragma unroll 1
                 for (int b = 0; b < end; b += 32) {
-                    const int4 hh = w.H[b + lane];
-                    const bool out = unsigned(hh.x) < unsigned(t);
+                    const unsigned ei = unsigned(w.EW[b + lane].x), fi = unsigned(w.F[b + lane]);
+                    const bool out = ei < unsigned(t);
                     if (!out) {
-                        f = min(f, unsigned(hh.w));
-                        e1 = min(e1, unsigned(hh.x));
+                        f = min(f, fi);
+                        e1 = min(e1, ei);
                     }
                     unsigned m = __ballot_sync(FULL, out);
                     #pragma unroll 1
                     while (m) {
                         const int pos = b + __ffs(m) - 1;
                         m &= m - 1;
-                        const int4 j = w.H[pos];
+                        const int bj = w.B[pos], fj = w.F[pos];
                         const int2 pi = w.C[pos];
                         __syncwarp();
-                        w.H[pos] = make_int4(-1, 0, 0, -1);
+                        free_slot<POL>(w, pos);
                         __syncwarp();
                         QEnt e;
                         e.key = 2 * t + 1;
                         e.idx = pi.y;
-                        e.s = j.z + pi.x - 1;
-                        e.o = j.w - pi.x + 1;
-                        need -= j.z + t;
+                        e.s = bj + pi.x - 1;
+                        e.o = fj - pi.x + 1;
+                        need -= bj + t;
                         --A;
                         ++nev;
                         if (INS) ++ev_step;
@@ -784,13 +796,22 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             while (need > M && q.dn < w.dcap) {
                 unsigned bk = UINT_MAX;
                 int lo = 0, hi = 0;
+                const int pq = max(py, qy);
                 over_slots(half, end, [&](auto slots, int p) {
                     constexpr int N = decltype(slots)::value;
                     unsigned k[N], m = UINT_MAX;
+                    int2 x[N];
 #pragma unroll
                     for (int j = 0; j < N; ++j) {
                         k[j] = w.K[p + 32 * j + lane];
+                        x[j] = w.EW[p + 32 * j + lane];
+                    }
+#pragma unroll
+                    for (int j = 0; j < N; ++j) {
                         m = min(m, k[j]);
+                        if (x[j].x <= py) x[j].y += x[j].x + pc;
+                        if (x[j].x <= qy) x[j].y -= x[j].x + qc;
+                        if (x[j].x <= pq) w.EW[p + 32 * j + lane].y = x[j].y;
                     }
                     int first = 0, last = 0;
 #pragma unroll
@@ -810,30 +831,26 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 }
                 if (pos != pos2)
                     pos = tie_position(w.K, w.C, pos, pos2, mk, tie_base(tie_seed, t), P.evict_index == 0);
-                const int4 j = w.H[pos];
+                const int ej = w.EW[pos].x, bj = w.B[pos], fj = w.F[pos];
                 const int2 pi = w.C[pos];
                 __syncwarp();
-                w.H[pos] = make_int4(-1, 0, 0, -1);
-                w.K[pos] = UINT_MAX;
+                free_slot<POL>(w, pos);
                 __syncwarp();
                 QEnt e;
                 e.key = max(int(mk), t - pi.x);  // refined lower bound: max(estimate, tokens generated)
                 e.idx = pi.y;
-                e.s = j.z + pi.x - 1;
-                e.o = j.w - pi.x + 1;
-                need -= j.z + t;
+                e.s = bj + pi.x - 1;
+                e.o = fj - pi.x + 1;
+                need -= bj + t;
                 --A;
                 ++nev;
                 if (INS) ++ev_step;
-                if (unsigned(j.w) == nextF) attn |= NEXTF;
-                // endpoints before t need no update, and the update is left pending if none is
-                const int do_sub = j.x < t ? 0 : (qy < 0 ? 1 : 2);
-                if (__reduce_max_sync(FULL, do_sub) == 2) {
-                    subtract_job(w, end, j.x, j.z);
-                } else if (do_sub) {
-                    qy = j.x;
-                    qc = j.z;
-                }
+                if (unsigned(fj) == nextF) attn |= NEXTF;
+                // the pass above applied the pending updates; this one waits for the next pass (endpoints
+                // before t need none)
+                py = -2;
+                qy = ej < t ? -2 : ej;
+                qc = bj;
                 delta_put(w, q, e);
                 if (qless(e, h)) {  // the head of R_t is the smaller of the two
                     h = e;
@@ -856,16 +873,20 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             const int pq = kSub ? max(py, qy) : py;
             over_slots(half, end, [&](auto slots, int p) {
                 constexpr int N = decltype(slots)::value;
-                int4 a[N];
-#pragma unroll
-                for (int j = 0; j < N; ++j) a[j] = w.H[p + 32 * j + lane];
+                int2 x[N];
+                int bb[N];
 #pragma unroll
                 for (int j = 0; j < N; ++j) {
-                    if (a[j].x <= py) a[j].y += a[j].x + pc;
-                    if (kSub && a[j].x <= qy) a[j].y -= a[j].x + qc;
-                    if (a[j].x <= pq) w.H[p + 32 * j + lane].y = a[j].y;
-                    if (a[j].x >= y) vy += a[j].z + y;
-                    if (unsigned(a[j].x - t) < unsigned(hL)) wm = max(wm, a[j].y);
+                    x[j] = w.EW[p + 32 * j + lane];
+                    bb[j] = w.B[p + 32 * j + lane];
+                }
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    if (x[j].x <= py) x[j].y += x[j].x + pc;
+                    if (kSub && x[j].x <= qy) x[j].y -= x[j].x + qc;
+                    if (x[j].x <= pq) w.EW[p + 32 * j + lane].y = x[j].y;
+                    if (x[j].x >= y) vy += bb[j] + y;
+                    if (unsigned(x[j].x - t) < unsigned(hL)) wm = max(wm, x[j].y);
                 }
             });
             py = qy = -2;
@@ -884,7 +905,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                     constexpr int N = decltype(slots)::value;
 #pragma unroll
                     for (int j = 0; j < N; ++j) {
-                        const int2 ew = *reinterpret_cast<const int2 *>(&w.H[p + 32 * j + lane]);
+                        const int2 ew = w.EW[p + 32 * j + lane];
                         em = min(em, unsigned(ew.x - y));
                         if (unsigned(ew.x - t) < unsigned(hL)) r2 = max(r2, min(max(ew.y, lim) - lim, ew.x - t + 1));
                     }
@@ -897,7 +918,9 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             } else {
                 // the pending update of its own admission adds the job's memory at y to its W
                 __syncwarp();
-                w.H[end] = make_int4(y, vy + y, h.s - t + 1, t + h.o - 1);
+                w.EW[end] = make_int2(y, vy + y);
+                w.B[end] = h.s - t + 1;
+                w.F[end] = t + h.o - 1;
                 w.C[end] = make_int2(t, h.idx);
                 if (POL == P_AMIN) w.K[end] = unsigned(h.key);
                 py = y;
@@ -933,11 +956,6 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 k_step = ev_step = 0;
             }
             // the jobs with F = t complete (C = t + 1)
-            if (P.completion) {
-                #pragma unroll 1
-                for (int i = lane; i < end; i += 32)
-                    if (w.H[i].w == t) P.completion[base + w.C[i].y] = int64_t(t) + 1;
-            }
             // A job that ends before its projected last step changes W: its slot keeps E (in place of
             // W) and B, and F = -2 - t tells it from the slots freed at other steps.
             constexpr bool kEarly = POL == P_AMAX || POL == P_AELL;
@@ -945,29 +963,35 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             unsigned f = UINT_MAX, e1 = UINT_MAX;
             over_slots(half, end, [&](auto slots, int p) {
                 constexpr int N = decltype(slots)::value;
-                int4 a[N];
-#pragma unroll
-                for (int j = 0; j < N; ++j) a[j] = w.H[p + 32 * j + lane];
+                int e[N], bb[N], fj[N];
 #pragma unroll
                 for (int j = 0; j < N; ++j) {
-                    const bool done = a[j].w == t, early = kEarly && done && a[j].x > t;
-                    sm += done ? a[j].z + t : 0;
+                    fj[j] = w.F[p + 32 * j + lane];
+                    bb[j] = w.B[p + 32 * j + lane];
+                    if (kEarly) e[j] = w.EW[p + 32 * j + lane].x;
+                }
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const int i = p + 32 * j + lane;
+                    const bool done = fj[j] == t;
+                    sm += done ? bb[j] + t : 0;
                     c += done ? 1 : 0;
-                    f = min(f, done ? UINT_MAX : unsigned(a[j].w));
-                    if (POL == P_AELL) e1 = min(e1, done ? UINT_MAX : unsigned(a[j].x));
+                    f = min(f, done ? UINT_MAX : unsigned(fj[j]));
                     if (kEarly) {
+                        const bool early = done && e[j] > t;
+                        if (POL == P_AELL) e1 = min(e1, done ? UINT_MAX : unsigned(e[j]));
                         ne += early ? 1 : 0;
-                        ek = early ? a[j].x : ek;
-                        bk = early ? a[j].z : bk;
-                    }
-                    if (kEarly) {
-                        a[j] = make_int4(-1, a[j].x, a[j].z, -2 - t);
-                        if (done) w.H[p + 32 * j + lane] = a[j];  // nothing else in the branch: one predicated store
+                        ek = early ? e[j] : ek;
+                        bk = early ? bb[j] : bk;
+                        if (done) w.EW[i] = make_int2(-1, e[j]);
                     } else if (done) {
-                        w.H[p + 32 * j + lane].x = -1;
-                        w.H[p + 32 * j + lane].w = -1;
-                        if (POL == P_AMIN) w.K[p + 32 * j + lane] = UINT_MAX;
+                        w.EW[i].x = -1;
                     }
+                    if (done) w.F[i] = kEarly ? -2 - t : -1;
+                    if (POL == P_AMIN)
+                        if (done) w.K[i] = UINT_MAX;
+                    if (P.completion)
+                        if (done) P.completion[base + w.C[i].y] = int64_t(t) + 1;
                 }
             });
             c = int(__reduce_add_sync(FULL, unsigned(c)));
@@ -994,13 +1018,13 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 } else if (most > 1) {
                     #pragma unroll 1
                     for (int b = 0; b < end; b += 32) {
-                        const int4 x = w.H[b + lane];
-                        unsigned m = __ballot_sync(FULL, x.w == -2 - t && x.y > t);
+                        const int xe = w.EW[b + lane].y, xb = w.B[b + lane];
+                        unsigned m = __ballot_sync(FULL, w.F[b + lane] == -2 - t && xe > t);
                         #pragma unroll 1
                         while (m) {
                             const int src = __ffs(m) - 1;
                             m &= m - 1;
-                            subtract_job(w, end, __shfl_sync(FULL, x.y, src), __shfl_sync(FULL, x.z, src));
+                            subtract_job(w, end, __shfl_sync(FULL, xe, src), __shfl_sync(FULL, xb, src));
                         }
                     }
                 }
