@@ -106,19 +106,6 @@ __device__ __forceinline__ int quotient_lb(int a, int b) {
 
 __device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
-// Projected length of a queue entry.  For A_max, A_min and H-SF the sort key is that length; A_r
-// projects the true length o and A_ell the current estimate (l before a promotion, u after:
-// promotions have odd keys).
-template <int POL>
-__device__ __forceinline__ int proj_len(const RunParams &P, int64_t base, const QEnt &e) {
-    if (POL == P_AR) return e.o;
-    if (POL == P_AELL) {
-        const int2 lu = __ldg(P.lu + base + e.idx);
-        return (e.key & 1) ? lu.y : lu.x;
-    }
-    return e.key;
-}
-
 // ---------------------------------------------------------------------------------------------
 // Per-warp workspace (layout: ws_bytes in sim_internal.h)
 // ---------------------------------------------------------------------------------------------
@@ -178,6 +165,10 @@ __device__ __forceinline__ int tie_position(const unsigned *K, const int2 *C, in
 // cached in the workspace) plus a small sorted delta array (descending, so the head is the last
 // entry).  Together they hold R_t in (key, idx) order.  Inserts go to the delta; a full delta is
 // merged into the main array.
+// A_ell's queue is first in, first out: its main array is a run of the staged records that arrivals extend,
+// and in place of the delta stand the promotions, appended to the instance's merge buffer (a request is
+// promoted at most once) and read through a second cached run of kMc entries in the delta's space.  The
+// projected lengths (l of an arrival, u of a promotion) are fetched with the cached runs, into K.
 // ---------------------------------------------------------------------------------------------
 struct Queue {
     const QEnt *mq;  // main array (global, ascending): the staged records or a merge buffer
@@ -185,13 +176,16 @@ struct Queue {
     int lim;         // entries of mq that may be read (the cache reads ahead of me up to here)
     int mbuf;        // -1: mq is the staged records; 0/1: ping-pong buffer in use
     int dn;          // delta size
+    int dh, dce;     // A_ell: head of the promotions, end of their cached run (from dcb)
+    int dcb;
     int mcb;         // main cache base: w.mc[i] = mq[mcb + i] for i < kMc; -1 invalid
 };
 
 // Make w.mc cover mq[mh].  The staged records are constant, so a cached run of them stays valid
 // when later arrivals extend the main array.  gb counts the global-memory bytes the queue moves (a
-// work counter of the instrumented kernel; a dead variable otherwise).
-__device__ __forceinline__ void main_cache_at_head(const Ws &w, Queue &q, int64_t &gb) {
+// work counter of the instrumented kernel; a dead variable otherwise).  lu: A_ell's (l, u) table.
+template <int POL>
+__device__ __forceinline__ void main_cache_at_head(const Ws &w, Queue &q, const int2 *lu, int64_t &gb) {
     if (q.mcb >= 0 && unsigned(q.mh - q.mcb) < unsigned(kMc)) return;
     const int lane = lane_id();
     gb += int64_t(min(kMc, q.lim - q.mh)) * int64_t(sizeof(QEnt));
@@ -202,8 +196,30 @@ __device__ __forceinline__ void main_cache_at_head(const Ws &w, Queue &q, int64_
     __syncwarp();
     if (i0 < q.lim) w.mc[lane] = a;
     if (i1 < q.lim) w.mc[32 + lane] = b;
+    if (POL == P_AELL) {
+        if (i0 < q.lim) w.K[lane] = unsigned(lu[a.idx].x);
+        if (i1 < q.lim) w.K[32 + lane] = unsigned(lu[b.idx].x);
+    }
     __syncwarp();
     q.mcb = q.mh;
+}
+
+// A_ell: make w.dq cover the head of the promotions `pl`, which must not be empty.
+__device__ __forceinline__ void promo_cache_at_head(const Ws &w, Queue &q, const QEnt *pl, const int2 *lu, int64_t &gb) {
+    if (q.dh < q.dce) return;
+    const int lane = lane_id();
+    const int m = min(q.dn, kMc);
+    gb += int64_t(m) * int64_t(sizeof(QEnt));
+    __syncwarp();
+    #pragma unroll 1
+    for (int i = lane; i < m; i += 32) {
+        const QEnt e = pl[q.dh + i];
+        w.dq[i] = e;
+        w.K[kMc + i] = unsigned(lu[e.idx].y);
+    }
+    __syncwarp();
+    q.dcb = q.dh;
+    q.dce = q.dh + m;
 }
 
 // Merge the delta into the main array (into the other ping-pong buffer).  Rare (a full delta, or
@@ -338,13 +354,17 @@ __device__ __forceinline__ void delta_insert(const RunParams &P, const Ws &w, Qu
     delta_put(w, q, e);
 }
 
-// Head of R_t (smallest (key, idx)) and which part holds it (src 0: main, 1: delta), or the kNoHead entry
-// if R_t is empty.  The main cache must cover q.mh.  No branches: both parts are read at a clamped
-// position and an absent one is replaced by the kNoHead entry.
-__device__ __forceinline__ QEnt queue_head(const Ws &w, const Queue &q, int &src) {
+// Head of R_t (smallest (key, idx)), its projected length and which part holds it (src 0: main, 1: delta),
+// or the kNoHead entry if R_t is empty.  The main cache must cover q.mh (A_ell: and w.dq q.dh).  No
+// branches: both parts are read at a clamped position and an absent one is replaced by the kNoHead
+// entry.  For A_max, A_min and H-SF the sort key is the projected length; A_r projects the true length.
+template <int POL>
+__device__ __forceinline__ QEnt queue_head(const Ws &w, const Queue &q, int &src, int &len) {
     const bool have_m = q.mh < q.me, have_d = q.dn > 0;
-    QEnt hm = w.mc[have_m ? (q.mh - q.mcb) & (kMc - 1) : 0];
-    QEnt hd = w.dq[have_d ? q.dn - 1 : 0];
+    const int im = have_m ? (q.mh - q.mcb) & (kMc - 1) : 0;
+    const int id = POL == P_AELL ? (q.dh - q.dcb) & (kMc - 1) : (have_d ? q.dn - 1 : 0);
+    QEnt hm = w.mc[im];
+    QEnt hd = w.dq[id];
     if (!have_m) {
         hm.key = hm.idx = INT_MAX;
         hm.s = kNoHead;
@@ -354,12 +374,14 @@ __device__ __forceinline__ QEnt queue_head(const Ws &w, const Queue &q, int &src
         hd.s = kNoHead;
     }
     src = qless(hd, hm) ? 1 : 0;
-    return src ? hd : hm;
+    const QEnt h = src ? hd : hm;
+    len = POL == P_AELL ? int(w.K[src ? kMc + id : im]) : POL == P_AR ? h.o : h.key;
+    return h;
 }
 
 // Arrival batch: the staged records [ap, ae), an ascending run.  It becomes the main array if that
-// is empty and extends it under A_ell when it follows it in the staged records (FIFO keys); a few
-// entries go into the delta one by one; a long batch is copied into the emptied delta in chunks.
+// is empty and extends it under A_ell (FIFO keys, and it follows it in the staged records); a few entries
+// go into the delta one by one; a long batch is copied into the emptied delta in chunks.
 template <int POL>
 __device__ __forceinline__ void insert_run(const RunParams &P, const Ws &w, Queue &q, int64_t base, int n, int ap,
                                            int ae, int64_t &gb, int64_t *gbp) {
@@ -367,6 +389,10 @@ __device__ __forceinline__ void insert_run(const RunParams &P, const Ws &w, Queu
     const int lane = lane_id();
     const int len = ae - ap;
     gb += int64_t(len) * int64_t(sizeof(QEnt));
+    if (POL == P_AELL) {
+        q.me = ae;
+        return;
+    }
     if (q.mh >= q.me) {
         if (q.mbuf != -1) {
             q.mq = rec;
@@ -375,10 +401,6 @@ __device__ __forceinline__ void insert_run(const RunParams &P, const Ws &w, Queu
             q.mcb = -1;
         }
         q.mh = ap;
-        q.me = ae;
-        return;
-    }
-    if (POL == P_AELL && q.mbuf == -1 && q.me == ap) {
         q.me = ae;
         return;
     }
@@ -503,8 +525,8 @@ __device__ __forceinline__ void compact(const Ws &w, int &end) {
 // Invariants of the simulation state between events (SIM_OPT_DEBUG_CHECKS; global-memory kernel
 // only): the live slots number A and sum to need; nextF is their smallest F; W is the projected memory
 // plus E at every endpoint not yet passed (with the pending updates); under A_max, H-SF and A_r no job runs
-// past its projected last step; free slots are free; the delta queue is strictly descending and the
-// cached head of the main array ascending.  Returns false on the first violation.
+// past its projected last step; free slots are free; the delta queue is strictly descending (A_ell: the
+// cached promotions ascending) and the cached head of the main array ascending.  Returns false on the first violation.
 template <int POL>
 __device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int need, int nextF, int py, int pc,
                          int qy, int qc, int filled) {
@@ -534,8 +556,12 @@ __device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int
     }
     if (int(__reduce_add_sync(FULL, unsigned(cnt))) != A || int(__reduce_add_sync(FULL, unsigned(sum))) != need) bad = true;
     #pragma unroll 1
-    for (int i = lane; i + 1 < q.dn; i += 32)
+    for (int i = lane; POL != P_AELL && i + 1 < q.dn; i += 32)
         if (!qless(w.dq[i + 1], w.dq[i])) bad = true;
+    if (POL == P_AELL)
+        #pragma unroll 1
+        for (int i = q.dh - q.dcb + lane; i + 1 < q.dce - q.dcb; i += 32)
+            if (!qless(w.dq[i], w.dq[i + 1])) bad = true;
     if (q.mcb >= 0)
         #pragma unroll 1
         for (int i = q.mh + lane; i + 1 < min(q.me, q.mcb + kMc); i += 32)
@@ -580,7 +606,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
     q.mh = q.me = 0;
     q.lim = n;
     q.mbuf = -1;
-    q.dn = 0;
+    q.dn = q.dh = q.dce = q.dcb = 0;
     q.mcb = -1;
     // global-memory bytes moved by the queue (instrumented kernel); the merge adds through gbp
     int64_t gbq = 0;
@@ -634,11 +660,8 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
     enum { HEAD = 1, NEXTF = 2, SLOTS = 4, IDLE = 8, MERGE = 16 };
     int attn = 0;
 
-    const auto load_head = [&](bool cached) {  // cached: w.mc covers q.mh (else h is reloaded before use)
-        h = queue_head(w, q, hsrc);
-        hL = h.key;
-        if (POL == P_AR || POL == P_AELL) hL = cached && h.s != kNoHead ? proj_len<POL>(P, base, h) : 1;
-    };
+    const auto promotions = [&]() { return P.mainbuf + 2 * (P.main_cap > 0 ? warp_slot() * P.main_cap : base); };
+    const auto load_head = [&]() { h = queue_head<POL>(w, q, hsrc, hL); };
 
     // The conditions of all warp-uniform branches below are warp reductions: the compiler then knows
     // that they are uniform and emits plain jumps (about 12 cycles) instead of reconvergence blocks
@@ -719,53 +742,72 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 if (ap < n) prefetch_l1(P.rec + base + min(ap + 8, n - 1));  // a line ahead of the next arrivals
             }
             // ---- A_ell: jobs that used up their estimate unfinished (E < t) leave the batch and
-            // re-enter the queue at its end with the estimate u (the delta orders their equal keys by
-            // index)
+            // re-enter the queue at its end, in index order, with the estimate u
             if (POL == P_AELL && unsigned(t) > nextE) {
                 if (t > kAellMaxStep) {
                     status = ST_STEPCAP;
                     break;
                 }
-                unsigned f = UINT_MAX, e1 = UINT_MAX;
+                // their indices, in the space of K behind the cached lengths (or, for sets that do not
+                // fit there, in the instance's second merge buffer), give each its place
+                QEnt *pl = promotions() + q.dh + q.dn;
+                int *ids = A <= w.ca - 2 * kMc
+                               ? reinterpret_cast<int *>(w.K) + 2 * kMc
+                               : reinterpret_cast<int *>(promotions() + (P.main_cap > 0 ? P.main_cap : int64_t(n)));
+                int cnt = 0;
                 #pragma unroll 1
                 for (int b = 0; b < end; b += 32) {
-                    const unsigned ei = unsigned(w.EW[b + lane].x), fi = unsigned(w.F[b + lane]);
-                    const bool out = ei < unsigned(t);
-                    if (!out) {
+                    const bool out = unsigned(w.EW[b + lane].x) < unsigned(t);
+                    const unsigned m = __ballot_sync(FULL, out);
+                    if (out) ids[cnt + __popc(m & ((1u << lane) - 1u))] = w.C[b + lane].y;
+                    cnt += __popc(m);
+                }
+                __syncwarp();
+                unsigned f = UINT_MAX, e1 = UINT_MAX;
+                int sm = 0;
+                #pragma unroll 1
+                for (int b = 0; b < end; b += 32) {
+                    const int i = b + lane;
+                    const unsigned ei = unsigned(w.EW[i].x), fi = unsigned(w.F[i]);
+                    if (ei >= unsigned(t)) {
                         f = min(f, fi);
                         e1 = min(e1, ei);
-                    }
-                    unsigned m = __ballot_sync(FULL, out);
-                    #pragma unroll 1
-                    while (m) {
-                        const int pos = b + __ffs(m) - 1;
-                        m &= m - 1;
-                        const int bj = w.B[pos], fj = w.F[pos];
-                        const int2 pi = w.C[pos];
-                        __syncwarp();
-                        free_slot<POL>(w, pos);
-                        __syncwarp();
+                    } else {
+                        const int2 pi = w.C[i];
+                        int place = 0;
+                        #pragma unroll 1
+                        for (int k = 0; k < cnt; ++k) place += ids[k] < pi.y ? 1 : 0;
                         QEnt e;
                         e.key = 2 * t + 1;
                         e.idx = pi.y;
-                        e.s = bj + pi.x - 1;
-                        e.o = fj - pi.x + 1;
-                        need -= bj + t;
-                        --A;
-                        ++nev;
-                        if (INS) ++ev_step;
-                        delta_insert(P, w, q, e, base, n, gbp);
+                        e.s = w.B[i] + pi.x - 1;
+                        e.o = int(fi) - pi.x + 1;
+                        pl[place] = e;
+                        sm += w.B[i] + t;
+                        free_slot<POL>(w, i);
                     }
+                }
+                __syncwarp();
+                __threadfence_block();
+                need -= int(__reduce_add_sync(FULL, unsigned(sm)));
+                A -= cnt;
+                nev += cnt;
+                q.dn += cnt;
+                if (INS) {
+                    ev_step += cnt;
+                    gbq += int64_t(cnt) * int64_t(sizeof(QEnt));
                 }
                 nextF = __reduce_min_sync(FULL, f);
                 nextE = __reduce_min_sync(FULL, e1);
                 dirty = true;
                 fit_lb = 0;
+                if (end - A >= max(16, A >> 3) && slot_pages(end) > slot_pages(A)) attn |= SLOTS;
             }
             if (dirty) {
                 const int hi = h.idx, hk = h.key;
-                if (q.mh < q.me) main_cache_at_head(w, q, gbq);
-                load_head(true);
+                if (q.mh < q.me) main_cache_at_head<POL>(w, q, P.lu + base, gbq);
+                if (POL == P_AELL && q.dn > 0) promo_cache_at_head(w, q, promotions(), P.lu + base, gbq);
+                load_head();
                 if (h.idx != hi || h.key != hk) fit_lb = 0;
             }
             if (A == 0 && h.s == kNoHead) {
@@ -933,11 +975,12 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 if (INS) ++k_step;
                 if (bt) bpf += h.s;  // prefill: the prompts of the admitted requests
                 q.dn -= hsrc;
+                if (POL == P_AELL) q.dh += hsrc;
                 q.mh += 1 - hsrc;
-                const bool miss = q.mh < q.me && unsigned(q.mh - q.mcb) >= unsigned(kMc);
-                if (miss) attn |= HEAD;
+                if (q.mh < q.me && unsigned(q.mh - q.mcb) >= unsigned(kMc)) attn |= HEAD;  // reloaded before use
+                if (POL == P_AELL && q.dn > 0 && q.dh >= q.dce) attn |= HEAD;
                 if (end == kHalf || (end & (kPage - 1)) == 0) attn |= SLOTS;
-                load_head(!miss);
+                load_head();
                 fit_lb = 0;
                 __syncwarp();
                 continue;

@@ -107,3 +107,24 @@ def test_sweep_instances_match_oracle(experiment):
     for pol in (0, 1, 2, 4):
         got, _ = gpu_run(pol, w)
         assert_same(got, oracle_run(pol, w), tag=f"{experiment} pol={pol}")
+
+
+@pytest.mark.parametrize("cap", [0, 128])
+def test_aell_promotions_in_bulk(cap):
+    """A_ell's promotions are a first-in-first-out list with its own cached run: hundreds promoted in one
+    step (equal l, started together), more of them than the shared-memory index list holds, arrivals in
+    between, runs longer than the cached one, and single promotions."""
+    from paper_2508_14544_gb300 import workloads as W
+    rng = np.random.default_rng(29)
+    parts = []
+    for k, (n, l, u, rate) in enumerate([(900, 3, 9, 0), (2000, 1, 4, 0), (1500, 5, 6, 2), (70, 2, 30, 0), (3000, 2, 5, 9)]):
+        o = np.where(rng.random(n) < 0.7, u, l) if k < 3 else rng.integers(l, u + 1, n)
+        a = np.zeros(n, np.int64) if rate == 0 else np.sort(rng.integers(0, n // rate, n))
+        parts.append(dict(a=a, s=rng.integers(1, 3, n), l=np.full(n, l), u=np.full(n, u), o=o))
+    w = W.concat_instances("promote", 2500, parts)
+    opts = {"smem_active_cap": cap} if cap else {}
+    for extra in ({}, {"debug_checks": 1}, {"batch_time": 1}):
+        got, comp = gpu_run(4, w, completions=True, **opts, **extra)
+        ref, rcomp = oracle_run(4, w, completions=True)
+        assert_same(got, ref, tag=f"promote cap={cap} {extra}")
+        assert np.array_equal(comp, rcomp)
