@@ -73,9 +73,15 @@ struct sim_ctx {
     double *d_btout = nullptr;           // 2 per instance
     bool bt_valid = false;
     cudaStream_t load_stream = nullptr;  // non-blocking stream of sim_load (independent of other threads' work)
-    int64_t *h_off = nullptr;            // pinned copy of the offsets (n_inst + 1) for their upload
+    int64_t *h_off = nullptr;            // pinned block: the offsets (n_inst + 1) for their upload, results, inputs
     int64_t launches = 0;
-    std::vector<DevResult> h_res;
+    DevResult *h_res = nullptr;          // results of the last run: behind the offsets, or h_res_big's
+    std::vector<DevResult> h_res_big;
+    unsigned char *h_in = nullptr;       // pinned copy of small host inputs (h_in_bytes, from the first such load)
+    size_t h_in_bytes = 0;
+    int n_sm = 0, smem_optin = 0;        // of the device (0: not asked yet)
+    int64_t occ_shape[5] = {-1, 0, 0, 0, 0};  // launch shape of occ_blocks (blocks per SM)
+    int occ_blocks = 1;
     std::string err;
 };
 
@@ -83,6 +89,13 @@ static_assert(sizeof(sim_result) == 56, "sim_result must be 56 bytes");
 static_assert(sizeof(DevResult) == sizeof(sim_result), "device result layout");
 
 namespace {
+
+// Host inputs of at most this many ints go through pinned memory and one copy instead of one pageable
+// copy per array (when they fit what the first load took); results of at most kPinnedResults instances
+// come back to pinned memory.  One instance of 50 requests, seeds + load + run from host arrays: 99 -> 90 us
+// with the launch set-up kept and no cursor to clear.
+constexpr int64_t kSmallInts = 1 << 15;
+constexpr int32_t kPinnedResults = 1 << 14;
 
 thread_local std::string g_create_err;
 
@@ -258,7 +271,37 @@ static int load_impl(sim_ctx *c, const int64_t *offsets, const int32_t *a, const
     const int nsrc = (c->policy == SIM_AR) ? 6 : 5;
     const int32_t *in[6];
     for (int k = 0; k < 6; ++k) in[k] = c->d_raw + size_t(k) * c->cap_total;
-    for (int k = 0; k < nsrc; ++k) {
+    bool small = !device_ptrs && nt > 0 && nsrc * nt <= kSmallInts;
+    // one pinned block: the offsets, the results (unless there are very many) and small inputs
+    if (!c->h_off) {
+        const size_t ob = (size_t(c->n_inst + 1) * sizeof(int64_t) + 255) & ~size_t(255);
+        const size_t rb = c->n_inst <= kPinnedResults ? (size_t(c->n_inst) * sizeof(DevResult) + 255) & ~size_t(255) : 0;
+        const size_t ib = small ? size_t(nsrc) * nt * sizeof(int32_t) : 0;
+        unsigned char *pin = nullptr;
+        if ((e = cudaMallocHost(&pin, ob + rb + ib)) != cudaSuccess) return cuda_fail(c, e, "sim_load: pinned buffer");
+        c->h_off = reinterpret_cast<int64_t *>(pin);
+        if (rb) {
+            c->h_res = reinterpret_cast<DevResult *>(pin + ob);
+        } else {
+            c->h_res_big.resize(size_t(c->n_inst));
+            c->h_res = c->h_res_big.data();
+        }
+        if (ib) {
+            c->h_in = pin + ob + rb;
+            c->h_in_bytes = ib;
+        }
+    }
+    if (small && c->h_in_bytes >= size_t(nsrc) * nt * sizeof(int32_t)) {
+        for (int k = 0; k < nsrc; ++k) {
+            std::memcpy(c->h_in + size_t(k) * nt * sizeof(int32_t), src[k], size_t(nt) * sizeof(int32_t));
+            in[k] = c->d_raw + size_t(k) * nt;
+        }
+        e = cudaMemcpyAsync(c->d_raw, c->h_in, size_t(nsrc) * nt * sizeof(int32_t), cudaMemcpyHostToDevice, ls);
+        if (e != cudaSuccess) return cuda_fail(c, e, "sim_load: copy of the input arrays");
+    } else {
+        small = false;
+    }
+    for (int k = 0; k < nsrc && !small; ++k) {
         if (nt == 0) break;
         if (device_ptrs) {
             in[k] = src[k];
@@ -267,10 +310,6 @@ static int load_impl(sim_ctx *c, const int64_t *offsets, const int32_t *a, const
         e = cudaMemcpyAsync(c->d_raw + size_t(k) * c->cap_total, src[k], size_t(nt) * sizeof(int32_t),
                             cudaMemcpyHostToDevice, ls);
         if (e != cudaSuccess) return cuda_fail(c, e, "sim_load: copy of the input arrays");
-    }
-    if (!c->h_off && (e = cudaMallocHost(&c->h_off, size_t(c->n_inst + 1) * sizeof(int64_t))) != cudaSuccess) {
-        c->h_off = nullptr;
-        return cuda_fail(c, e, "sim_load: pinned offsets buffer");
     }
     std::memcpy(c->h_off, offsets, size_t(c->n_inst + 1) * sizeof(int64_t));
     e = cudaMemcpyAsync(c->d_off, c->h_off, size_t(c->n_inst + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, ls);
@@ -332,9 +371,11 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
                       int warps_per_sm, bool dense = false) {
     cudaError_t e;
     int dev = c->device;
-    int n_sm = 0, smem_optin = 0;
-    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (!c->n_sm) {
+        cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&c->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    }
+    const int n_sm = c->n_sm, smem_optin = c->smem_optin;
     dense = dense && smem;
     // more instances than the default copy holds at once (12 warps per SM), none of which can outgrow
     // the dense copy's slots: its 16 warps per SM (8192 instances of 300 requests, A_min 11.5 -> 10.1 ms,
@@ -360,9 +401,14 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
         while (wpb > 1 && per_warp * wpb > size_t(smem_optin)) --wpb;
         if (per_warp * wpb > size_t(smem_optin)) return fail(c, SIM_E_INVAL, "workspace does not fit shared memory");
         smem_bytes = per_warp * wpb;
-        e = simgb::run_blocks_per_sm(c->policy, p, wpb, smem_bytes, &per_sm);
-        if (e != cudaSuccess) return cuda_fail(c, e, "sim_run: kernel set-up");
-        per_sm = std::max(per_sm, 1);
+        // the same launch shape needs no new set-up (the kernel copy follows from these)
+        const int64_t shape[5] = {wpb, int64_t(smem_bytes), p.wide, p.ca, p.work_count || p.batch_time};
+        if (!std::equal(shape, shape + 5, c->occ_shape)) {
+            e = simgb::run_blocks_per_sm(c->policy, p, wpb, smem_bytes, &c->occ_blocks);
+            if (e != cudaSuccess) return cuda_fail(c, e, "sim_run: kernel set-up");
+            std::copy(shape, shape + 5, c->occ_shape);
+        }
+        per_sm = std::max(c->occ_blocks, 1);
     }
     if (warps_per_sm > 0 && !dense) per_sm = std::max(1, std::min(per_sm, warps_per_sm / wpb));
     int64_t blocks = int64_t(n_sm) * per_sm;
@@ -407,7 +453,7 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
     p.gws_stride = int64_t(per_warp);
     p.mainbuf = c->d_main;
     p.main_cap = main_cap;
-    if ((e = cudaMemsetAsync(c->d_counter, 0, sizeof(int32_t), st)) != cudaSuccess)
+    if (n_work > slots && (e = cudaMemsetAsync(c->d_counter, 0, sizeof(int32_t), st)) != cudaSuccess)
         return cuda_fail(c, e, "cudaMemsetAsync");
     e = simgb::launch_run(c->policy, p, int(blocks), wpb, smem_bytes, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "sim_run: kernel launch");
@@ -428,8 +474,7 @@ static int simulate(sim_ctx *c, cudaStream_t st, int wps, bool dense, float *ms)
     }
     int rc = run_launch(c, st, nullptr, c->n_inst, !c->debug_checks, wps, dense);
     if (rc == SIM_OK) {
-        c->h_res.resize(size_t(c->n_inst));
-        e = cudaMemcpyAsync(c->h_res.data(), c->d_res, sizeof(DevResult) * size_t(c->n_inst), cudaMemcpyDeviceToHost,
+        e = cudaMemcpyAsync(c->h_res, c->d_res, sizeof(DevResult) * size_t(c->n_inst), cudaMemcpyDeviceToHost,
                             st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) rc = cuda_fail(c, e, "sim_run: simulation kernel");
@@ -444,8 +489,7 @@ static int simulate(sim_ctx *c, cudaStream_t st, int wps, bool dense, float *ms)
         if (e != cudaSuccess) rc = cuda_fail(c, e, "sim_run: work list");
         if (rc == SIM_OK) rc = run_launch(c, st, c->d_work, int32_t(redo.size()), false, c->warps_per_sm);
         if (rc == SIM_OK) {
-            e = cudaMemcpyAsync(c->h_res.data(), c->d_res, sizeof(DevResult) * size_t(c->n_inst),
-                                cudaMemcpyDeviceToHost, st);
+            e = cudaMemcpyAsync(c->h_res, c->d_res, sizeof(DevResult) * size_t(c->n_inst), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
             if (e != cudaSuccess) rc = cuda_fail(c, e, "sim_run: simulation kernel (global workspace)");
         }

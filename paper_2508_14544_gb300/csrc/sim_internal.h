@@ -63,7 +63,7 @@ struct RunParams {
     int32_t n_work;            // instances to run in this launch
     const int32_t *n_work_dev; // optional: their number on the device (the redo count of an earlier launch)
     const int32_t *work;       // instance ids (n_work)
-    int32_t *counter;          // work-queue cursor (zeroed before launch)
+    int32_t *counter;          // work-queue cursor (zeroed before a launch of more instances than warps)
     int32_t *redo;             // optional: ids of the instances that outgrew the capacity are listed here
     int32_t *redo_count;       // their number (zeroed before launch)
     const QEnt *rec;

@@ -1160,13 +1160,14 @@ __global__ void __launch_bounds__(WIDE ? 128 : 256, WIDE ? 3 : 2) k_run(RunParam
     else base = P.gws + warp_slot() * P.gws_stride;
     Ws w = carve_ws(base, ca, P.dcap);
     const int n_work = P.n_work_dev ? *P.n_work_dev : P.n_work;
-    for (;;) {
-        int k = 0;
-        if (lane == 0) k = atomicAdd(P.counter, 1);
-        k = __shfl_sync(FULL, k, 0);
-        if (k >= n_work) break;
+    // a warp's first instance is its slot's; the cursor hands out the rest, if there are any
+    const int n_slots = int(gridDim.x * (blockDim.x >> 5));
+    for (int k = int(warp_slot()); k < n_work;) {
         const int inst = P.work ? P.work[k] : k;
         sim_instance<POL, SMEM, INS>(P, w, inst);
+        if (n_work <= n_slots) break;
+        if (lane == 0) k = n_slots + atomicAdd(P.counter, 1);
+        k = __shfl_sync(FULL, k, 0);
     }
 }
 
@@ -1199,8 +1200,13 @@ KernelFn run_fn(int policy, const RunParams &p, int warps_per_block) {
 cudaError_t run_blocks_per_sm(int policy, const RunParams &p, int warps_per_block, size_t smem_bytes, int *blocks) {
     const KernelFn fn = run_fn(policy, p, warps_per_block);
     if (smem_bytes > 48 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem_bytes));
+        // to the device's limit, not to this launch's bytes: contexts with other launch shapes share the
+        // kernel, also from other threads
+        int dev = 0, most = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e != cudaSuccess) return e;
     }
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, (const void *)fn, 32 * warps_per_block, smem_bytes);
