@@ -99,16 +99,18 @@ enum {
                                        (0, the default: as many as shared memory allows).  Results
                                        do not depend on it. */
     SIM_OPT_DEBUG_CHECKS = 6,       /* 0/1: run every instance in the global-memory kernel and check
-                                       the simulation state's invariants between events (active set
-                                       sorted by projected end, suffix sums and prefix maxima of the
-                                       set, queue order; no job past its projected end under A_max,
-                                       H-SF and A_r).  A violation gives that instance SIM_E_STATE.
+                                       the simulation state's invariants between events (memory of
+                                       the coming step, projected memory at every endpoint, next
+                                       completion, queue order; no job past its projected end under
+                                       A_max, H-SF and A_r).  A violation gives that instance
+                                       SIM_E_STATE.
                                        Slower; results are otherwise identical. */
     SIM_OPT_TUNE_RESIDENCY = 7,     /* 0/1: on the first sim_run of a load shape (n_instances, total
                                        and largest instance size), time three residencies -- one
-                                       simulation warp per scheduler (4 per SM), the default (two),
-                                       and the dense configuration of SIM_OPT_DENSE_RESIDENCY
-                                       (three) -- each with its global-memory re-runs, and use the
+                                       simulation warp per scheduler (4 per SM), the default
+                                       (three), and the dense configuration of
+                                       SIM_OPT_DENSE_RESIDENCY
+                                       (four) -- each with its global-memory re-runs, and use the
                                        fastest for every later sim_run of that shape, across
                                        sim_load calls (default 0).  A launch is as long as its
                                        slowest instance: one warp per scheduler wins when a few
@@ -126,14 +128,16 @@ enum {
     SIM_OPT_BATCH_TIME = 10,        /* 0/1: record per instance the integer sums that give total
                                        latency and makespan in time units under a linear batch-time
                                        model (sim_batch_time, sim_get_batch_time_sums; default 0). */
-    SIM_OPT_DENSE_RESIDENCY = 11    /* 0/1: simulate with three blocks of four warps per SM (12
-                                       warps; a kernel copy limited to 170 registers a thread) and
-                                       384 active-set slots in shared memory per instance, instead
-                                       of two blocks and SIM_OPT_SMEM_ACTIVE_CAP slots (default 0).
-                                       Faster when there are many instances whose active sets stay
-                                       below 384 jobs; instances that need more are re-run in global
-                                       memory.  Not used with SIM_OPT_COUNT_WORK or
-                                       SIM_OPT_BATCH_TIME.  Results do not depend on it. */
+    SIM_OPT_DENSE_RESIDENCY = 11    /* 0/1: simulate with four blocks of four warps per SM (16 warps,
+                                       128 registers a thread) and 384 active-set slots in shared
+                                       memory per instance, instead of three blocks and
+                                       SIM_OPT_SMEM_ACTIVE_CAP slots (default 0).  Faster when there
+                                       are many instances whose active sets stay below 384 jobs;
+                                       instances that need more are re-run in global memory.  Used
+                                       without being asked when no instance has more than 384
+                                       requests and there are more than 12 instances per SM (unless
+                                       the block size, the residency or the slots were set).
+                                       Results do not depend on it. */
 };
 
 /*
@@ -227,7 +231,7 @@ int sim_set_tie_seeds(sim_ctx *ctx, const uint64_t *seeds);
  *   [2] sum_t (A'_t + k_t) * ceil(log2(Q_t + 1))     (endpoint evaluations of an admission that
  *                                                     binary-searches the largest feasible prefix)
  *   [3] bytes of global memory the waiting queue moved (arrival runs, head reloads, merges).
- * The simulator itself skips most of this work (quiet steps in closed form, incremental order);
+ * The simulator itself skips most of this work (quiet steps in closed form, incremental sums);
  * the counters measure the method, not the kernel.  Returns SIM_OK, SIM_E_INVAL, SIM_E_STATE
  * (counting was off for the last sim_run) or SIM_E_CUDA.
  */

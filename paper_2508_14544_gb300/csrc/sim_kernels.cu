@@ -458,6 +458,22 @@ __device__ __forceinline__ void subtract_job(const Ws &w, int end, int e, int b)
     }
 }
 
+// The same for two jobs in one pass (e = -2: none); W of free slots is not kept.
+__device__ __forceinline__ void subtract_two(const Ws &w, int end, int e0, int b0, int e1, int b1) {
+    const int most = max(e0, e1);
+    #pragma unroll 1
+    for (int p = 0; p < end; p += kPage) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int i = p + 32 * j + lane_id();
+            int2 ew = w.EW[i];
+            if (ew.x <= e0) ew.y -= b0 + ew.x;
+            if (ew.x <= e1) ew.y -= b1 + ew.x;
+            if (ew.x <= most) w.EW[i].y = ew.y;
+        }
+    }
+}
+
 template <int POL>
 __device__ __forceinline__ void free_slot(const Ws &w, int i) {
     w.EW[i].x = -1;
@@ -1067,23 +1083,38 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             nextF = __reduce_min_sync(FULL, f);
             if (POL == P_AELL) nextE = __reduce_min_sync(FULL, e1);
             if (kEarly) {
-                // the lanes that hold such a job (several on one lane: found again by their mark)
-                const int most = __reduce_max_sync(FULL, ne);
-                if (most == 1) {
+                // decided on reductions (uniform jumps); the first update is left pending if none is
+                const int most = __reduce_max_sync(FULL, ne), tot = int(__reduce_add_sync(FULL, unsigned(ne)));
+                const int e1st = __reduce_max_sync(FULL, ek), b1st = __reduce_max_sync(FULL, bk);
+                const bool free_q = __reduce_max_sync(FULL, qy) < 0;
+                if (tot == 1) {
+                    if (free_q) {
+                        qy = e1st;
+                        qc = b1st;
+                    } else {
+                        subtract_job(w, end, e1st, b1st);
+                    }
+                } else if (most == 1) {  // one such job on each of several lanes
                     unsigned m = __ballot_sync(FULL, ne > 0);
-                    if (qy < 0) {
+                    int k = 0;
+                    if (free_q) {
                         const int src = __ffs(m) - 1;
                         m &= m - 1;
                         qy = __shfl_sync(FULL, ek, src);
                         qc = __shfl_sync(FULL, bk, src);
+                        k = 1;
                     }
                     #pragma unroll 1
-                    while (m) {
-                        const int src = __ffs(m) - 1;
+                    for (; k < tot; k += 2) {
+                        const int s0 = __ffs(m) - 1;
                         m &= m - 1;
-                        subtract_job(w, end, __shfl_sync(FULL, ek, src), __shfl_sync(FULL, bk, src));
+                        const int s1 = __ffs(m) - 1;  // -1: no second one
+                        m &= m - 1;
+                        const int e2 = __shfl_sync(FULL, ek, s1 & 31);
+                        subtract_two(w, end, __shfl_sync(FULL, ek, s0), __shfl_sync(FULL, bk, s0), s1 < 0 ? -2 : e2,
+                                     __shfl_sync(FULL, bk, s1 & 31));
                     }
-                } else if (most > 1) {
+                } else if (most > 1) {  // several on one lane: found again by their mark
                     #pragma unroll 1
                     for (int b = 0; b < end; b += 32) {
                         const int xe = w.EW[b + lane].y, xb = w.B[b + lane];
