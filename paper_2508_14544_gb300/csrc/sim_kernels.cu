@@ -1,4 +1,4 @@
-// Simulation kernel of the batched scheduler simulator (sm_103a): k_run<policy, shared, instrumented, wide>.
+// Simulation kernel of the batched scheduler simulator (sm_103a): k_run<policy, shared, instrumented, wide, slots>.
 //
 // One warp simulates one instance at a time (persistent warps pull instance ids from a work
 // queue).  Each step follows the paper's algorithms:
@@ -26,7 +26,7 @@
 //   F = p + o - 1      true last step (completion at step F, C = F + 1)
 //   P = p, I = request index, K = the estimate (A_min cancellation key)
 // A free slot has E = F = -1 and K = 2^32 - 1, which no test below selects, so a pass over the set
-// reads whole blocks of 64 slots without bounds checks.  With V(x) = sum over E_j >= x of
+// reads whole half pages (64 slots) or pages (128) without bounds checks.  With V(x) = sum over E_j >= x of
 // (B_j + x) the projected memory of the set at step x (eq. Constraint restricted to S'), a
 // candidate (prompt s, estimate L) started at step t ends at y = t + L - 1 and fits iff
 //   (1) need + s + 1 <= M, need = sum of (B_j + t), the memory of the coming step,
@@ -34,18 +34,21 @@
 //       t <= E_i <= y,
 //   (3) V(y) + s + L <= M at its own last step.
 // Between endpoints V(x) grows, so these points decide every future step.  (2) and (3) are one pass
-// over the slots and three warp reductions.  A job (E, B) that joins or leaves adds or subtracts
-// B + E_i in W_i at every endpoint E_i <= E: that update is left pending and applied by the next pass that
-// tests a candidate, so an admission costs one pass, and a job that leaves at or after its E
-// (every H-SF, A_r and A_min completion, every A_ell promotion) changes no W at all.  There are no
-// sorted arrays, prefix sums or moves; freed slots are reclaimed by a compaction once they outnumber
-// half of the live ones.  A candidate that fails yields the first later step at which (2) and
-// (3) could hold with the set unchanged; the steps up to the next event (that step, a completion, an
-// arrival, an A_min overflow, an A_ell promotion) are processed in closed form.
+// over the slots and two warp reductions.  A job (E, B) that joins or leaves adds or subtracts
+// B + E_i in W_i at every endpoint E_i <= E: one such update of each kind is left pending and applied by
+// the next pass that reads the slots anyway (a candidate's test, A_min's scan for the smallest
+// estimate), so an admission costs one pass, and a job that leaves at or after its E (every H-SF, A_r
+// and A_min completion, every A_ell promotion) changes no W at all.  There are no sorted arrays, prefix
+// sums or moves; freed slots are reclaimed by a compaction when that saves a page.  A candidate that
+// fails yields the first later step at which (2) and (3) could hold with the set unchanged; the steps up
+// to the next event (that step, a completion, an arrival, an A_min overflow, an A_ell promotion) are
+// processed in closed form.
 //
 // What bounds it: every instance is a serial chain of events, each a few dependent warp operations
-// (a shared-memory round trip, three reductions, a decision), so the time of an event is latency and
-// the rate of a full launch is the number of resident warps over that latency.
+// (a shared-memory round trip, two reductions, a decision), so the time of an event is latency, and
+// with many instances the issue slots (64-68 % used at 16 warps per SM).  Against the set kept sorted with
+// suffix sums and prefix maxima: A_min on 40960 x 2000 248 -> 105 ms, A_max 50 -> 34, H-SF 38 -> 23;
+// A_min's slowest instance of 1024 x 1000 alone 14.8 -> 7.9 ms; A_max on 64 x 10^5 402 -> 145 ms.
 #include <climits>
 #include <cstdint>
 
@@ -96,12 +99,9 @@ __device__ __forceinline__ bool qless(const QEnt &a, const QEnt &b) {
 // off by less than one); a lower bound of it for larger a (there the estimate is off by less than 40).
 // About half the latency of the integer division.
 __device__ __forceinline__ int quotient_lb(int a, int b) {
-    int q = __float2int_rz(__fdividef(float(a), float(b)));
-    if (a >= (1 << 22)) return max(q - 40, 0);
+    const int q = __float2int_rz(__fdividef(float(a), float(b)));
     const int r = a - q * b;
-    if (r < 0) --q;
-    if (r >= b) ++q;
-    return q;
+    return a >= (1 << 22) ? max(q - 40, 0) : q + (r >= b ? 1 : 0) - (r < 0 ? 1 : 0);
 }
 
 __device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
@@ -145,8 +145,9 @@ __device__ __forceinline__ int tie_position(const unsigned *K, const int2 *C, in
                                             uint64_t base, int rnd) {
     unsigned br = UINT_MAX, bi = UINT_MAX;
     int bp = 0;
+    int b = first & ~31;
     #pragma unroll 1
-    for (int b = first & ~31; b <= last; b += 32) {
+    do {
         const int i = b + lane_id();
         const unsigned id = unsigned(C[i].y);
         const unsigned r = rnd ? tie_key(base, int(id)) : id;
@@ -154,7 +155,8 @@ __device__ __forceinline__ int tie_position(const unsigned *K, const int2 *C, in
         br = less ? r : br;
         bi = less ? id : bi;
         bp = less ? i : bp;
-    }
+        b += 32;
+    } while (b <= last);
     const unsigned mr = __reduce_min_sync(FULL, br);
     const unsigned mi = __reduce_min_sync(FULL, br == mr ? bi : UINT_MAX);
     return int(__reduce_min_sync(FULL, br == mr && bi == mi ? unsigned(bp) : UINT_MAX));
