@@ -27,9 +27,10 @@
 //               parts).  Every term is positive, so nothing cancels, and v' A v = sum_i (2 i - 1) S_i S'_i.
 //               A thread-block cluster works on one u, each thread on a run of consecutive i: sums of
 //               its run, a scan over the block and the cluster (one cluster barrier per step), then its
-//               run again.  The arrays stay in shared memory when they fit.  About 18 FP64 operations
-//               per index and step; FP64 rate and the serial steps (about 15) bound it.  u = 20,000:
-//               0.47 ms, 10^5: 1.4 ms, 2^20: 11.5 ms; 25 values up to 20,000: 0.56 ms.  (One warp per u,
+//               run again.  The arrays stay in shared memory when they fit.  12 FP64 operations per
+//               index and step (constants from arrays); FP64 rate and the serial steps (about 15) bound it.  u = 20,000:
+//               0.37 ms, 10^5: 0.71 ms, 2^20: 4.8 ms; 25 values up to 20,000: 0.50 ms, half of it the call's
+//               allocation and copies.  (One warp per u,
 //               with four scans of totals minus prefixes, seven divisions per index and the tridiagonal
 //               B^{-1} applied to A v: 573 ms for the 25 values, relative error 2e-9 at u = 20,000 against
 //               4e-16 now.)
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(256) k_lemma(int32_t n_hist, int32_t len, int3
 }
 
 constexpr int kRhoThreads = 256;
-constexpr int kRhoArrays = 4;  // S, T, 1/(i(i-1)), 1/(8(2i-1)) per i
+constexpr int kRhoArrays = 7;  // per i: S, T, 1/(i(i-1)), 1/(8(2i-1)), w_i, 3 - 2/i, 2i - 1
 
 __global__ void __launch_bounds__(kRhoThreads) k_rho(const int32_t *__restrict__ us, double *__restrict__ out,
                                                       double *scratch, int64_t stride, int32_t max_iter) {
@@ -187,27 +188,32 @@ __global__ void __launch_bounds__(kRhoThreads) k_rho(const int32_t *__restrict__
     // arrays over the block's indices, in shared memory or in the scratch of this u
     double *S = scratch ? scratch + id * stride + int64_t(kRhoArrays) * lo : rho_smem;
     double *tv = S + (hi - lo), *rk = tv + (hi - lo), *bb = rk + (hi - lo);
+    double *ww = bb + (hi - lo), *cc = ww + (hi - lo), *dd = cc + (hi - lo);
     S -= lo;
     tv -= lo;
     rk -= lo;
     bb -= lo;
+    ww -= lo;
+    cc -= lo;
+    dd -= lo;
     for (int e = a; e < b; ++e) {
         const double i = double(e + 1);
         S[e] = double(u - e);
         rk[e] = e == 0 ? 0.0 : 1.0 / (i * (i - 1.0));
         bb[e] = 0.125 / (2.0 * i - 1.0);  // a quarter of 1 / (2 (2 i - 1)): S neither grows nor vanishes
+        ww[e] = fma(3.0 * i, i - 1.0, 1.0);
+        cc[e] = 3.0 - 2.0 / i;
+        dd[e] = 2.0 * i - 1.0;
     }
     double lam = 0.0, num = 0.0, den = 0.0;
     for (int it = 0; it <= max_iter; ++it) {
         // sums over this thread's run
         double p1 = 0.0, Q = 0.0, T = 0.0;
-        double im = double(a);  // i - 1
         for (int e = a; e < b; ++e) {
             const double v = S[e];
             p1 += v;
-            Q = fma(fma(3.0 * im, im + 1.0, 1.0), v, Q);
+            Q = fma(ww[e], v, Q);
             T = fma(rk[e], v, T);
-            im += 1.0;
         }
         // exclusive prefix of Q, suffix of T, and totals, over the warp, the block and the cluster
         double tq, tt;
@@ -254,17 +260,13 @@ __global__ void __launch_bounds__(kRhoThreads) k_rho(const int32_t *__restrict__
         }
         // the step, from its start
         num = den = 0.0;
-        im = double(a);
         for (int e = a; e < b; ++e) {
-            const double v = S[e], r = rk[e];
-            const double w = fma(3.0 * im, im + 1.0, 1.0);
-            const double c = e == 0 ? 1.0 : fma(-2.0 * im, r, 3.0);  // 3 - 2 / i
-            const double br = fma(w, tv[e], fma(r, q, fma(c, v, tot[0])));
+            const double v = S[e], w = ww[e];
+            const double br = fma(w, tv[e], fma(rk[e], q, fma(cc[e], v, tot[0])));
             num = fma(v, br, num);
-            den = fma(fma(2.0, im, 1.0) * v, v, den);
+            den = fma(dd[e] * v, v, den);
             q = fma(w, v, q);
             S[e] = bb[e] * br;
-            im += 1.0;
         }
     }
     if (rank == 0 && tid == 0) out[id] = lam;
@@ -306,32 +308,36 @@ cudaError_t launch_lemma(int32_t n_hist, int32_t len, int32_t l, double s, const
     return cudaGetLastError();
 }
 
-// Blocks per cluster: about 512 indices of the largest u each, at most 8 blocks.
-static int rho_cluster(int32_t u_max) {
+// Blocks per cluster: about 512 indices of the largest u each, at most 8 blocks, or 16 (which k_rho opts
+// in to) for a few values: a GPU partition holds few clusters of 16, and 25 values of up to 20,000 took
+// 0.79 ms with 16 blocks each, one of 10^5 0.70 ms (8 blocks: 1.0).
+static int rho_cluster(int32_t n_u, int32_t u_max) {
+    const int most = n_u <= 8 ? 16 : 8;
     int c = 1;
-    while (c < 8 && 512 * c < u_max) c <<= 1;
+    while (c < most && 512 * c < u_max) c <<= 1;
     return c;
 }
 
-static size_t rho_smem_bytes(int32_t u_max) {
-    const int c = rho_cluster(u_max);
+static size_t rho_smem_bytes(int32_t n_u, int32_t u_max) {
+    const int c = rho_cluster(n_u, u_max);
     return size_t((u_max + c - 1) / c) * kRhoArrays * sizeof(double);
 }
 
-int64_t rho_scratch_doubles(int32_t u_max) {
-    return rho_smem_bytes(u_max) <= size_t(200) * 1024 ? 0 : int64_t(kRhoArrays) * u_max;
+int64_t rho_scratch_doubles(int32_t n_u, int32_t u_max) {
+    return rho_smem_bytes(n_u, u_max) <= size_t(200) * 1024 ? 0 : int64_t(kRhoArrays) * u_max;
 }
 
 cudaError_t launch_rho(int32_t n_u, int32_t u_max, const int32_t *us, double *out, double *scratch, int32_t max_iter,
                        cudaStream_t st) {
     if (n_u <= 0) return cudaSuccess;
-    const int64_t stride = rho_scratch_doubles(u_max);
-    const size_t smem = stride ? 0 : rho_smem_bytes(u_max);
+    const size_t smem = scratch ? 0 : rho_smem_bytes(n_u, u_max);
+    const int64_t stride = int64_t(kRhoArrays) * u_max;
     cudaError_t e =
         cudaFuncSetAttribute((const void *)k_rho, cudaFuncAttributeMaxDynamicSharedMemorySize, int(size_t(200) * 1024));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute((const void *)k_rho, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    const int c = rho_cluster(u_max);
+    const int c = rho_cluster(n_u, u_max);
     cfg.gridDim = dim3(unsigned(n_u) * unsigned(c));
     cfg.blockDim = dim3(kRhoThreads);
     cfg.dynamicSmemBytes = smem;
@@ -342,7 +348,7 @@ cudaError_t launch_rho(int32_t n_u, int32_t u_max, const int32_t *us, double *ou
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_rho, us, out, stride ? scratch : static_cast<double *>(nullptr), stride, max_iter);
+    return cudaLaunchKernelEx(&cfg, k_rho, us, out, scratch, stride, max_iter);
 }
 
 }  // namespace simgb

@@ -769,7 +769,7 @@ int sim_cr_amin_rho(int32_t n_u, const int32_t *u_values, double *rho_out) {
         umax = std::max(umax, u_values[k]);
     }
     // batches of at most 1 GB of scratch, 2^20 values; one allocation: scratch, results, values
-    const int64_t stride = simgb::rho_scratch_doubles(umax);
+    const int64_t stride = simgb::rho_scratch_doubles(n_u, umax);
     const int64_t per_batch = stride ? std::max<int64_t>(1, (int64_t(1) << 30) / (stride * int64_t(sizeof(double)))) : 1 << 20;
     const int32_t nb = int32_t(std::min<int64_t>(per_batch, n_u));
     double *scratch = nullptr;
@@ -784,7 +784,7 @@ int sim_cr_amin_rho(int32_t n_u, const int32_t *u_values, double *rho_out) {
     for (int32_t b = 0; b < n_u && rc == SIM_OK; b += nb) {
         const int32_t m = std::min(nb, n_u - b);
         if ((e = cudaMemcpy(dus, u_values + b, size_t(m) * sizeof(int32_t), cudaMemcpyHostToDevice)) != cudaSuccess ||
-            (e = simgb::launch_rho(m, umax, dus, dout, scratch, 200, nullptr)) != cudaSuccess ||
+            (e = simgb::launch_rho(m, umax, dus, dout, stride ? scratch : nullptr, 200, nullptr)) != cudaSuccess ||
             (e = cudaMemcpy(rho_out + b, dout, size_t(m) * sizeof(double), cudaMemcpyDeviceToHost)) != cudaSuccess)
             rc = cuda_fail(nullptr, e, "sim_cr_amin_rho");
     }

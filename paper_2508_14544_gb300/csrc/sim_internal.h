@@ -117,8 +117,9 @@ cudaError_t launch_batch_time(const int64_t *sums, const DevResult *res, const d
                               cudaStream_t st);
 cudaError_t launch_lemma(int32_t n_hist, int32_t len, int32_t l, double s, const double *x, double *out,
                          cudaStream_t st);
-// Global scratch per value (doubles) that launch_rho needs when the largest value is u_max.
-int64_t rho_scratch_doubles(int32_t u_max);
+// Global scratch per value (doubles) that launch_rho needs for n_u values when the largest is u_max; 0: none,
+// and scratch must be null.
+int64_t rho_scratch_doubles(int32_t n_u, int32_t u_max);
 cudaError_t launch_rho(int32_t n_u, int32_t u_max, const int32_t *us, double *out, double *scratch, int32_t max_iter,
                        cudaStream_t st);
 

@@ -116,16 +116,19 @@ def test_lemma_shared_histograms(n, length):
 
 
 def test_rho_cluster_sizes_and_scratch():
-    """Values around the cluster sizes (512 indices per block), blocks without indices, and one above
-    the shared-memory limit (global scratch), alone and next to a larger one: the value does not
-    depend on the launch (sums in another order: 1e-13), and equals the dense eigensolver."""
+    """Values around the cluster sizes (512 indices per block, up to 8 blocks, 16 for a few values), blocks
+    without indices, and a largest value on both sides of the shared-memory limit (global scratch), alone
+    and next to each other: the value does not depend on the launch (sums in another order: 1e-13), and
+    equals the dense eigensolver."""
     from oracle import analytic as an
     from paper_2508_14544_gb300 import cr_amin_rho
-    us = [1, 2, 5, 511, 512, 513, 1024, 1025, 2049, 4097]
+    us = [1, 2, 5, 511, 512, 513, 1024, 1025, 2049, 4097, 8193]
     alone = np.array([cr_amin_rho([u])[0] for u in us])
-    for big in (5000, 51200, 51300):
+    for big in (9000, 29257, 29300):  # 8 blocks of 7 arrays hold 29257 indices in 200 KB each
         got = cr_amin_rho(us + [big])
         assert np.all(np.abs(got[:-1] - alone) <= 1e-13 * alone)
-        assert got[-1] > got[-2]
+        one = cr_amin_rho([big])[0]
+        assert got[-1] > got[-2] and abs(got[-1] - one) <= 1e-13 * one
+    assert abs(cr_amin_rho([58600])[0] - cr_amin_rho([58600] * 9)[4]) <= 1e-12  # scratch, 16 and 8 blocks
     for u, r in zip(us[:8], alone):
         assert abs(r - an.rho(u)) <= 1e-10 * r, u
