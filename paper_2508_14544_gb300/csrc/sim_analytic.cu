@@ -13,7 +13,7 @@
 //               pipes; otherwise each lane first sums its segment of lengths (four operations per
 //               length), the lanes' sums are scanned and each lane walks its segment with the sums of
 //               the segments above it.  2^20 histograms of 64 lengths take 0.97 ms (14 operations per
-//               length and a cancelling T - k S2 in place of G: 1.72 ms); 333 of 1999 lengths 0.05 ms
+//               length and a cancelling T - k S2 in place of G: 1.72 ms); 333 of 1999 lengths 0.044 ms
 //               (one lane each: 1.96 ms).  RMS error against 128-bit sums 1.0e-16 and 1.4e-16 (before:
 //               1.3e-16 and 1.1e-15).
 //   k_rho     - spectral radius of B_u^{-1} A_u (Corollary A/B; s = 0, l = 1), the bound on the
@@ -291,10 +291,11 @@ cudaError_t launch_lemma(int32_t n_hist, int32_t len, int32_t l, double s, const
     int T = 1;
     for (int c = 2; c <= 32 && c <= len; c <<= 1)
         if (cost(c) < cost(T)) T = c;
-    // blocks small enough that every SM gets one
+    // blocks of four warps (one per scheduler, which also share the table's divisions) unless larger ones
+    // still give every SM one: 333 histograms of 1999 lengths take 44 us with 128 threads, 50 with 64 and
+    // 66 with 256
     const int64_t lanes = int64_t(n_hist) * T;
-    int threads = 256;
-    while (threads > 64 && (lanes + threads - 1) / threads < n_sm) threads >>= 1;
+    const int threads = (lanes + 255) / 256 < n_sm ? 128 : 256;
     const unsigned blocks = unsigned((lanes + threads - 1) / threads);
     const size_t smem = size_t(3) * len * sizeof(double);
     using Fn = void (*)(int32_t, int32_t, int32_t, double, const double *, double *);
