@@ -42,13 +42,19 @@
 // sums or moves; freed slots are reclaimed by a compaction when that saves a page.  A candidate that
 // fails yields the first later step at which (2) and (3) could hold with the set unchanged; the steps up
 // to the next event (that step, a completion, an arrival, an A_min overflow, an A_ell promotion) are
-// processed in closed form.
+// processed in closed form.  It also leaves a witness (c, V(c)): the violated step that would last longest.
+// V(c) is carried along through admissions and completions (a job with E >= c counts B + c), and a head
+// with t <= c <= y, the same or another, cannot fit before V(c) + s + 1 + (c - t) <= M or c has passed: a
+// few instructions in place of most of the tests that fail after every change of the set.  A_max takes
+// 5-17 % less with it (64 x 10^5 online 145 -> 129 ms, load sweep 1.61 -> 1.34, a tenth of the alpha sweep
+// 4.43 -> 4.23), A_r 13 % (4.36 -> 3.80), A_ell 6 % (11.2 -> 10.5), H-SF 5-7 %, but 1 % more on 64 x 10^5
+// online.  A_min, whose tests follow cancellations and mostly admit, took 0-4 % longer: it keeps none.
 //
 // What bounds it: every instance is a serial chain of events, each a few dependent warp operations
 // (a shared-memory round trip, two reductions, a decision), so the time of an event is latency, and
 // with many instances the issue slots (64-68 % used at 16 warps per SM).  Against the set kept sorted with
 // suffix sums and prefix maxima: A_min on 40960 x 2000 248 -> 105 ms, A_max 50 -> 34, H-SF 38 -> 23;
-// A_min's slowest instance of 1024 x 1000 alone 14.8 -> 7.9 ms; A_max on 64 x 10^5 402 -> 145 ms.
+// A_min's slowest instance of 1024 x 1000 alone 14.8 -> 7.9 ms; A_max on 64 x 10^5 402 -> 129 ms.
 #include <climits>
 #include <cstdint>
 
@@ -540,15 +546,16 @@ __device__ __forceinline__ void compact(const Ws &w, int &end) {
 // Invariants of the simulation state between events (SIM_OPT_DEBUG_CHECKS; global-memory kernel
 // only): the live slots number A and sum to need; nextF is their smallest F; W is the projected memory
 // plus E at every endpoint not yet passed (with the pending updates); under A_max, H-SF and A_r no job runs
-// past its projected last step; free slots are free; the delta queue is strictly descending (A_ell: the
-// cached promotions ascending) and the cached head of the main array ascending.  Returns false on the first violation.
+// past its projected last step; a witness not yet passed has V(ct) = cv; free slots are free; the delta
+// queue is strictly descending (A_ell: the cached promotions ascending) and the cached head of the main
+// array ascending.  Returns false on the first violation.
 template <int POL>
 __device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int need, int nextF, int py, int pc,
-                         int qy, int qc, int filled) {
+                         int qy, int qc, int filled, int ct, int cv) {
     const int lane = lane_id();
     bool bad = false;
     unsigned fmin = UINT_MAX;
-    int cnt = 0, sum = 0;
+    int cnt = 0, sum = 0, vc = 0;
     #pragma unroll 1
     for (int i = lane; i < filled; i += 32) {
         const int4 h = make_int4(w.EW[i].x, w.EW[i].y, w.B[i], w.F[i]);
@@ -563,6 +570,7 @@ __device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int
         if ((POL == P_AMAX || POL == P_HSF || POL == P_AR) && h.w > h.x) bad = true;
         if (POL == P_AMIN && w.K[i] != unsigned(h.x - w.C[i].x + 1)) bad = true;
         if (h.x < t) continue;
+        if (h.x >= ct) vc += h.z + ct;
         int v = h.x;
         #pragma unroll 1
         for (int j = 0; j < end; ++j)
@@ -581,6 +589,8 @@ __device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int
         #pragma unroll 1
         for (int i = q.mh + lane; i + 1 < min(q.me, q.mcb + kMc); i += 32)
             if (i >= q.mcb && !qless(w.mc[i - q.mcb], w.mc[i + 1 - q.mcb])) bad = true;
+    vc = int(__reduce_add_sync(FULL, unsigned(vc)));
+    if (POL != P_AMIN && ct >= t && vc != cv) bad = true;
     fmin = __reduce_min_sync(FULL, fmin);
     if (A > 0 && fmin != unsigned(nextF)) bad = true;
     return __ballot_sync(FULL, bad) == 0;
@@ -671,6 +681,14 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
     h.s = kNoHead;
     h.o = 0;
     int hL = 1, hsrc = 0, fit_lb = 0;
+    // the witness: the step ct that kept the last head that failed out for longest, and cv = V(ct), kept up
+    // to date (see the top); no head whose own steps cover ct fits before bound()
+    constexpr bool kWit = POL != P_AMIN;
+    int ct = -1, cv = 0;
+    const auto bound = [&]() {  // (the sum may wrap when there is no head: (1) fails then)
+        if (!kWit) return 0;
+        return unsigned(ct - t) < unsigned(hL) ? min(int(unsigned(cv - M + h.s + 1) + unsigned(ct)), ct + 1) : 0;
+    };
     // what the next iteration has to look at first
     enum { HEAD = 1, NEXTF = 2, SLOTS = 4, IDLE = 8, MERGE = 16 };
     int attn = 0;
@@ -683,7 +701,8 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
     // (about 45, measured), and one reduction (29) decides several of them.  Single-value stores are
     // made by all lanes alike, for the same reason.
     for (;;) {
-        if (!SMEM && P.debug && attn == 0 && !state_ok<POL>(w, q, A, end, t, need, int(nextF), py, pc, qy, qc, filled)) {
+        if (!SMEM && P.debug && attn == 0 &&
+            !state_ok<POL>(w, q, A, end, t, need, int(nextF), py, pc, qy, qc, filled, ct, cv)) {
             status = ST_STATE;  // a consistency check of SIM_OPT_DEBUG_CHECKS failed
             break;
         }
@@ -815,7 +834,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 nextF = __reduce_min_sync(FULL, f);
                 nextE = __reduce_min_sync(FULL, e1);
                 dirty = true;
-                fit_lb = 0;
+                fit_lb = bound();
                 if (end - A >= max(16, A >> 3) && slot_pages(end) > slot_pages(A)) attn |= SLOTS;
             }
             if (dirty) {
@@ -823,7 +842,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 if (q.mh < q.me) main_cache_at_head<POL>(w, q, P.lu + base, gbq);
                 if (POL == P_AELL && q.dn > 0) promo_cache_at_head(w, q, promotions(), P.lu + base, gbq);
                 load_head();
-                if (h.idx != hi || h.key != hk) fit_lb = 0;
+                if (h.idx != hi || h.key != hk) fit_lb = bound();
             }
             if (A == 0 && h.s == kNoHead) {
                 if (ap >= n) {
@@ -927,12 +946,11 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
         }
         // ---- S4/S5: admit the largest feasible prefix of R_t, one candidate at a time ((1) holds)
         if (fl & 4u) {
-            // a candidate that fits is followed by the next one while nothing else needs a look
-            // A candidate that fits is followed by the next one while nothing else needs a look; A_max
-            // and A_ell, whose admissions are mostly single, go back to the top after each (with the
-            // inner loop the load sweep of A_max took 12 % longer, its online workloads 2-3 %; A_min takes
-            // 2-4 % less with it, H-SF 3 %).
-            constexpr bool kBurst = POL != P_AMAX && POL != P_AELL;
+            // A candidate that fits is followed by the next one while nothing else needs a look; A_max,
+            // whose admissions are mostly single, goes back to the top after each (with the inner loop
+            // the load sweep takes 11 % longer, the online workloads 2-3 %; A_min takes 2-4 % less with it,
+            // A_ell and H-SF 3 %).
+            constexpr bool kBurst = POL != P_AMAX;
             const int A0 = A;
             unsigned st = fl & 8u;  // A_min: fl after the last admission, so that the batch can follow
             bool more;
@@ -967,9 +985,12 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 if (d > 0) {
                     // A second pass finds the first later step that could fit: W_i > lim violates (2) at
                     // endpoint i until the overlap has shrunk (W_i <= lim + tau - t) or the endpoint has
-                    // passed, and (3) cannot hold before y has passed the next endpoint after it.  (In the
-                    // same pass as the test it cost more than it saved, also where half of the tests fail.)
-                    int r2 = 1;
+                    // passed, and (3) cannot hold before y has passed the next endpoint after it.  The witness
+                    // is the endpoint that makes it so late, else y (all endpoints at one step have the same
+                    // W; the endpoint with the largest W held heads out less: A_max +2 to +8 %; two witnesses
+                    // cost more than they save, +3 %).  (In the same pass as the test it cost more than it
+                    // saved, also where half of the tests fail.)
+                    int r2 = 1, we = y, ww = vy + y;
                     unsigned em = UINT_MAX;
                     over_slots(half, end, [&](auto slots, int p) {
                         constexpr int N = decltype(slots)::value;
@@ -977,11 +998,19 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                         for (int j = 0; j < N; ++j) {
                             const int2 ew = w.EW[p + 32 * j + lane];
                             em = min(em, unsigned(ew.x - y));
-                            if (unsigned(ew.x - t) < unsigned(hL)) r2 = max(r2, min(max(ew.y, lim) - lim, ew.x - t + 1));
+                            const int r = unsigned(ew.x - t) < unsigned(hL) ? min(max(ew.y, lim) - lim, ew.x - t + 1) : 0;
+                            if (kWit) we = r > r2 ? ew.x : we;
+                            if (kWit) ww = r > r2 ? ew.y : ww;
+                            r2 = max(r2, r);
                         }
                     });
                     em = __reduce_min_sync(FULL, em);
+                    const int r1 = r2;
                     r2 = __reduce_max_sync(FULL, r2);
+                    if (kWit) {
+                        ct = __reduce_max_sync(FULL, r1 == r2 ? we : -1);
+                        cv = __reduce_max_sync(FULL, r1 == r2 && we == ct ? ww : 0) - ct;
+                    }
                     if (vy + h.s + hL > M) r2 = max(r2, int(em) + 1);
                     more = false;
                     // no fit before step t + r2, and none at all if (1) fails there
@@ -996,6 +1025,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                     if (POL == P_AMIN) w.K[end] = unsigned(h.key);
                     py = y;
                     pc = h.s - t + 1;
+                    if (kWit) cv += y < ct ? 0 : pc + ct;
                     ++end;
                     ++A;
                     need += h.s + 1;
@@ -1010,7 +1040,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                     if (POL == P_AELL && q.dn > 0 && q.dh >= q.dce) attn |= HEAD;
                     if (end == kHalf || (end & (kPage - 1)) == 0) attn |= SLOTS;
                     load_head();
-                    fit_lb = 0;
+                    fit_lb = bound();
                     __syncwarp();
                     more = false;
                     if (POL == P_AMIN) {
@@ -1018,7 +1048,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                                                         (unsigned(t) == nextF ? 8u : 0u));
                         more = (st & 5u) == 4u;
                     } else if (kBurst) {
-                        more = __reduce_max_sync(FULL, attn == 0 && need + h.s < M && end != kHalf + 1);
+                        more = __reduce_max_sync(FULL, attn == 0 && t >= fit_lb && need + h.s < M && end != kHalf + 1);
                     }
                 }
             } while (more);
@@ -1045,7 +1075,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             // A job that ends before its projected last step changes W: its slot keeps E (in place of
             // W) and B, and F = -2 - t tells it from the slots freed at other steps.
             constexpr bool kEarly = POL == P_AMAX || POL == P_AELL;
-            int c = 0, sm = 0, ne = 0, ek = -1, bk = INT_MIN;
+            int c = 0, sm = 0, ne = 0, ek = -1, bk = INT_MIN, dv = 0;
             unsigned f = UINT_MAX, e1 = UINT_MAX;
             over_slots(half, end, [&](auto slots, int p) {
                 constexpr int N = decltype(slots)::value;
@@ -1067,6 +1097,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                         const bool early = done && e[j] > t;
                         if (POL == P_AELL) e1 = min(e1, done ? UINT_MAX : unsigned(e[j]));
                         ne += early ? 1 : 0;
+                        dv += early && e[j] >= ct ? bb[j] + ct : 0;
                         ek = early ? e[j] : ek;
                         bk = early ? bb[j] : bk;
                         if (done) w.EW[i] = make_int2(-1, e[j]);
@@ -1089,6 +1120,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 const int most = __reduce_max_sync(FULL, ne), tot = int(__reduce_add_sync(FULL, unsigned(ne)));
                 const int e1st = __reduce_max_sync(FULL, ek), b1st = __reduce_max_sync(FULL, bk);
                 const bool free_q = __reduce_max_sync(FULL, qy) < 0;
+                cv -= int(__reduce_add_sync(FULL, unsigned(dv)));
                 if (tot == 1) {
                     if (free_q) {
                         qy = e1st;
@@ -1142,7 +1174,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 bx3 += int64_t(c) * bpf;
             }
             ndone += c;
-            fit_lb = 0;
+            fit_lb = bound();
             if (A == 0) attn |= IDLE;
             if (end - A >= max(16, A >> 3) && slot_pages(end) > slot_pages(A)) attn |= SLOTS;
             if (ndone >= n) break;
@@ -1204,7 +1236,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
 
 // WIDE: up to 168 registers a thread (12 warps per SM), for launches whose time is one instance's serial
 // chain; otherwise 128 (16 warps per SM), for launches with more instances than that.  On the
-// 40960 x 2000 workload A_min takes 111 ms at 16 warps per SM and 133 at 12; the 256 x 10^4 online
+// 40960 x 2000 workload A_min takes 105 ms at 16 warps per SM and 131 at 12; the 256 x 10^4 online
 // workload 26.2 ms with 168 registers and 28.5 with 128 (spills).
 // CA: the slots per warp when fixed at compile time (the workspace arrays are then constant offsets from
 // one address: 2-5 % on every policy), or 0 for P.ca (the global-memory kernel and other capacities).
