@@ -53,7 +53,7 @@
 // What bounds it: every instance is a serial chain of events, each a few dependent warp operations
 // (a shared-memory round trip, two reductions, a decision), so the time of an event is latency, and
 // with many instances the issue slots (64-68 % used at 16 warps per SM).  Against the set kept sorted with
-// suffix sums and prefix maxima: A_min on 40960 x 2000 248 -> 105 ms, A_max 50 -> 34, H-SF 38 -> 23;
+// suffix sums and prefix maxima: A_min on 40960 x 2000 248 -> 105 ms, A_max 50 -> 33, H-SF 38 -> 22;
 // A_min's slowest instance of 1024 x 1000 alone 14.8 -> 7.9 ms; A_max on 64 x 10^5 402 -> 129 ms.
 #include <climits>
 #include <cstdint>
