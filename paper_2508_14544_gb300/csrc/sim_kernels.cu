@@ -737,6 +737,9 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 for (int i = lane; i < end; i += 32) f = min(f, unsigned(w.F[i]));
                 nextF = __reduce_min_sync(FULL, f);
             }
+            // (an admission that used up a cached run loaded the head from slots of the cache that hold no
+            // entry of the queue: whatever they were, the head and its bound are new)
+            const bool reload = (attn & HEAD) != 0;
             bool dirty = (attn & (HEAD | MERGE)) != 0;
             if (POL == P_AMIN && (attn & MERGE)) merge_delta(P, w, q, base, n, gbp);
             attn = 0;
@@ -842,7 +845,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 if (q.mh < q.me) main_cache_at_head<POL>(w, q, P.lu + base, gbq);
                 if (POL == P_AELL && q.dn > 0) promo_cache_at_head(w, q, promotions(), P.lu + base, gbq);
                 load_head();
-                if (h.idx != hi || h.key != hk) fit_lb = bound();
+                if (reload || h.idx != hi || h.key != hk) fit_lb = bound();
             }
             if (A == 0 && h.s == kNoHead) {
                 if (ap >= n) {

@@ -128,3 +128,24 @@ def test_aell_promotions_in_bulk(cap):
         ref, rcomp = oracle_run(4, w, completions=True)
         assert_same(got, ref, tag=f"promote cap={cap} {extra}")
         assert np.array_equal(comp, rcomp)
+
+
+def test_aell_head_after_the_last_cached_promotion():
+    """The admission of the last cached promotion leaves the workspace to a reload; what the warp's previous
+    instance left there must not stand for the next head.  Many small instances per warp, whose promotions
+    have few distinct steps and indices, so that leftovers with the next head's (key, index) but other lengths
+    are frequent; their order on the warps changes from run to run."""
+    from paper_2508_14544_gb300 import workloads as W
+    rng = np.random.default_rng(61)
+    parts = []
+    for _ in range(20000):
+        n = int(rng.integers(6, 25))
+        l = rng.integers(1, 3, n)
+        u = l + rng.integers(1, 30, n)
+        parts.append(dict(a=np.zeros(n, np.int64), s=rng.integers(1, 12, n), l=l, u=u, o=rng.integers(l, u + 1)))
+    w = W.concat_instances("leftovers", 60, parts)
+    ref, rcomp = oracle_run(4, w, completions=True)
+    for opts in ({}, {"warps_per_block": 1, "warps_per_sm": 1}, {}):
+        got, comp = gpu_run(4, w, completions=True, **opts)
+        assert_same(got, ref, tag=f"leftovers {opts}")
+        assert np.array_equal(comp, rcomp)
