@@ -134,7 +134,7 @@ enum {
                                        SIM_OPT_SMEM_ACTIVE_CAP slots (default 0).  Faster when there
                                        are many instances whose active sets stay below 384 jobs;
                                        instances that need more are re-run in global memory.  Used
-                                       without being asked when no instance has more than 384
+                                       without being asked when every instance has fewer than 384
                                        requests and there are more than 12 instances per SM (unless
                                        the block size, the residency or the slots were set).
                                        Results do not depend on it. */
@@ -302,7 +302,7 @@ int64_t sim_kernel_launches(const sim_ctx *ctx);
  *   results     DEVICE, n_instances sim_result, written by the kernels.
  *   cuda_stream a cudaStream_t or NULL.  The call only enqueues work: read `results` after
  *               synchronising the stream.  Per-instance statuses are in results[i].status.
- * Everything except the inputs and outputs lives in one fixed array of about 21 MB that every GPU
+ * Everything except the inputs and outputs lives in one fixed array of about 23 MB that every GPU
  * loading the library holds until the process exits.  Limits: at most 2048 requests per instance
  * and 262,144 requests per call; larger inputs are rejected with SIM_E_INVAL and a message in
  * sim_last_error(NULL).  The staging kernel checks the offsets it reads against the same limits

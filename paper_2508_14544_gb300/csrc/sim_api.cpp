@@ -365,7 +365,7 @@ int sim_load(sim_ctx *c, int32_t n, const int32_t *a, const int32_t *s, const in
 }
 
 // One launch of the simulation kernel over n_work instances (all, or the device list work_dev).
-// smem: the active sets in shared memory (else a global-memory workspace of n_max slots);
+// smem: the active sets in shared memory (else a global-memory workspace of more than n_max slots);
 // dense: kDenseCa shared-memory slots per warp, as many warps per SM as then fit.
 static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int32_t n_work, bool smem,
                       int warps_per_sm, bool dense = false) {
@@ -377,18 +377,17 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
     }
     const int n_sm = c->n_sm, smem_optin = c->smem_optin;
     dense = dense && smem;
-    // more instances than the default copy holds at once (12 warps per SM), none of which can outgrow
+    // more instances than the default copy holds at once (12 warps per SM), none of which can fill
     // the dense copy's slots: its 16 warps per SM (8192 instances of 300 requests, A_min 11.5 -> 10.1 ms,
     // A_max 1.42 -> 1.20; of 60 requests, A_min 1.73 -> 1.53)
     if (smem && !c->wpb_set && warps_per_sm == 0 && c->smem_ca == simgb::kSmemCaDefault &&
-        c->n_max <= simgb::kDenseCa && n_work > 12 * n_sm)
+        c->n_max < simgb::kDenseCa && n_work > 12 * n_sm)
         dense = true;
     int wpb = dense ? simgb::kDenseWarps : c->wpb;
     // no more instances than SMs: one warp per block, so that each instance gets an SM to itself
     if (!dense && !c->wpb_set && n_work <= n_sm) wpb = 1;
     simgb::RunParams p;
-    const int all = ((std::max(c->n_max, 128) + 127) / 128) * 128;
-    p.ca = smem ? (dense ? simgb::kDenseCa : c->smem_ca) : all;
+    p.ca = smem ? (dense ? simgb::kDenseCa : c->smem_ca) : simgb::ca_above(c->n_max);
     p.dcap = simgb::delta_cap(c->n_max);
     p.use_smem = smem ? 1 : 0;
     p.wide = dense ? 0 : 1;

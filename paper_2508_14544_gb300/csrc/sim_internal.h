@@ -77,7 +77,7 @@ struct RunParams {
                                // evaluations of the per-step method, global bytes moved by the queue
     int64_t *batch_time;       // optional, 6 per instance: the batch-time sums X0..X3, F2, F3
     // workspace
-    int32_t ca;                // active-set capacity per instance (multiple of 64)
+    int32_t ca;                // active-set capacity per instance (a multiple of kCaUnit)
     int32_t dcap;              // delta-queue capacity per warp slot (at most kDcap)
     int32_t use_smem;          // 1: active set + delta queue in shared memory; 0: global workspace
     int32_t wide;              // 1: the copy with more registers a thread and at most 12 warps per SM
@@ -88,6 +88,10 @@ struct RunParams {
     QEnt *mainbuf;             // ping-pong main-queue buffers, 2 * main_cap per warp slot
     int64_t main_cap;          // 0: two buffers of n entries per instance, at twice its first request
 };
+
+constexpr int kCaUnit = 128;       // active-set slots are passed over and allotted in pages of this many
+// Slots that no instance of n requests fills (one that fills the slots stops with kStatusCapacity).
+__host__ __device__ constexpr int ca_above(int64_t n) { return int(n / kCaUnit + 1) * kCaUnit; }
 
 constexpr int kDenseCa = 384;      // active-set slots per warp of the dense configuration
 constexpr int kDenseWarps = 4;     // warps per block of the dense configuration

@@ -69,7 +69,7 @@ enum { P_AMAX = 0, P_AMIN = 1, P_HSF = 2, P_AR = 3, P_AELL = 4 };
 enum { ST_OK = 0, ST_INVAL = -1, ST_STEPCAP = -3, ST_STATE = -5 };
 // Loops whose trip count is known only at run time carry `#pragma unroll 1`: unrolled copies grow
 // the simulation loop, which the warps of a scheduler share through its instruction cache.
-constexpr int kPage = 128;  // active-set slots per pass iteration (four per lane)
+constexpr int kPage = kCaUnit;  // active-set slots per pass iteration (four per lane)
 constexpr int kHalf = 64;   // sets whose slots end here are passed over in one half page (two per lane)
 // s of the entry that stands for the head of an empty queue: never fits, greater than every entry
 constexpr int kNoHead = 1 << 28;
@@ -719,8 +719,11 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 if (end - A >= max(16, A >> 3) || (end >= w.ca && A < end)) {
                     compact<POL>(w, end);
                 } else if (end >= w.ca) {
-                    status = kStatusCapacity;
-                    break;
+                    // a full set is no obstacle once every request has been admitted and none can return
+                    if (POL == P_AMIN || POL == P_AELL || ndone + A < n) {
+                        status = kStatusCapacity;
+                        break;
+                    }
                 } else if (end >= filled) {
                     free_page<POL>(w, filled);
                     filled += kPage;

@@ -46,8 +46,8 @@ constexpr int64_t kNaSlots = int64_t(kNaBlocks) * kNaWarpsPerBlock;  // warps of
 
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Workspace bytes per warp for an active-set capacity of kNaMaxPerInstance.
-constexpr size_t ws_bytes_max() { return simgb::ws_bytes(int(kNaMaxPerInstance), simgb::kDcap); }
+// Workspace bytes per warp for the largest instances.
+constexpr size_t ws_bytes_max() { return simgb::ws_bytes(simgb::ca_above(kNaMaxPerInstance), simgb::kDcap); }
 
 constexpr size_t kOffOff = 0;
 constexpr size_t kOffRec = align256(kOffOff + size_t(kNaMaxInstances + 1) * sizeof(int64_t));
@@ -57,7 +57,7 @@ constexpr size_t kOffCounter = align256(kOffInfo + size_t(kNaMaxInstances) * siz
 constexpr size_t kOffRedo = align256(kOffCounter + 256);
 constexpr size_t kOffMain = align256(kOffRedo + size_t(kNaMaxInstances) * sizeof(int32_t));
 constexpr size_t kOffWs = align256(kOffMain + size_t(kNaMaxTotal) * 2 * sizeof(simgb::QEnt));
-constexpr size_t kScratchBytes = align256(kOffWs + size_t(kNaSlots) * ws_bytes_max());  // about 21 MB
+constexpr size_t kScratchBytes = align256(kOffWs + size_t(kNaSlots) * ws_bytes_max());  // about 23 MB
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
@@ -171,7 +171,7 @@ extern "C" int sim_run_noalloc(int policy, int64_t M, int32_t n_instances, const
     // shared memory: one warp per block (no slots or buffers depend on the launch), every SM
     int n_sm = 0, per_sm = 1;
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    const int all = int(((std::max<int64_t>(n_max, 128) + 127) / 128) * 128);  // >= any active set
+    const int all = simgb::ca_above(n_max);  // more than any active set
     p.ca = simgb::kSmemCaDefault;
     p.dcap = simgb::delta_cap(n_max);
     p.use_smem = 1;

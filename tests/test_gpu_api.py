@@ -350,3 +350,20 @@ def test_step_counter_limit_is_a_step_cap():
     got, _ = gpu_run(4, late)
     assert got["status"].tolist() == [-3]
     del ref
+
+
+@pytest.mark.parametrize("pol", [0, 1, 2, 3, 4])
+@pytest.mark.parametrize("opts", [{}, {"smem_active_cap": 128}, {"dense_residency": 1}, {"debug_checks": 1}])
+def test_every_request_active_at_once(pol, opts):
+    """Sets that fill the active-set slots to the last one (128, 384, 512, 640 and 1024 requests that all fit
+    M and run at once), and one request fewer or more: alone (the slots follow from the instance) and next to
+    each other."""
+    rng = np.random.default_rng(12)
+    parts = []
+    for n in (1, 127, 128, 129, 383, 384, 385, 511, 512, 513, 640, 1024):
+        o = rng.integers(1, 40, n)
+        parts.append(dict(a=np.zeros(n, np.int64), s=rng.integers(1, 9, n), l=np.maximum(o // 2, 1), u=o + 3, o=o))
+    for sel in [[p] for p in parts] + [parts]:
+        w = _w(sel, 100_000)
+        got, _ = gpu_run(pol, w, **opts)
+        assert_same(got, oracle_run(pol, w), tag=f"full pol={pol} n={len(sel[0]['o'])} {opts}")

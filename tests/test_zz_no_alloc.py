@@ -152,3 +152,19 @@ def test_noalloc_more_instances_than_warps():
     w = W.concat_instances("many", 120, parts)
     out = torch.zeros(w.n_instances * L.RESULT_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
     _check(_noalloc(L.SIM_AMIN, w, _dev(w), out), _oracle(L.SIM_AMIN, w), "many")
+
+
+@pytest.mark.parametrize("pol", [0, 1, 2])
+def test_noalloc_every_request_active_at_once(pol):
+    """Sets that fill the shared-memory slots (512), or the array's (2048), to the last one."""
+    import torch
+
+    from paper_2508_14544_gb300 import workloads as W
+    from paper_2508_14544_gb300 import _lib as L
+    rng = np.random.default_rng(19)
+    for n in (128, 511, 512, 513, 2047, 2048):
+        o = rng.integers(1, 9, n)
+        w = W.concat_instances("full", 100_000, [dict(a=np.zeros(n, np.int64), s=np.ones(n, np.int64),
+                                                      l=np.maximum(o // 2, 1), u=o + 2, o=o)] * 3)
+        out = torch.zeros(w.n_instances * L.RESULT_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+        _check(_noalloc(pol, w, _dev(w), out), _oracle(pol, w), f"full pol={pol} n={n}")
