@@ -196,6 +196,32 @@ __device__ int32_t *radix_sort_idx(const int32_t *kk, const int32_t *ka, int32_t
     return in;
 }
 
+// An instance that is larger than the n_max the launch was made for: the offsets were read again, by the
+// replay of a captured call, after the caller changed them.  Every request counts those before it.
+__device__ __noinline__ void stage_by_counting(const StageParams &S, int inst, int64_t base, int n, int64_t *sh64) {
+    StageSums z = {0, 0, 0, 0, 0, 0};
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int64_t g = base + j;
+        stage_check(S, g, S.a[g], S.s[g], S.o[g], stage_key(S, g), z);
+    }
+    if (stage_finish(S, inst, base, n, z, sh64) != ST_OK) return;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int64_t g = base + j;
+        const int a = S.a[g];
+        QEnt e;
+        e.key = stage_key(S, g);
+        e.idx = j;
+        e.s = S.s[g];
+        e.o = S.o[g];
+        int place = 0;
+        for (int k = 0; k < n; ++k) {
+            const int ak = S.a[base + k], kk = stage_key(S, base + k);
+            place += ak < a || (ak == a && (kk < e.key || (kk == e.key && k < j))) ? 1 : 0;
+        }
+        S.rec[base + place] = e;
+        S.rec_a[base + place] = a;
+    }
+}
 
 __global__ void __launch_bounds__(kStageThreads) k_stage(StageParams S, int np) {
     __shared__ int64_t sh64[32];
@@ -208,7 +234,10 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageParams S, int np) 
     // instance before anything is written: it is staged as empty with status INVAL
     const bool oob = base < 0 || n64 < 0 || n64 > S.max_n || base + n64 > S.max_total;
     const int n = oob ? 0 : int(n64);
-    if (n > np) return;  // k_stage_large
+    if (n > np) {
+        if (S.n_max <= np) stage_by_counting(S, inst, base, n, sh64);
+        return;  // otherwise k_stage_large follows
+    }
     int32_t *kk = reinterpret_cast<int32_t *>(stage_smem);
     int32_t *ka = kk + np;
     int32_t *ss = ka + np;

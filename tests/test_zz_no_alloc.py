@@ -168,3 +168,53 @@ def test_noalloc_every_request_active_at_once(pol):
                                                       l=np.maximum(o // 2, 1), u=o + 2, o=o)] * 3)
         out = torch.zeros(w.n_instances * L.RESULT_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
         _check(_noalloc(pol, w, _dev(w), out), _oracle(pol, w), f"full pol={pol} n={n}")
+
+
+@pytest.mark.parametrize("pol", [0, 1, 2])
+def test_noalloc_captured_with_other_sizes(pol):
+    """A captured call copies the offsets again on every replay: instances that have grown past the sizes at
+    capture are staged all the same (their sets fit the slots), and those that reach past the arrays' limits
+    get SIM_E_INVAL."""
+    import torch
+
+    from paper_2508_14544_gb300 import workloads as W
+    from paper_2508_14544_gb300 import _lib as L
+    rng = np.random.default_rng(27)
+
+    def workload(sizes):
+        parts = []
+        for n in sizes:
+            o = rng.integers(1, 40, n)
+            l = rng.integers(1, o + 1)
+            parts.append(dict(a=rng.integers(0, 30, n), s=rng.integers(1, 9, n), l=l, u=o + 5, o=o))
+        return W.concat_instances("replay", 300, parts)
+
+    room, off = 8192, torch.zeros(5, dtype=torch.int64).pin_memory()
+    dev = [torch.zeros(room, dtype=torch.int32, device="cuda") for _ in range(5)]
+    out = torch.zeros(4 * L.RESULT_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+
+    def put(w):
+        off.numpy()[:] = w.offsets
+        for d, x in zip(dev, (w.arrival, w.prompt, w.lower, w.upper, w.true_o)):
+            d[: x.size].copy_(torch.from_numpy(np.ascontiguousarray(x)))
+
+    small = workload((10, 7, 0, 9))
+    put(small)
+    _check(_noalloc(pol, small, dev, out), _oracle(pol, small), "plain")
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=side):
+        rc = L.sim_run_noalloc(pol, small.M, off.numpy(), *dev, out, stream=side.cuda_stream)
+    assert rc == L.SIM_OK, L.sim_last_error(None)
+    for sizes in ((10, 7, 0, 9), (17, 300, 1, 16), (2048, 5, 33, 600)):
+        w = workload(sizes)
+        put(w)
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        got = out.cpu().numpy().view(L.RESULT_DTYPE).reshape(-1).copy()
+        _check(got, _oracle(pol, w), f"replay pol={pol} {sizes}")
+    off.numpy()[:] = [0, 10, 10 + 2049, 2060, 2070]
+    graph.replay()
+    torch.cuda.synchronize()
+    assert out.cpu().numpy().view(L.RESULT_DTYPE)["status"].reshape(-1)[1] == L.SIM_E_INVAL
