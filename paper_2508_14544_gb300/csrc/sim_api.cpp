@@ -73,10 +73,12 @@ struct sim_ctx {
     double *d_btout = nullptr;           // 2 per instance
     bool bt_valid = false;
     cudaStream_t load_stream = nullptr;  // non-blocking stream of sim_load (independent of other threads' work)
-    int64_t *h_off = nullptr;            // pinned block: the offsets (n_inst + 1) for their upload, results, inputs
+    int64_t *h_off = nullptr;            // pinned block: the offsets (n_inst + 1) for their upload, results, seeds, inputs
     int64_t launches = 0;
     DevResult *h_res = nullptr;          // results of the last run: behind the offsets, or h_res_big's
     std::vector<DevResult> h_res_big;
+    uint64_t *h_seed = nullptr;          // pinned copy of the tie seeds (A_min, up to kPinnedResults instances)
+    bool seeds_pending = false;          // their upload is in load_stream and has not been waited for
     unsigned char *h_in = nullptr;       // pinned copy of small host inputs (h_in_bytes, from the first such load)
     size_t h_in_bytes = 0;
     int n_sm = 0, smem_optin = 0;        // of the device (0: not asked yet)
@@ -138,6 +140,10 @@ int check_device(sim_ctx *c) {
                     c->device);
     c->device = dev;
     return SIM_OK;
+}
+
+cudaError_t make_load_stream(sim_ctx *c) {
+    return c->load_stream ? cudaSuccess : cudaStreamCreateWithFlags(&c->load_stream, cudaStreamNonBlocking);
 }
 
 }  // namespace
@@ -262,8 +268,7 @@ static int load_impl(sim_ctx *c, const int64_t *offsets, const int32_t *a, const
             return e == cudaErrorMemoryAllocation ? fail(c, SIM_E_NOMEM, "sim_load: device allocation failed")
                                                   : cuda_fail(c, e, "cudaMalloc");
     }
-    if (!c->load_stream && (e = cudaStreamCreateWithFlags(&c->load_stream, cudaStreamNonBlocking)) != cudaSuccess)
-        return cuda_fail(c, e, "sim_load: stream creation");
+    if ((e = make_load_stream(c)) != cudaSuccess) return cuda_fail(c, e, "sim_load: stream creation");
     const cudaStream_t ls = c->load_stream;
     // Device inputs are read in place by the staging kernel (sim_load returns only after it has
     // finished, so the caller may reuse them afterwards); host inputs are copied in first.
@@ -272,13 +277,14 @@ static int load_impl(sim_ctx *c, const int64_t *offsets, const int32_t *a, const
     const int32_t *in[6];
     for (int k = 0; k < 6; ++k) in[k] = c->d_raw + size_t(k) * c->cap_total;
     bool small = !device_ptrs && nt > 0 && nsrc * nt <= kSmallInts;
-    // one pinned block: the offsets, the results (unless there are very many) and small inputs
+    // one pinned block: the offsets, the results and seeds (unless there are very many) and small inputs
     if (!c->h_off) {
         const size_t ob = (size_t(c->n_inst + 1) * sizeof(int64_t) + 255) & ~size_t(255);
         const size_t rb = c->n_inst <= kPinnedResults ? (size_t(c->n_inst) * sizeof(DevResult) + 255) & ~size_t(255) : 0;
+        const size_t sb = c->policy == SIM_AMIN && rb ? (size_t(c->n_inst) * sizeof(uint64_t) + 255) & ~size_t(255) : 0;
         const size_t ib = small ? size_t(nsrc) * nt * sizeof(int32_t) : 0;
         unsigned char *pin = nullptr;
-        if ((e = cudaMallocHost(&pin, ob + rb + ib)) != cudaSuccess) return cuda_fail(c, e, "sim_load: pinned buffer");
+        if ((e = cudaMallocHost(&pin, ob + rb + sb + ib)) != cudaSuccess) return cuda_fail(c, e, "sim_load: pinned buffer");
         c->h_off = reinterpret_cast<int64_t *>(pin);
         if (rb) {
             c->h_res = reinterpret_cast<DevResult *>(pin + ob);
@@ -286,8 +292,9 @@ static int load_impl(sim_ctx *c, const int64_t *offsets, const int32_t *a, const
             c->h_res_big.resize(size_t(c->n_inst));
             c->h_res = c->h_res_big.data();
         }
+        if (sb) c->h_seed = reinterpret_cast<uint64_t *>(pin + ob + rb);
         if (ib) {
-            c->h_in = pin + ob + rb;
+            c->h_in = pin + ob + rb + sb;
             c->h_in_bytes = ib;
         }
     }
@@ -338,6 +345,7 @@ static int load_impl(sim_ctx *c, const int64_t *offsets, const int32_t *a, const
     if (c->n_inst > 0) ++c->launches;
     e = cudaStreamSynchronize(ls);
     if (e != cudaSuccess) return cuda_fail(c, e, "sim_load: staging kernel");
+    c->seeds_pending = false;
     c->n_total = nt;
     c->n_max = int32_t(n_max);
     c->loaded = true;
@@ -513,6 +521,9 @@ int sim_run(sim_ctx *c, sim_result *out, void *stream) {
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e;
+    if (c->seeds_pending && (e = cudaStreamSynchronize(c->load_stream)) != cudaSuccess)
+        return cuda_fail(c, e, "sim_run: tie seeds");
+    c->seeds_pending = false;
     if (c->record_completions) {
         if (!c->d_comp && (e = dalloc(c->d_comp, size_t(c->cap_total) * sizeof(int64_t))) != cudaSuccess)
             return fail(c, SIM_E_NOMEM, "sim_run: completion buffer");
@@ -607,7 +618,16 @@ int sim_set_tie_seeds(sim_ctx *c, const uint64_t *seeds) {
     if (!c->d_seed && (e = dalloc(c->d_seed, size_t(c->n_inst) * sizeof(uint64_t))) != cudaSuccess)
         return e == cudaErrorMemoryAllocation ? fail(c, SIM_E_NOMEM, "sim_set_tie_seeds: device allocation failed")
                                               : cuda_fail(c, e, "cudaMalloc");
-    e = cudaMemcpy(c->d_seed, seeds, size_t(c->n_inst) * sizeof(uint64_t), cudaMemcpyHostToDevice);
+    // A plain cudaMemcpy may return before small data has left the staging buffer, and runs on non-blocking
+    // streams would not wait for it.  From pinned memory the wait is left to the next load or run.
+    if ((e = make_load_stream(c)) != cudaSuccess ||
+        (c->seeds_pending && (e = cudaStreamSynchronize(c->load_stream)) != cudaSuccess))
+        return cuda_fail(c, e, "sim_set_tie_seeds: stream");
+    const void *src = seeds;
+    if (c->h_seed) src = std::memcpy(c->h_seed, seeds, size_t(c->n_inst) * sizeof(uint64_t));
+    e = cudaMemcpyAsync(c->d_seed, src, size_t(c->n_inst) * sizeof(uint64_t), cudaMemcpyHostToDevice, c->load_stream);
+    c->seeds_pending = c->h_seed != nullptr;
+    if (e == cudaSuccess && !c->h_seed) e = cudaStreamSynchronize(c->load_stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "sim_set_tie_seeds: copy");
     return SIM_OK;
 }

@@ -1,0 +1,71 @@
+"""The host side of the C ABI (csrc/sim_api.cpp) on the CPU, compiled against a fake CUDA runtime
+(tests/host/fake_cuda.cpp): what is ordered before what, and what happens when memory runs out."""
+import ctypes
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from tests.conftest import ROOT
+
+A_MIN, NOMEM = 1, -6
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    cxx, cuda = shutil.which("g++"), "/usr/local/cuda/include"
+    if not cxx:
+        pytest.skip("no host compiler")
+    so = tmp_path_factory.mktemp("host") / "libhost.so"
+    csrc = ROOT / "paper_2508_14544_gb300" / "csrc"
+    subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", f"-I{ROOT / 'include'}", f"-I{csrc}",
+                    f"-I{cuda}", str(csrc / "sim_api.cpp"), str(ROOT / "tests" / "host" / "fake_cuda.cpp"), "-o", str(so)],
+                   check=True)
+    lib = ctypes.CDLL(str(so))
+    for f in ("fake_used", "fake_seed"):
+        getattr(lib, f).restype = ctypes.c_uint64
+    for f in ("fake_slots", "fake_rho_calls"):
+        getattr(lib, f).restype = ctypes.c_int64
+    lib.fake_stream.restype = ctypes.c_void_p
+    lib.fake_limits.argtypes = [ctypes.c_size_t, ctypes.c_size_t]
+    lib.sim_last_error.restype = ctypes.c_char_p
+    yield lib
+    lib.fake_limits(1 << 40, (1 << 64) - 1)
+
+
+class Ctx:
+    def __init__(self, lib, n_inst, policy=A_MIN):
+        self.lib, self.n, self.h = lib, n_inst, ctypes.c_void_p()
+        assert lib.sim_create(policy, ctypes.c_int64(1000), n_inst, ctypes.byref(self.h)) == 0
+
+    def load(self, sizes):
+        off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+        x = np.ones(16, np.int32)  # device pointers: never read here
+        p = ctypes.c_void_p(x.ctypes.data)
+        return self.lib.sim_load_csr(self.h, ctypes.c_void_p(off.ctypes.data), p, p, p, p, p, 1)
+
+    def run(self, stream=None):
+        self.out = np.zeros(7 * self.n, np.int64)
+        return self.lib.sim_run(self.h, ctypes.c_void_p(self.out.ctypes.data), ctypes.c_void_p(stream))
+
+    def seeds(self, values):
+        v = np.array(values, np.uint64)
+        return self.lib.sim_set_tie_seeds(self.h, ctypes.c_void_p(v.ctypes.data))
+
+    def close(self):
+        self.lib.sim_destroy(self.h)
+
+
+@pytest.mark.parametrize("n_inst", [2, 20000])
+def test_a_run_finds_the_tie_seeds_just_set(lib, n_inst):
+    """Also on a stream that does not wait for the legacy default stream, with or without a load between, and
+    when they are set twice."""
+    c = Ctx(lib, n_inst)
+    stream = lib.fake_stream()
+    for first, load in ((7, True), (8, False), (9, True), (10, False)):
+        assert c.seeds([99] * n_inst) == 0 and c.seeds([first] * n_inst) == 0
+        assert not load or c.load([3] * n_inst) == 0
+        assert c.run(stream) == 0
+        assert lib.fake_seed() == first
+    c.close()
