@@ -128,6 +128,7 @@ cudaError_t dalloc(T *&p, size_t bytes) {
     void *q = nullptr;
     cudaError_t e = cudaMalloc(&q, bytes);
     if (e == cudaSuccess) p = static_cast<T *>(q);
+    else cudaGetLastError();  // reported by the caller, not again by the next launch
     return e;
 }
 
@@ -759,8 +760,8 @@ int sim_cr_amin_lemma(int32_t n_hist, int32_t len, int32_t l, double s, const do
     }
     double *dx = nullptr, *dout = nullptr;
     const size_t nx = size_t(n_hist) * size_t(len);
-    if ((e = cudaMalloc(&dx, nx * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&dout, size_t(n_hist) * sizeof(double))) != cudaSuccess) {
+    if ((e = dalloc(dx, nx * sizeof(double))) != cudaSuccess ||
+        (e = dalloc(dout, size_t(n_hist) * sizeof(double))) != cudaSuccess) {
         cudaFree(dx);
         return e == cudaErrorMemoryAllocation ? fail(nullptr, SIM_E_NOMEM, "sim_cr_amin_lemma: device allocation")
                                               : cuda_fail(nullptr, e, "sim_cr_amin_lemma: cudaMalloc");
@@ -794,7 +795,7 @@ int sim_cr_amin_rho(int32_t n_u, const int32_t *u_values, double *rho_out) {
     double *scratch = nullptr;
     cudaError_t e;
     const size_t bytes = size_t(nb) * (size_t(stride + 1) * sizeof(double) + sizeof(int32_t));
-    if ((e = cudaMalloc(&scratch, bytes)) != cudaSuccess)
+    if ((e = dalloc(scratch, bytes)) != cudaSuccess)
         return e == cudaErrorMemoryAllocation ? fail(nullptr, SIM_E_NOMEM, "sim_cr_amin_rho: device allocation")
                                               : cuda_fail(nullptr, e, "sim_cr_amin_rho: cudaMalloc");
     double *dout = scratch + size_t(nb) * size_t(stride);

@@ -69,3 +69,21 @@ def test_a_run_finds_the_tie_seeds_just_set(lib, n_inst):
         assert c.run(stream) == 0
         assert lib.fake_seed() == first
     c.close()
+
+
+def test_a_load_that_fits_succeeds_after_one_that_did_not(lib):
+    """The failed allocation is reported once: no later launch takes it for an error of its own."""
+    c = Ctx(lib, 1)
+    lib.fake_limits(lib.fake_used() + 10**6, (1 << 64) - 1)
+    assert c.load([1_000_000]) == NOMEM
+    assert c.load([100]) == 0 and c.run() == 0
+    lib.fake_limits(1 << 40, (1 << 64) - 1)
+    c.close()
+    assert lib.fake_used() == 0
+    lib.fake_limits(10**6, (1 << 64) - 1)
+    u, out = np.array([1 << 20], np.int32), np.zeros(1)
+    rho = lambda: lib.sim_cr_amin_rho(1, ctypes.c_void_p(u.ctypes.data), ctypes.c_void_p(out.ctypes.data))
+    assert rho() == NOMEM
+    u[0] = 9
+    assert rho() == 0 and out[0] == 9
+    lib.fake_limits(1 << 40, (1 << 64) - 1)
