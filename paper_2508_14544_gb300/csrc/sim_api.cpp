@@ -132,6 +132,15 @@ cudaError_t dalloc(T *&p, size_t bytes) {
     return e;
 }
 
+// Replaces the buffer p of `have` bytes by one of `need` if it is smaller.
+template <typename T>
+cudaError_t grow(T *&p, size_t &have, size_t need) {
+    if (need <= have) return cudaSuccess;
+    const cudaError_t e = dalloc(p, need);
+    have = e == cudaSuccess ? need : 0;
+    return e;
+}
+
 int check_device(sim_ctx *c) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
@@ -422,25 +431,20 @@ static int run_launch(sim_ctx *c, cudaStream_t st, const int32_t *work_dev, int3
     int64_t blocks = int64_t(n_sm) * per_sm;
     blocks = std::min<int64_t>(blocks, (n_work + wpb - 1) / wpb);
     blocks = std::max<int64_t>(blocks, 1);
-    const int64_t slots = blocks * wpb;
+    // queue buffers and, without shared memory, workspaces of every warp; fewer warps if they do not fit
     const int64_t main_cap = std::max<int64_t>(c->n_max, 1);
-    const size_t main_need = size_t(slots) * 2 * main_cap * sizeof(QEnt);
-    if (main_need > c->main_bytes) {
-        if ((e = dalloc(c->d_main, main_need)) != cudaSuccess) {
-            c->main_bytes = 0;
-            return e == cudaErrorMemoryAllocation ? fail(c, SIM_E_NOMEM, "sim_run: queue buffers") : cuda_fail(c, e, "cudaMalloc");
-        }
-        c->main_bytes = main_need;
-    }
-    if (!smem) {
-        const size_t need = size_t(slots) * per_warp;
-        if (need > c->gws_bytes) {
-            if ((e = dalloc(c->d_gws, need)) != cudaSuccess) {
-                c->gws_bytes = 0;
-                return e == cudaErrorMemoryAllocation ? fail(c, SIM_E_NOMEM, "sim_run: workspace") : cuda_fail(c, e, "cudaMalloc");
-            }
-            c->gws_bytes = need;
-        }
+    int64_t slots;
+    for (;;) {
+        slots = blocks * wpb;
+        e = grow(c->d_main, c->main_bytes, size_t(slots) * 2 * main_cap * sizeof(QEnt));
+        if (e == cudaSuccess && !smem) e = grow(c->d_gws, c->gws_bytes, size_t(slots) * per_warp);
+        if (e == cudaSuccess) break;
+        if (e != cudaErrorMemoryAllocation) return cuda_fail(c, e, "cudaMalloc");
+        dfree(c->d_main);
+        dfree(c->d_gws);
+        c->main_bytes = c->gws_bytes = 0;
+        if (blocks == 1) return fail(c, SIM_E_NOMEM, "sim_run: queue buffers and workspace");
+        blocks = (blocks + 1) / 2;
     }
     p.M = c->M;
     p.n_work = n_work;

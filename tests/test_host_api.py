@@ -87,3 +87,21 @@ def test_a_load_that_fits_succeeds_after_one_that_did_not(lib):
     u[0] = 9
     assert rho() == 0 and out[0] == 9
     lib.fake_limits(1 << 40, (1 << 64) - 1)
+
+
+def test_runs_with_fewer_warps_when_the_queue_buffers_do_not_fit(lib):
+    """The queue buffers of a launch take 32 bytes x largest instance per simulating warp: 292 GB for one of five
+    million on 12 warps per SM.  With 100 GB left fewer warps simulate, also in the global-memory re-run, whose
+    workspace needs room too."""
+    for status in (0, -100):  # -100: every instance outgrew the shared-memory slots
+        c = Ctx(lib, 3000)
+        assert c.load([5_000_000] + [2] * 2999) == 0
+        lib.fake_status(status)
+        lib.fake_limits(lib.fake_used() + 100 * 10**9, (1 << 64) - 1)
+        assert c.run() == 0 and 200 <= lib.fake_slots() <= 600
+        lib.fake_limits(lib.fake_used() + 10**6, (1 << 64) - 1)
+        assert c.run() == 0  # the same buffers again
+        c.close()
+        lib.fake_status(0)
+        lib.fake_limits(1 << 40, (1 << 64) - 1)
+    assert lib.fake_used() == 0
