@@ -792,14 +792,18 @@ int sim_cr_amin_rho(int32_t n_u, const int32_t *u_values, double *rho_out) {
             return fail(nullptr, SIM_E_INVAL, "sim_cr_amin_rho: u_values[%d]=%d outside [1, 2^20]", k, u_values[k]);
         umax = std::max(umax, u_values[k]);
     }
-    // batches of at most 1 GB of scratch, 2^20 values; one allocation: scratch, results, values
+    // batches of at most 1 GB of scratch (half as many values while that does not fit), 2^20 values; one
+    // allocation: scratch, results, values
     const int64_t stride = simgb::rho_scratch_doubles(n_u, umax);
     const int64_t per_batch = stride ? std::max<int64_t>(1, (int64_t(1) << 30) / (stride * int64_t(sizeof(double)))) : 1 << 20;
-    const int32_t nb = int32_t(std::min<int64_t>(per_batch, n_u));
+    int32_t nb = int32_t(std::min<int64_t>(per_batch, n_u));
     double *scratch = nullptr;
     cudaError_t e;
-    const size_t bytes = size_t(nb) * (size_t(stride + 1) * sizeof(double) + sizeof(int32_t));
-    if ((e = dalloc(scratch, bytes)) != cudaSuccess)
+    while ((e = dalloc(scratch, size_t(nb) * (size_t(stride + 1) * sizeof(double) + sizeof(int32_t)))) ==
+               cudaErrorMemoryAllocation &&
+           nb > 1)
+        nb = (nb + 1) / 2;
+    if (e != cudaSuccess)
         return e == cudaErrorMemoryAllocation ? fail(nullptr, SIM_E_NOMEM, "sim_cr_amin_rho: device allocation")
                                               : cuda_fail(nullptr, e, "sim_cr_amin_rho: cudaMalloc");
     double *dout = scratch + size_t(nb) * size_t(stride);

@@ -92,10 +92,9 @@ cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int) {
 cudaError_t cudaMalloc(void **p, size_t n) {
     *p = nullptr;
     if (g_used + n > g_limit) return g_last = cudaErrorMemoryAllocation;
-    // large blocks are never read here: their size is all that counts
-    const size_t m = n < (size_t(1) << 26) ? n : 64;
-    *p = std::malloc(m);
-    std::memset(*p, 0xab, m);
+    // of very large blocks (queue buffers, never touched here) only the size counts
+    *p = std::malloc(n < (size_t(1) << 31) ? n : 64);
+    if (n < (size_t(1) << 26)) std::memset(*p, 0xab, n);
     g_blocks[*p] = n;
     g_used += n;
     return cudaSuccess;

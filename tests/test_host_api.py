@@ -105,3 +105,16 @@ def test_runs_with_fewer_warps_when_the_queue_buffers_do_not_fit(lib):
         lib.fake_status(0)
         lib.fake_limits(1 << 40, (1 << 64) - 1)
     assert lib.fake_used() == 0
+
+
+def test_rho_works_in_smaller_batches_when_its_scratch_does_not_fit(lib):
+    """18 values of 2^20 ask for 1 GB of scratch at once (59 MB each): with 300 MB left they are computed in
+    batches of a few, with the same results."""
+    u, out = np.full(18, 1 << 20, np.int32) - np.arange(18, dtype=np.int32), np.zeros(18)
+    for room in (1 << 40, lib.fake_used() + 300 * 10**6):
+        lib.fake_limits(room, (1 << 64) - 1)
+        out[:] = 0
+        assert lib.sim_cr_amin_rho(18, ctypes.c_void_p(u.ctypes.data), ctypes.c_void_p(out.ctypes.data)) == 0
+        assert np.array_equal(out, u)
+    lib.fake_limits(1 << 40, (1 << 64) - 1)
+    assert lib.fake_used() == 0
