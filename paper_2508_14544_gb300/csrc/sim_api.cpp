@@ -9,9 +9,9 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
-#include <vector>
 
 #include "sim.h"
 #include "sim_internal.h"
@@ -76,7 +76,7 @@ struct sim_ctx {
     int64_t *h_off = nullptr;            // pinned block: the offsets (n_inst + 1) for their upload, results, seeds, inputs
     int64_t launches = 0;
     DevResult *h_res = nullptr;          // results of the last run: behind the offsets, or h_res_big's
-    std::vector<DevResult> h_res_big;
+    std::unique_ptr<DevResult[]> h_res_big;
     uint64_t *h_seed = nullptr;          // pinned copy of the tie seeds (A_min, up to kPinnedResults instances)
     bool seeds_pending = false;          // their upload is in load_stream and has not been waited for
     unsigned char *h_in = nullptr;       // pinned copy of small host inputs (h_in_bytes, from the first such load)
@@ -293,14 +293,15 @@ static int load_impl(sim_ctx *c, const int64_t *offsets, const int32_t *a, const
         const size_t rb = c->n_inst <= kPinnedResults ? (size_t(c->n_inst) * sizeof(DevResult) + 255) & ~size_t(255) : 0;
         const size_t sb = c->policy == SIM_AMIN && rb ? (size_t(c->n_inst) * sizeof(uint64_t) + 255) & ~size_t(255) : 0;
         const size_t ib = small ? size_t(nsrc) * nt * sizeof(int32_t) : 0;
+        if (!rb && !c->h_res_big) c->h_res_big.reset(new (std::nothrow) DevResult[size_t(c->n_inst)]);
+        if (!rb && !c->h_res_big) return fail(c, SIM_E_NOMEM, "sim_load: host memory for the results");
         unsigned char *pin = nullptr;
         if ((e = cudaMallocHost(&pin, ob + rb + sb + ib)) != cudaSuccess) return cuda_fail(c, e, "sim_load: pinned buffer");
         c->h_off = reinterpret_cast<int64_t *>(pin);
         if (rb) {
             c->h_res = reinterpret_cast<DevResult *>(pin + ob);
         } else {
-            c->h_res_big.resize(size_t(c->n_inst));
-            c->h_res = c->h_res_big.data();
+            c->h_res = c->h_res_big.get();
         }
         if (sb) c->h_seed = reinterpret_cast<uint64_t *>(pin + ob + rb);
         if (ib) {
@@ -377,9 +378,10 @@ int sim_load(sim_ctx *c, int32_t n, const int32_t *a, const int32_t *s, const in
              const int32_t *o, int device_ptrs) {
     if (!c) return SIM_E_INVAL;
     if (n < 0) return fail(c, SIM_E_INVAL, "sim_load: n_per_instance=%d < 0", n);
-    std::vector<int64_t> off(size_t(c->n_inst) + 1);
+    const std::unique_ptr<int64_t[]> off(new (std::nothrow) int64_t[size_t(c->n_inst) + 1]);
+    if (!off) return fail(c, SIM_E_NOMEM, "sim_load: host memory for the offsets");
     for (int32_t i = 0; i <= c->n_inst; ++i) off[i] = int64_t(i) * n;
-    return sim_load_csr(c, off.data(), a, s, l, u, o, device_ptrs);
+    return sim_load_csr(c, off.get(), a, s, l, u, o, device_ptrs);
 }
 
 // One launch of the simulation kernel over n_work instances (all, or the device list work_dev).
@@ -492,14 +494,20 @@ static int simulate(sim_ctx *c, cudaStream_t st, int wps, bool dense, float *ms)
         if (e != cudaSuccess) rc = cuda_fail(c, e, "sim_run: simulation kernel");
     }
     // instances whose active set outgrew the shared-memory workspace: re-run from global memory
-    std::vector<int32_t> redo;
+    int32_t n_redo = 0;
     if (rc == SIM_OK)
-        for (int32_t i = 0; i < c->n_inst; ++i)
-            if (c->h_res[i].status == simgb::kStatusCapacity) redo.push_back(i);
-    if (rc == SIM_OK && !redo.empty()) {
-        e = cudaMemcpyAsync(c->d_work, redo.data(), redo.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st);
+        for (int32_t i = 0; i < c->n_inst; ++i) n_redo += c->h_res[i].status == simgb::kStatusCapacity;
+    std::unique_ptr<int32_t[]> redo;
+    if (n_redo) {
+        redo.reset(new (std::nothrow) int32_t[size_t(n_redo)]);
+        if (!redo) rc = fail(c, SIM_E_NOMEM, "sim_run: host memory for the work list");
+    }
+    if (rc == SIM_OK && n_redo) {
+        for (int32_t i = 0, k = 0; i < c->n_inst; ++i)
+            if (c->h_res[i].status == simgb::kStatusCapacity) redo[k++] = i;
+        e = cudaMemcpyAsync(c->d_work, redo.get(), size_t(n_redo) * sizeof(int32_t), cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) rc = cuda_fail(c, e, "sim_run: work list");
-        if (rc == SIM_OK) rc = run_launch(c, st, c->d_work, int32_t(redo.size()), false, c->warps_per_sm);
+        if (rc == SIM_OK) rc = run_launch(c, st, c->d_work, n_redo, false, c->warps_per_sm);
         if (rc == SIM_OK) {
             e = cudaMemcpyAsync(c->h_res, c->d_res, sizeof(DevResult) * size_t(c->n_inst), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);

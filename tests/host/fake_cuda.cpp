@@ -56,11 +56,14 @@ void later_copy(Stream &st, void *dst, const void *src, size_t n, bool staged) {
 }  // namespace
 
 // an allocation on the host above the limit fails
+void *operator new(size_t n, const std::nothrow_t &) noexcept { return n > g_throw_above ? nullptr : std::malloc(n ? n : 1); }
 void *operator new(size_t n) {
-    void *p = n > g_throw_above ? nullptr : std::malloc(n ? n : 1);
+    void *p = operator new(n, std::nothrow);
     if (!p) throw std::bad_alloc();
     return p;
 }
+void *operator new[](size_t n, const std::nothrow_t &t) noexcept { return operator new(n, t); }
+void operator delete[](void *p) noexcept { std::free(p); }
 void operator delete(void *p) noexcept { std::free(p); }
 void operator delete(void *p, size_t) noexcept { std::free(p); }
 

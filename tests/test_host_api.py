@@ -118,3 +118,23 @@ def test_rho_works_in_smaller_batches_when_its_scratch_does_not_fit(lib):
         assert np.array_equal(out, u)
     lib.fake_limits(1 << 40, (1 << 64) - 1)
     assert lib.fake_used() == 0
+
+
+@pytest.mark.parametrize("entry", ["csr", "uniform", "redo"])
+def test_host_memory_that_runs_out_is_an_error_code(lib, entry):
+    """No exception leaves the C entry points, and the context works again once there is memory."""
+    n = 20000  # results above 16384 instances are kept in ordinary memory: 1.1 MB
+    c = Ctx(lib, n)
+    one = np.ones(16, np.int32)
+    p = ctypes.c_void_p(one.ctypes.data)
+    if entry == "redo":  # the list of the instances to run again takes 80 kB
+        lib.fake_status(-100)
+        assert c.load([2] * n) == 0
+    lib.fake_limits(1 << 40, 50_000)
+    for _ in range(2):
+        assert (c.run() if entry == "redo" else c.load([2] * n) if entry == "csr" else
+                lib.sim_load(c.h, 2, p, p, p, p, p, 1)) == NOMEM
+    lib.fake_limits(1 << 40, (1 << 64) - 1)
+    assert c.load([2] * n) == 0 and c.run() == 0
+    lib.fake_status(0)
+    c.close()
