@@ -110,6 +110,11 @@ __device__ __forceinline__ int quotient_lb(int a, int b) {
     return a >= (1 << 22) ? max(q - 40, 0) : q + (r >= b ? 1 : 0) - (r < 0 ? 1 : 0);
 }
 
+// Sums modulo 2^32.  W of a free slot or of an endpoint before t, and V of a witness that has passed, go on
+// taking updates that nobody reads, and wrap on long streams.
+__device__ __forceinline__ int plus(int a, int b) { return int(unsigned(a) + unsigned(b)); }
+__device__ __forceinline__ int minus(int a, int b) { return int(unsigned(a) - unsigned(b)); }
+
 __device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
 // ---------------------------------------------------------------------------------------------
@@ -461,7 +466,7 @@ __device__ __forceinline__ void subtract_job(const Ws &w, int end, int e, int b)
         for (int j = 0; j < 4; ++j) {
             const int i = p + 32 * j + lane_id();
             const int2 ew = w.EW[i];
-            if (unsigned(ew.x) <= unsigned(e)) w.EW[i].y = ew.y - b - ew.x;
+            if (unsigned(ew.x) <= unsigned(e)) w.EW[i].y = minus(ew.y, b + ew.x);
         }
     }
 }
@@ -475,8 +480,8 @@ __device__ __forceinline__ void subtract_two(const Ws &w, int end, int e0, int b
         for (int j = 0; j < 4; ++j) {
             const int i = p + 32 * j + lane_id();
             int2 ew = w.EW[i];
-            if (ew.x <= e0) ew.y -= b0 + ew.x;
-            if (ew.x <= e1) ew.y -= b1 + ew.x;
+            if (ew.x <= e0) ew.y = minus(ew.y, b0 + ew.x);
+            if (ew.x <= e1) ew.y = minus(ew.y, b1 + ew.x);
             if (ew.x <= most) w.EW[i].y = ew.y;
         }
     }
@@ -602,7 +607,8 @@ __device__ bool state_ok(const Ws &w, const Queue &q, int A, int end, int t, int
 // batch-time sums; the plain copy has neither.
 // All memory sums are at most M <= 2^26 where they are compared (V, need and a candidate's points
 // belong to feasible schedules, a violated one exceeds M by one job's memory at most) and a projected
-// step at most kMaxStep + 2^26, so 32 bits hold them and W <= 2^31 - 1.
+// step at most kMaxStep + 2^26, so 32 bits hold them and W <= 2^31 - 1 at the endpoints that are still to
+// come (the sums that are not compared wrap: plus, minus).
 // ---------------------------------------------------------------------------------------------
 template <int POL, bool SMEM, bool INS>
 __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, int inst) {
@@ -891,8 +897,8 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
 #pragma unroll
                     for (int j = 0; j < N; ++j) {
                         m = min(m, k[j]);
-                        if (x[j].x <= py) x[j].y += x[j].x + pc;
-                        if (x[j].x <= qy) x[j].y -= x[j].x + qc;
+                        if (x[j].x <= py) x[j].y = plus(x[j].y, x[j].x + pc);
+                        if (x[j].x <= qy) x[j].y = minus(x[j].y, x[j].x + qc);
                         if (x[j].x <= pq) w.EW[p + 32 * j + lane].y = x[j].y;
                     }
                     int first = 0, last = 0;
@@ -976,8 +982,8 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                     }
 #pragma unroll
                     for (int j = 0; j < N; ++j) {
-                        if (x[j].x <= py) x[j].y += x[j].x + pc;
-                        if (kSub && x[j].x <= qy) x[j].y -= x[j].x + qc;
+                        if (x[j].x <= py) x[j].y = plus(x[j].y, x[j].x + pc);
+                        if (kSub && x[j].x <= qy) x[j].y = minus(x[j].y, x[j].x + qc);
                         if (x[j].x <= pq) w.EW[p + 32 * j + lane].y = x[j].y;
                         if (x[j].x >= y) vy += bb[j] + y;
                         if (unsigned(x[j].x - t) < unsigned(hL)) wm = max(wm, x[j].y);
@@ -1031,7 +1037,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                     if (POL == P_AMIN) w.K[end] = unsigned(h.key);
                     py = y;
                     pc = h.s - t + 1;
-                    if (kWit) cv += y < ct ? 0 : pc + ct;
+                    if (kWit) cv = plus(cv, y < ct ? 0 : pc + ct);
                     ++end;
                     ++A;
                     need += h.s + 1;
@@ -1103,7 +1109,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                         const bool early = done && e[j] > t;
                         if (POL == P_AELL) e1 = min(e1, done ? UINT_MAX : unsigned(e[j]));
                         ne += early ? 1 : 0;
-                        dv += early && e[j] >= ct ? bb[j] + ct : 0;
+                        dv = plus(dv, early && e[j] >= ct ? bb[j] + ct : 0);
                         ek = early ? e[j] : ek;
                         bk = early ? bb[j] : bk;
                         if (done) w.EW[i] = make_int2(-1, e[j]);
@@ -1126,7 +1132,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
                 const int most = __reduce_max_sync(FULL, ne), tot = int(__reduce_add_sync(FULL, unsigned(ne)));
                 const int e1st = __reduce_max_sync(FULL, ek), b1st = __reduce_max_sync(FULL, bk);
                 const bool free_q = __reduce_max_sync(FULL, qy) < 0;
-                cv -= int(__reduce_add_sync(FULL, unsigned(dv)));
+                cv = minus(cv, int(__reduce_add_sync(FULL, unsigned(dv))));
                 if (tot == 1) {
                     if (free_q) {
                         qy = e1st;

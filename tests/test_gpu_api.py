@@ -367,3 +367,24 @@ def test_every_request_active_at_once(pol, opts):
         w = _w(sel, 100_000)
         got, _ = gpu_run(pol, w, **opts)
         assert_same(got, oracle_run(pol, w), tag=f"full pol={pol} n={len(sel[0]['o'])} {opts}")
+
+
+@pytest.mark.parametrize("pol", [0, 1, 2, 3, 4])
+def test_busy_streams_at_late_steps(pol):
+    """Steps of about 10^9 (below A_ell's limit of 2^30): every admission changes the unread sums of passed
+    endpoints and witnesses by about that much, so they wrap many times; the compared ones stay exact."""
+    rng = np.random.default_rng(52)
+    parts = []
+    for i in range(12):
+        n = 1500
+        o = rng.integers(1, 120, n)
+        l = rng.integers(1, o + 1)
+        a = 1_000_000_000 + np.sort(rng.integers(0, 20 * n // (i + 1), n))
+        parts.append(dict(a=a, s=rng.integers(1, 30, n), l=l, u=o + rng.integers(0, 60, n), o=o))
+    w = _w(parts, 1500)
+    ref, rcomp = oracle_run(pol, w, completions=True)
+    assert np.all(ref["status"] == 0)
+    for opts in ({}, {"debug_checks": 1}):
+        got, comp = gpu_run(pol, w, completions=True, **opts)
+        assert_same(got, ref, tag=f"late pol={pol} {opts}")
+        assert np.array_equal(comp, rcomp)
