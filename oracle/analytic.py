@@ -14,6 +14,10 @@ shares no code with the CUDA evaluators (``csrc/sim_analytic.cu``), which use di
 * ``rho(u)`` - the largest generalized eigenvalue of (A_u, B_u), i.e. the spectral radius of
   B_u^{-1} A_u that bounds the Rayleigh quotient (Section 4.1), by scipy's symmetric generalized
   eigensolver on the dense matrices.
+* ``rho_long(u)`` - the same in O(u) operations per step and long double, for large u: an eigenvector by
+  power iteration (prefix sums for A_u v, the printed tridiagonal inverse of B_u), and its Rayleigh
+  quotient from the lemma's sums, all of whose terms are positive (an error d of the vector changes
+  the quotient by about d^2).
 * ``binv_closed(u)`` - the tridiagonal inverse of B_u printed in Section 4.1, as exact Fractions.
 * ``lg_cr(q)`` - the closed form of the LG theorem (linearly weighted geometric outputs).
 * ``two_point_cr(alpha, t)`` - the two-point form in the proof of Theorem thm:no,
@@ -70,6 +74,38 @@ def rho(u: int) -> float:
     from scipy.linalg import eigh
     A, B = matrices(u)
     return float(eigh(A, B, eigvals_only=True).max())
+
+
+def rho_long(u: int) -> float:
+    ld = np.longdouble
+    i = np.arange(1, u + 1).astype(ld)
+    diag = 4 * i / (4 * i * i - 1)
+    diag[-1] = 1 / (2 * i[-1] - 1)
+    off = 1 / (2 * i + 1)
+
+    def tail(x):  # sums over j >= i
+        return np.cumsum(x[::-1])[::-1]
+
+    def after(x):  # sums over j > i
+        return np.append(tail(x)[1:], ld(0))
+
+    v, lam = np.ones(u, ld), ld(0)
+    for _ in range(100):
+        w = tail(v / i)
+        num = np.sum(tail(i * v) * (w + 2 * after(w)))
+        den = np.sum(i * i * v * (v + 2 * after(v)))
+        new = num / den
+        if abs(new - lam) <= 4 * np.finfo(ld).eps * new:
+            break
+        lam = new
+        # a_ij = i j / 2 + j^2 - j^3 / (2 i) for j <= i, symmetric
+        av = (i * np.sum(i * v) / 2 + np.cumsum(i * i * v) - np.cumsum(i ** 3 * v) / (2 * i) + i * i * after(v)
+              - i ** 3 * after(v / i) / 2)
+        z = diag * av
+        z[1:] -= off[:-1] * av[:-1]
+        z[:-1] -= off[:-1] * av[1:]
+        v = z / np.max(np.abs(z))
+    return float(new)
 
 
 def binv_closed(u: int):

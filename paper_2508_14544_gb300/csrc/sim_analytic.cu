@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(256) k_lemma(int32_t n_hist, int32_t len, int3
 }
 
 constexpr int kRhoThreads = 256;
+constexpr size_t kRhoSmemMax = size_t(200) * 1024;
 constexpr int kRhoArrays = 7;  // per i: S, T, 1/(i(i-1)), 1/(8(2i-1)), w_i, 3 - 2/i, 2i - 1
 
 __global__ void __launch_bounds__(kRhoThreads) k_rho(const int32_t *__restrict__ us, double *__restrict__ out,
@@ -309,47 +310,56 @@ cudaError_t launch_lemma(int32_t n_hist, int32_t len, int32_t l, double s, const
     return cudaGetLastError();
 }
 
+static size_t rho_smem_bytes(int cluster, int32_t u_max) {
+    const size_t b = size_t((u_max + cluster - 1) / cluster) * kRhoArrays * sizeof(double);
+    return b <= kRhoSmemMax ? b : 0;  // 0: the arrays live in global scratch
+}
+
+static cudaLaunchConfig_t rho_config(const RhoPlan &plan, int32_t n_u, cudaLaunchAttribute *attr, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(n_u) * unsigned(plan.cluster));
+    cfg.blockDim = dim3(kRhoThreads);
+    cfg.dynamicSmemBytes = plan.smem;
+    cfg.stream = st;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = unsigned(plan.cluster);
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
 // Blocks per cluster: about 512 indices of the largest u each, at most 8 blocks, or 16 (which k_rho opts
 // in to) for a few values: a GPU partition holds few clusters of 16, and 25 values of up to 20,000 took
 // 0.79 ms with 16 blocks each, one of 10^5 0.70 ms (8 blocks: 1.0).
-static int rho_cluster(int32_t n_u, int32_t u_max) {
-    const int most = n_u <= 8 ? 16 : 8;
-    int c = 1;
-    while (c < most && 512 * c < u_max) c <<= 1;
-    return c;
-}
-
-static size_t rho_smem_bytes(int32_t n_u, int32_t u_max) {
-    const int c = rho_cluster(n_u, u_max);
-    return size_t((u_max + c - 1) / c) * kRhoArrays * sizeof(double);
-}
-
-int64_t rho_scratch_doubles(int32_t n_u, int32_t u_max) {
-    return rho_smem_bytes(n_u, u_max) <= size_t(200) * 1024 ? 0 : int64_t(kRhoArrays) * u_max;
-}
-
-cudaError_t launch_rho(int32_t n_u, int32_t u_max, const int32_t *us, double *out, double *scratch, int32_t max_iter,
-                       cudaStream_t st) {
-    if (n_u <= 0) return cudaSuccess;
-    const size_t smem = scratch ? 0 : rho_smem_bytes(n_u, u_max);
-    const int64_t stride = int64_t(kRhoArrays) * u_max;
-    cudaError_t e =
-        cudaFuncSetAttribute((const void *)k_rho, cudaFuncAttributeMaxDynamicSharedMemorySize, int(size_t(200) * 1024));
+cudaError_t rho_plan(int32_t n_u, int32_t u_max, RhoPlan *plan) {
+    cudaError_t e = cudaFuncSetAttribute((const void *)k_rho, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kRhoSmemMax));
     if (e == cudaSuccess) e = cudaFuncSetAttribute((const void *)k_rho, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    const int c = rho_cluster(n_u, u_max);
-    cfg.gridDim = dim3(unsigned(n_u) * unsigned(c));
-    cfg.blockDim = dim3(kRhoThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr = {};
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = unsigned(c);
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_rho, us, out, scratch, stride, max_iter);
+    const int most = n_u <= 8 ? 16 : 8;
+    plan->cluster = 1;
+    while (plan->cluster < most && 512 * plan->cluster < u_max) plan->cluster <<= 1;
+    plan->smem = rho_smem_bytes(plan->cluster, u_max);
+    if (plan->cluster == 16) {  // needs 16 SMs of one partition, where not every SM need be available
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t cfg = rho_config(*plan, 1, &attr, nullptr);
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, k_rho, &cfg) != cudaSuccess || fit < 1) {
+            cudaGetLastError();
+            plan->cluster = 8;
+            plan->smem = rho_smem_bytes(8, u_max);
+        }
+    }
+    plan->scratch = plan->smem ? 0 : int64_t(kRhoArrays) * u_max;
+    return cudaSuccess;
+}
+
+cudaError_t launch_rho(const RhoPlan &plan, int32_t n_u, const int32_t *us, double *out, double *scratch,
+                       int32_t max_iter, cudaStream_t st) {
+    if (n_u <= 0) return cudaSuccess;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = rho_config(plan, n_u, &attr, st);
+    return cudaLaunchKernelEx(&cfg, k_rho, us, out, scratch, plan.scratch, max_iter);
 }
 
 }  // namespace simgb

@@ -802,11 +802,13 @@ int sim_cr_amin_rho(int32_t n_u, const int32_t *u_values, double *rho_out) {
     }
     // batches of at most 1 GB of scratch (half as many values while that does not fit), 2^20 values; one
     // allocation: scratch, results, values
-    const int64_t stride = simgb::rho_scratch_doubles(n_u, umax);
+    simgb::RhoPlan plan;
+    cudaError_t e = simgb::rho_plan(n_u, umax, &plan);
+    if (e != cudaSuccess) return cuda_fail(nullptr, e, "sim_cr_amin_rho: kernel set-up");
+    const int64_t stride = plan.scratch;
     const int64_t per_batch = stride ? std::max<int64_t>(1, (int64_t(1) << 30) / (stride * int64_t(sizeof(double)))) : 1 << 20;
     int32_t nb = int32_t(std::min<int64_t>(per_batch, n_u));
     double *scratch = nullptr;
-    cudaError_t e;
     while ((e = dalloc(scratch, size_t(nb) * (size_t(stride + 1) * sizeof(double) + sizeof(int32_t)))) ==
                cudaErrorMemoryAllocation &&
            nb > 1)
@@ -820,7 +822,7 @@ int sim_cr_amin_rho(int32_t n_u, const int32_t *u_values, double *rho_out) {
     for (int32_t b = 0; b < n_u && rc == SIM_OK; b += nb) {
         const int32_t m = std::min(nb, n_u - b);
         if ((e = cudaMemcpy(dus, u_values + b, size_t(m) * sizeof(int32_t), cudaMemcpyHostToDevice)) != cudaSuccess ||
-            (e = simgb::launch_rho(m, umax, dus, dout, stride ? scratch : nullptr, 200, nullptr)) != cudaSuccess ||
+            (e = simgb::launch_rho(plan, m, dus, dout, stride ? scratch : nullptr, 200, nullptr)) != cudaSuccess ||
             (e = cudaMemcpy(rho_out + b, dout, size_t(m) * sizeof(double), cudaMemcpyDeviceToHost)) != cudaSuccess)
             rc = cuda_fail(nullptr, e, "sim_cr_amin_rho");
     }

@@ -121,10 +121,14 @@ cudaError_t launch_batch_time(const int64_t *sums, const DevResult *res, const d
                               cudaStream_t st);
 cudaError_t launch_lemma(int32_t n_hist, int32_t len, int32_t l, double s, const double *x, double *out,
                          cudaStream_t st);
-// Global scratch per value (doubles) that launch_rho needs for n_u values when the largest is u_max; 0: none,
-// and scratch must be null.
-int64_t rho_scratch_doubles(int32_t n_u, int32_t u_max);
-cudaError_t launch_rho(int32_t n_u, int32_t u_max, const int32_t *us, double *out, double *scratch, int32_t max_iter,
-                       cudaStream_t st);
+// Launch shape of the spectral-radius kernel for n_u values of which the largest is u_max.
+struct RhoPlan {
+    int cluster;      // blocks per value
+    size_t smem;      // bytes of shared memory per block, 0 when the arrays live in scratch
+    int64_t scratch;  // doubles of global scratch per value (0: none, and scratch must be null)
+};
+cudaError_t rho_plan(int32_t n_u, int32_t u_max, RhoPlan *plan);
+cudaError_t launch_rho(const RhoPlan &plan, int32_t n_u, const int32_t *us, double *out, double *scratch,
+                       int32_t max_iter, cudaStream_t st);
 
 }  // namespace simgb

@@ -168,8 +168,11 @@ cudaError_t launch_batch_time(const int64_t *, const DevResult *, const double *
     return cudaSuccess;
 }
 cudaError_t launch_lemma(int32_t, int32_t, int32_t, double, const double *, double *, cudaStream_t) { return cudaSuccess; }
-int64_t rho_scratch_doubles(int32_t, int32_t u_max) { return 7 * int64_t(u_max); }
-cudaError_t launch_rho(int32_t n_u, int32_t, const int32_t *us, double *out, double *, int32_t, cudaStream_t) {
+cudaError_t rho_plan(int32_t, int32_t u_max, RhoPlan *plan) {
+    *plan = {8, 0, 7 * int64_t(u_max)};
+    return cudaSuccess;
+}
+cudaError_t launch_rho(const RhoPlan &, int32_t n_u, const int32_t *us, double *out, double *, int32_t, cudaStream_t) {
     ++g_rho_calls;
     of(nullptr).ops.push_back([=] {
         for (int k = 0; k < n_u; ++k) out[k] = us[k];

@@ -93,3 +93,31 @@ def test_rho_bounds_and_fit(u):
     if u >= 10:
         fit = 0.2555 * np.log(u + 0.2793) + 1.1587
         assert abs(r - fit) / fit < 0.02
+
+
+@pytest.mark.parametrize("u", [1, 2, 3, 10, 30])
+def test_rho_long_equals_sixty_digits(u):
+    """Power iteration on the matrices as defined, in 60-digit arithmetic: the long-double value is its
+    correctly rounded double to 2 units."""
+    from decimal import Decimal as D, localcontext
+    with localcontext() as c:
+        c.prec = 60
+        A, B = _exact_AB(u)
+        A, B = ([[D(x.numerator) / D(x.denominator) for x in row] for row in m] for m in (A, B))
+        Bi = [[D(x.numerator) / D(x.denominator) for x in row] for row in an.binv_closed(u)]
+
+        def mul(m, x):
+            return [sum(a * b for a, b in zip(row, x)) for row in m]
+
+        v = [D(1)] * u
+        for _ in range(40):
+            v = mul(Bi, mul(A, v))
+            top = max(v)
+            v = [x / top for x in v]
+        ref = float(sum(a * b for a, b in zip(v, mul(A, v))) / sum(a * b for a, b in zip(v, mul(B, v))))
+    assert abs(an.rho_long(u) - ref) <= 2.0 ** -51 * ref
+
+
+def test_rho_long_against_the_dense_solver():
+    for u in (100, 300):
+        assert abs(an.rho_long(u) - an.rho(u)) <= 1e-10 * an.rho(u)

@@ -132,3 +132,18 @@ def test_rho_cluster_sizes_and_scratch():
     assert abs(cr_amin_rho([58600])[0] - cr_amin_rho([58600] * 9)[4]) <= 1e-12  # scratch, 16 and 8 blocks
     for u, r in zip(us[:8], alone):
         assert abs(r - an.rho(u)) <= 1e-10 * r, u
+
+
+def test_rho_to_rounding():
+    """Every launch shape against the long-double value: one block to 16, arrays in shared memory up to 200 KB
+    a block (u = 58500 alone) and in global scratch, alone and next to each other (8 blocks each).  Sums of
+    positive terms over a thread's run (up to 50), its warp, block and cluster: below 100 roundings of
+    1.1e-16 each in numerator and denominator."""
+    from oracle import analytic as an
+    from paper_2508_14544_gb300 import cr_amin_rho
+    us = [1, 2, 3, 10, 33, 100, 512, 513, 1025, 2049, 8193, 20000, 33000, 58500, 58600]
+    ref = np.array([an.rho_long(u) for u in us])
+    alone = np.array([cr_amin_rho([u])[0] for u in us])
+    assert np.all(np.abs(alone - ref) <= 2.2e-14 * ref), (alone - ref) / ref
+    for k in (9, 12, len(us)):
+        assert np.all(np.abs(cr_amin_rho(us[:k]) - ref[:k]) <= 2.2e-14 * ref[:k])
