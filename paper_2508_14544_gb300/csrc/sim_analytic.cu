@@ -92,6 +92,8 @@ __device__ __forceinline__ LemmaSums then(const LemmaSums &a, const LemmaSums &b
     return {a.X + b.X, a.S1 + b.S1, a.S2 + b.S2, fma(double(b.n), a.S2, a.G) + b.G, a.n + b.n};
 }
 
+static_assert(3 * kLemmaMaxLen * sizeof(double) <= 227 * 1024, "k_lemma's table");
+
 template <int T>
 __global__ void __launch_bounds__(256) k_lemma(int32_t n_hist, int32_t len, int32_t l, double s,
                                                 const double *__restrict__ x, double *__restrict__ out) {
@@ -303,7 +305,9 @@ cudaError_t launch_lemma(int32_t n_hist, int32_t len, int32_t l, double s, const
     const Fn fn = T == 1 ? k_lemma<1> : T == 2 ? k_lemma<2> : T == 4 ? k_lemma<4> : T == 8 ? k_lemma<8>
                   : T == 16 ? k_lemma<16> : k_lemma<32>;
     if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        // to the longest histograms' bytes, not to this launch's: other threads share the kernel
+        e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(3 * kLemmaMaxLen * sizeof(double)));
         if (e != cudaSuccess) return e;
     }
     fn<<<blocks, threads, smem, st>>>(n_hist, len, l, s, x, out);

@@ -119,6 +119,7 @@ cudaError_t launch_run(int policy, const RunParams &p, int blocks, int warps_per
 cudaError_t launch_ratio(const DevResult *pol, const DevResult *ref, double *out, int32_t n, cudaStream_t st);
 cudaError_t launch_batch_time(const int64_t *sums, const DevResult *res, const double *coef, double *out, int32_t n,
                               cudaStream_t st);
+constexpr int kLemmaMaxLen = 8192;  // lengths of a histogram
 cudaError_t launch_lemma(int32_t n_hist, int32_t len, int32_t l, double s, const double *x, double *out,
                          cudaStream_t st);
 // Launch shape of the spectral-radius kernel for n_u values of which the largest is u_max.

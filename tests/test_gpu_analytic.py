@@ -147,3 +147,30 @@ def test_rho_to_rounding():
     assert np.all(np.abs(alone - ref) <= 2.2e-14 * ref), (alone - ref) / ref
     for k in (9, 12, len(us)):
         assert np.all(np.abs(cr_amin_rho(us[:k]) - ref[:k]) <= 2.2e-14 * ref[:k])
+
+
+def test_lemma_from_several_threads():
+    """Threads with short, long and the longest histograms at once: the kernel's shared-memory limit is
+    shared by all of them."""
+    import threading
+
+    from paper_2508_14544_gb300 import cr_amin_lemma
+    rng = np.random.default_rng(13)
+    xs = [rng.random((3, n)) for n in (8192, 2100, 4000, 40)]
+    want = [cr_amin_lemma(x, 1, 0.0) for x in xs]
+    wrong = []
+
+    def work(x, w):
+        try:
+            for _ in range(300):
+                if not np.array_equal(cr_amin_lemma(x, 1, 0.0), w):
+                    wrong.append("value")
+        except Exception as e:
+            wrong.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=xw) for xw in zip(xs, want)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong, wrong[:3]
