@@ -351,9 +351,10 @@ static int load_impl(sim_ctx *c, const int64_t *offsets, const int32_t *a, const
     sp.rec = c->d_rec;
     sp.rec_a = c->d_rec_a;
     sp.info = c->d_info;
-    e = simgb::launch_stage(sp, ls);
+    int launches = 0;
+    e = simgb::launch_stage(sp, ls, &launches);
     if (e != cudaSuccess) return cuda_fail(c, e, "sim_load: staging kernel launch");
-    if (c->n_inst > 0) ++c->launches;
+    c->launches += launches;
     e = cudaStreamSynchronize(ls);
     if (e != cudaSuccess) return cuda_fail(c, e, "sim_load: staging kernel");
     c->seeds_pending = false;

@@ -111,7 +111,7 @@ __host__ __device__ constexpr size_t ws_bytes(int ca, int dcap) {
     return size_t(ca) * 28 + kWsCacheBytes + size_t(dcap) * sizeof(QEnt);
 }
 
-cudaError_t launch_stage(const StageParams &p, cudaStream_t st);
+cudaError_t launch_stage(const StageParams &p, cudaStream_t st, int *launches);
 // Blocks of the kernel that p selects that one SM holds at a time; raises its shared-memory limit.
 cudaError_t run_blocks_per_sm(int policy, const RunParams &p, int warps_per_block, size_t smem_bytes, int *blocks);
 cudaError_t launch_run(int policy, const RunParams &p, int blocks, int warps_per_block, size_t smem_bytes,

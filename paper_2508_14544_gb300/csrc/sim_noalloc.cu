@@ -140,7 +140,8 @@ extern "C" int sim_run_noalloc(int policy, int64_t M, int32_t n_instances, const
     sp.rec = d_rec;
     sp.rec_a = d_rec_a;
     sp.info = d_info;
-    e = simgb::launch_stage(sp, st);
+    int launches = 0;
+    e = simgb::launch_stage(sp, st, &launches);
     if (e != cudaSuccess) return fail(SIM_E_CUDA, "sim_run_noalloc: staging kernel launch failed");
 
     e = cudaMemsetAsync(d_counter, 0, 3 * sizeof(int32_t), st);  // two work cursors, the redo count

@@ -480,7 +480,8 @@ cudaError_t launch_batch_time(const int64_t *sums, const DevResult *res, const d
     return cudaGetLastError();
 }
 
-cudaError_t launch_stage(const StageParams &p, cudaStream_t st) {
+cudaError_t launch_stage(const StageParams &p, cudaStream_t st, int *launches) {
+    *launches = 0;
     if (p.n_inst <= 0) return cudaSuccess;
     // shared memory for the largest instance up to kStageSmemN, rounded up to a power of two
     int np = 1;
@@ -492,7 +493,11 @@ cudaError_t launch_stage(const StageParams &p, cudaStream_t st) {
         if (e != cudaSuccess) return e;
     }
     k_stage<<<p.n_inst, kStageThreads, smem, st>>>(p, np);
-    if (p.n_max > np) k_stage_large<<<p.n_inst, kLargeThreads, 256 * kLargeWarps * sizeof(int32_t), st>>>(p, np);
+    *launches = 1;
+    if (p.n_max > np) {
+        k_stage_large<<<p.n_inst, kLargeThreads, 256 * kLargeWarps * sizeof(int32_t), st>>>(p, np);
+        *launches = 2;
+    }
     return cudaGetLastError();
 }
 

@@ -388,3 +388,15 @@ def test_busy_streams_at_late_steps(pol):
         got, comp = gpu_run(pol, w, completions=True, **opts)
         assert_same(got, ref, tag=f"late pol={pol} {opts}")
         assert np.array_equal(comp, rcomp)
+
+
+def test_launch_count_of_a_load():
+    """One staging kernel, and a second one when an instance has more than 2048 requests."""
+    from paper_2508_14544_gb300 import SIM_HSF, Simulator
+    for n, launches in ((2048, 1), (2049, 2)):
+        one = np.ones(n, np.int64)
+        w = _w([dict(a=0 * one, s=one, l=one, u=one, o=one)], 100)
+        with Simulator(SIM_HSF, w.M, 1) as sim:
+            sim.load_workload(w)
+            assert sim.kernel_launches() == launches
+            assert sim.run()["status"][0] == 0 and sim.kernel_launches() == launches + 1
