@@ -400,3 +400,51 @@ def test_launch_count_of_a_load():
             sim.load_workload(w)
             assert sim.kernel_launches() == launches
             assert sim.run()["status"][0] == 0 and sim.kernel_launches() == launches + 1
+
+
+def _small_ragged(n_max):
+    rng = np.random.default_rng(n_max)
+    parts = []
+    for k in range(2500):
+        n = n_max if k % 500 == 0 else int(rng.integers(0, 40))
+        o = rng.integers(1, 25, n)
+        l = rng.integers(1, o + 1)
+        a = np.sort(rng.integers(0, 30, n)) if k % 2 else np.zeros(n, np.int64)
+        # the first instance holds all its requests at once, in the others they queue
+        parts.append(dict(a=a, s=rng.integers(100, 2000, n) if k else np.ones(n, np.int64), l=l, u=o + 4, o=o))
+    return _w(parts, 11_000)
+
+
+@pytest.mark.parametrize("pol", [0, 1, 2, 3, 4])
+@pytest.mark.parametrize("n_max", [383, 384, 385])
+def test_many_small_instances(pol, n_max):
+    """More instances than 12 per SM: of up to 383 requests the dense copy runs them without being asked; with
+    more requests, a set block size or a set residency the default one does."""
+    w = _small_ragged(n_max)
+    ref, rcomp = oracle_run(pol, w, completions=True)
+    for opts in ({}, {"warps_per_sm": 12}, {"warps_per_block": 4}, {"dense_residency": 1}):
+        got, comp = gpu_run(pol, w, completions=True, **opts)
+        assert_same(got, ref, tag=f"small pol={pol} {n_max} {opts}")
+        assert np.array_equal(comp, rcomp)
+
+
+@pytest.mark.parametrize("pol", [0, 1, 2, 3, 4])
+def test_dense_layout_with_counters(pol):
+    """The dense layout with the instrumented kernel (asked for, and chosen for many small instances): results
+    and batch-time sums equal the oracle's, and the work counters equal the default layout's but for the queue's
+    bytes."""
+    from oracle import plain
+    from paper_2508_14544_gb300 import Simulator
+    from paper_2508_14544_gb300 import workloads as W
+    from tests.gpu_helpers import n_threads
+    for w in (_small_ragged(300), W.make_workload("c2", range(0, 1024, 16))):
+        ref, sums = plain.run_workload(pol, w, n_threads=n_threads(), time_sums=True)
+        counts = []
+        for opts in ({"warps_per_block": 4}, {"dense_residency": 1}, {}):
+            with Simulator(pol, w.M, w.n_instances, batch_time=1, count_work=1, **opts) as sim:
+                sim.load_workload(w)
+                got = sim.run()
+                assert_same(got, ref, tag=f"dense counters pol={pol} {opts}")
+                assert np.array_equal(sim.batch_time_sums(), sums)
+                counts.append(sim.work_counts()[:, :3])
+        assert np.array_equal(counts[0], counts[1]) and np.array_equal(counts[0], counts[2])
