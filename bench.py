@@ -482,6 +482,8 @@ def run_ours(args) -> None:
     hbm_peak = float(_peaks().get("hbm_gbs", 6800.0))
     hbm = {"achieved": wd["hbm_bytes"] / sec / 1e9, "peak": hbm_peak, "unit": "GB/s",
            "frac": wd["hbm_bytes"] / sec / 1e9 / hbm_peak}
+    # the ceiling that the model's work would reach first
+    bound, top = max((("alu", alu), ("smem", smem), ("hbm", hbm)), key=lambda kv: kv[1]["frac"])
 
     # the other configurations, and the latency regime of the 1024-instance workload
     subs = {name: sub_record(name, dev, stream, peaks_live) for name in SUB_WORKLOADS}
@@ -549,17 +551,18 @@ def run_ours(args) -> None:
                                        "frac_of_measured_hbm": round(lemma_gbs / hbm_peak, 3),
                                        "fp64_tflops": round(lemma_tflops, 3),
                                        "frac_of_nominal_fp64_1.25": round(lemma_tflops / 1.25, 3)}},
-        "roofline": {"bound": "alu", "kernel": f"k_run<{POLICY_NAMES[dom]}>",
-                     "achieved": alu["achieved"], "peak": alu["peak"], "unit": alu["unit"], "frac": alu["frac"],
+        "roofline": {"bound": bound, "kernel": f"k_run<{POLICY_NAMES[dom]}>",
+                     "achieved": top["achieved"], "peak": top["peak"], "unit": top["unit"], "frac": top["frac"],
                      "traffic": _dram_traffic(f"k_run<{POLICY_NAMES[dom]}>"),
-                     "smem": smem, "hbm": hbm,
+                     "alu": alu, "smem": smem, "hbm": hbm,
                      "peaks": "measured live by sim_measure_peaks (integer issue: add/xor chains; shared memory: "
                               "conflict-free 16-byte loads); HBM: MEASURED_PEAKS.json copy bandwidth",
                      "work_per_launch": wd,
                      "model": "work of the per-step method (Theorem complexity) counted by SIM_OPT_COUNT_WORK: "
                               "4 ops/8 B per request-step, 1 op per S2 add, 3 ops/8 B per S3 compare-exchange, "
                               "6 ops/16 B per S5 endpoint evaluation, 1 op/16 B per S4 queue operation; "
-                              "achieved = that work / the launch's CUDA-event time"},
+                              "achieved = that work / the launch's CUDA-event time; the kernel computes the same "
+                              "outputs without executing that work, so a fraction may pass 1"},
         "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
         "gpu_launches": launches,
         "clocks": clocks,
