@@ -307,7 +307,9 @@ int64_t sim_kernel_launches(const sim_ctx *ctx);
  * and 262,144 requests per call; larger inputs are rejected with SIM_E_INVAL and a message in
  * sim_last_error(NULL).  The staging kernel checks the offsets it reads against the same limits
  * again: an instance that reaches past them gets status SIM_E_INVAL in its result and nothing of
- * it is staged.  Active sets of up to 512 jobs are simulated in shared memory on the whole GPU, as
+ * it is staged.  A captured call copies the offsets again on every replay; instances may then be
+ * larger than at capture, within these limits, as long as their active sets fit the slots.  Active
+ * sets of up to 512 jobs are simulated in shared memory on the whole GPU, as
  * by sim_run; the instances that outgrow it run afterwards on the array's global-memory workspaces,
  * 128 at a time.  All calls share that array and it keeps the last call's contents: calls that
  * overlap on the GPU (different streams or threads) race; calls on one stream are safe.

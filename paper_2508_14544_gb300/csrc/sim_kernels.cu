@@ -702,10 +702,10 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
     const auto promotions = [&]() { return P.mainbuf + 2 * (P.main_cap > 0 ? warp_slot() * P.main_cap : base); };
     const auto load_head = [&]() { h = queue_head<POL>(w, q, hsrc, hL); };
 
-    // The conditions of all warp-uniform branches below are warp reductions: the compiler then knows
-    // that they are uniform and emits plain jumps (about 12 cycles) instead of reconvergence blocks
-    // (about 45, measured), and one reduction (29) decides several of them.  Single-value stores are
-    // made by all lanes alike, for the same reason.
+    // The conditions of all branches below that the whole warp takes alike are results of warp reductions:
+    // such a branch costs about 12 cycles, one on another value that the lanes happen to share about 45
+    // (both measured), and one reduction (29) decides several of them.  Single-value stores are made by all
+    // lanes alike, for the same reason.
     for (;;) {
         if (!SMEM && P.debug && attn == 0 &&
             !state_ok<POL>(w, q, A, end, t, need, int(nextF), py, pc, qy, qc, filled, ct, cv)) {
@@ -1128,7 +1128,7 @@ __device__ __forceinline__ void sim_instance(const RunParams &P, const Ws &w0, i
             nextF = __reduce_min_sync(FULL, f);
             if (POL == P_AELL) nextE = __reduce_min_sync(FULL, e1);
             if (kEarly) {
-                // decided on reductions (uniform jumps); the first update is left pending if none is
+                // decided on reductions, as above; the first update is left pending if none is
                 const int most = __reduce_max_sync(FULL, ne), tot = int(__reduce_add_sync(FULL, unsigned(ne)));
                 const int e1st = __reduce_max_sync(FULL, ek), b1st = __reduce_max_sync(FULL, bk);
                 const bool free_q = __reduce_max_sync(FULL, qy) < 0;

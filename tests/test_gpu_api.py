@@ -144,7 +144,7 @@ def test_residency_tuning():
 
 @pytest.mark.parametrize("pol", [0, 1, 2, 3, 4])
 def test_dense_residency(pol):
-    """SIM_OPT_DENSE_RESIDENCY (12 warps per SM, 384 shared-memory slots) gives the oracle's results;
+    """SIM_OPT_DENSE_RESIDENCY (16 warps per SM, 384 shared-memory slots) gives the oracle's results;
     an instance of 1000 one-token-prompt jobs holds more than 384 of them at once and is re-run in
     global memory (two launches)."""
     from paper_2508_14544_gb300 import workloads as W
@@ -233,9 +233,8 @@ def test_unsorted_arrivals():
 
 
 def test_long_requests_narrow_and_wide_kernels_agree():
-    """Lengths of ~3e5 steps: with the default 512-slot shared-memory capacity the 32-bit kernel is
-    valid (512 x (2 lmax + 2) + 2^27 < 2^31); with a 4096-slot capacity it is not, so every
-    instance is re-run by the 64-bit global-memory kernel.  Both equal the oracle."""
+    """Lengths of ~3e5 steps under a memory limit of 10^6: the kernel's 32-bit sums hold with the default 512
+    shared-memory slots and with 4096.  Both equal the oracle."""
     from paper_2508_14544_gb300 import workloads as W
     rng = np.random.default_rng(21)
     parts = []
@@ -315,8 +314,8 @@ def test_debug_checks_hold_and_change_nothing(pol):
 
 
 def test_largest_memory_limit():
-    """M = 2^26 (the largest the ABI accepts) with requests of up to ~2^25 tokens: the 32-bit
-    bound fails, so the 64-bit kernel runs every instance; results equal the oracle (which steps
+    """M = 2^26 (the largest the ABI accepts) with requests of up to ~2^25 tokens: the largest
+    memory sums that the kernel's 32 bits have to hold; results equal the oracle (which steps
     every one of the ~10^8 batches)."""
     from paper_2508_14544_gb300 import workloads as W
     M = 1 << 26

@@ -65,7 +65,7 @@ def test_random_tiny_batch(pol, arrivals):
 
 def _random_mixed_workload(seed, M):
     """Instance sizes around the kernel's size thresholds (delta capacity 64 / 128 / 256 at 1024 /
-    4096 requests, one-chunk active sets up to 128 jobs, windows of 32), random accuracy, memory
+    4096 requests, half pages of 64 slots and pages of 128), random accuracy, memory
     limits from tight to loose, and arrivals at t=0, spread out, or in bursts."""
     from fractions import Fraction
 
@@ -92,7 +92,7 @@ def _random_mixed_workload(seed, M):
 
 def _staging_workload(seed):
     """Instances sized around the staging sort's boundaries (radix passes take 256 elements per
-    round, shared memory holds up to 2048 requests, larger ones go to the global-memory sort), with
+    round, shared memory holds up to 2048 requests, larger ones are sorted in global memory), with
     arrival steps in random order over a wide range (several arrival-digit passes) and keys drawn
     from a few values (long runs of ties, which the sort must keep in index order)."""
     from fractions import Fraction
