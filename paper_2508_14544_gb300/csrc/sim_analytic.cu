@@ -167,14 +167,20 @@ __global__ void __launch_bounds__(256) k_lemma(int32_t n_hist, int32_t len, int3
     if (g == 0 && h < n_hist) out[h] = num / den;
 }
 
+// Blocks of 256 threads, or of one warp for small u: threads without an index take part in the scans all the
+// same, and those keep the FP64 pipes busy (10^5 values of u = 7: 42.4 ms with 256 threads, 7.1 with one warp;
+// of u = 128: 45.8 and 14.0).  A few values fill no pipe and gain from more threads above one index per lane
+// (u = 7: 0.215 and 0.192 ms, u = 128: 0.212 and 0.244).
 constexpr int kRhoThreads = 256;
+static int rho_threads(int32_t n_u, int32_t u_max) { return u_max <= (n_u > 1024 ? 128 : 32) ? 32 : kRhoThreads; }
 constexpr size_t kRhoSmemMax = size_t(200) * 1024;
 constexpr int kRhoArrays = 7;  // per i: S, T, 1/(i(i-1)), 1/(8(2i-1)), w_i, 3 - 2/i, 2i - 1
 
-__global__ void __launch_bounds__(kRhoThreads) k_rho(const int32_t *__restrict__ us, double *__restrict__ out,
+template <int NT>
+__global__ void __launch_bounds__(NT) k_rho(const int32_t *__restrict__ us, double *__restrict__ out,
                                                       double *scratch, int64_t stride, int32_t max_iter) {
     namespace cg = cooperative_groups;
-    constexpr int kW = kRhoThreads / 32;
+    constexpr int kW = NT / 32;
     extern __shared__ double rho_smem[];
     __shared__ double wsum[5][kW];  // per warp: p1, Q, T, numerator, denominator
     __shared__ double part[2][5];   // per block, double-buffered over steps, read by the cluster
@@ -186,7 +192,7 @@ __global__ void __launch_bounds__(kRhoThreads) k_rho(const int32_t *__restrict__
     // this block's indices [lo, hi) (0-based: entry e is i = e + 1), this thread's [a, b)
     const int R = (u + C - 1) / C;
     const int lo = min(rank * R, u), hi = min(lo + R, u);
-    const int m = ((hi - lo + kRhoThreads - 1) / kRhoThreads) | 1;  // odd: the runs start on different banks
+    const int m = ((hi - lo + NT - 1) / NT) | 1;  // odd: the runs start on different banks
     const int a = min(lo + tid * m, hi), b = min(a + m, hi);
     // arrays over the block's indices, in shared memory or in the scratch of this u
     double *S = scratch ? scratch + id * stride + int64_t(kRhoArrays) * lo : rho_smem;
@@ -322,7 +328,7 @@ static size_t rho_smem_bytes(int cluster, int32_t u_max) {
 static cudaLaunchConfig_t rho_config(const RhoPlan &plan, int32_t n_u, cudaLaunchAttribute *attr, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(n_u) * unsigned(plan.cluster));
-    cfg.blockDim = dim3(kRhoThreads);
+    cfg.blockDim = dim3(unsigned(plan.threads));
     cfg.dynamicSmemBytes = plan.smem;
     cfg.stream = st;
     attr->id = cudaLaunchAttributeClusterDimension;
@@ -337,9 +343,10 @@ static cudaLaunchConfig_t rho_config(const RhoPlan &plan, int32_t n_u, cudaLaunc
 // in to) for a few values: a GPU partition holds few clusters of 16, and 25 values of up to 20,000 took
 // 0.79 ms with 16 blocks each, one of 10^5 0.70 ms (8 blocks: 1.0).
 cudaError_t rho_plan(int32_t n_u, int32_t u_max, RhoPlan *plan) {
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_rho, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kRhoSmemMax));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute((const void *)k_rho, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaError_t e = cudaFuncSetAttribute((const void *)k_rho<kRhoThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kRhoSmemMax));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute((const void *)k_rho<kRhoThreads>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
+    plan->threads = rho_threads(n_u, u_max);
     const int most = n_u <= 8 ? 16 : 8;
     plan->cluster = 1;
     while (plan->cluster < most && 512 * plan->cluster < u_max) plan->cluster <<= 1;
@@ -348,7 +355,7 @@ cudaError_t rho_plan(int32_t n_u, int32_t u_max, RhoPlan *plan) {
         cudaLaunchAttribute attr;
         const cudaLaunchConfig_t cfg = rho_config(*plan, 1, &attr, nullptr);
         int fit = 0;
-        if (cudaOccupancyMaxActiveClusters(&fit, k_rho, &cfg) != cudaSuccess || fit < 1) {
+        if (cudaOccupancyMaxActiveClusters(&fit, k_rho<kRhoThreads>, &cfg) != cudaSuccess || fit < 1) {
             cudaGetLastError();
             plan->cluster = 8;
             plan->smem = rho_smem_bytes(8, u_max);
@@ -363,7 +370,8 @@ cudaError_t launch_rho(const RhoPlan &plan, int32_t n_u, const int32_t *us, doub
     if (n_u <= 0) return cudaSuccess;
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = rho_config(plan, n_u, &attr, st);
-    return cudaLaunchKernelEx(&cfg, k_rho, us, out, scratch, plan.scratch, max_iter);
+    return cudaLaunchKernelEx(&cfg, plan.threads == 32 ? k_rho<32> : k_rho<kRhoThreads>, us, out, scratch, plan.scratch,
+                              max_iter);
 }
 
 }  // namespace simgb

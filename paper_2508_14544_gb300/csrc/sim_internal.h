@@ -124,6 +124,7 @@ cudaError_t launch_lemma(int32_t n_hist, int32_t len, int32_t l, double s, const
                          cudaStream_t st);
 // Launch shape of the spectral-radius kernel for n_u values of which the largest is u_max.
 struct RhoPlan {
+    int threads;      // per block
     int cluster;      // blocks per value
     size_t smem;      // bytes of shared memory per block, 0 when the arrays live in scratch
     int64_t scratch;  // doubles of global scratch per value (0: none, and scratch must be null)

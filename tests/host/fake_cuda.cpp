@@ -169,7 +169,7 @@ cudaError_t launch_batch_time(const int64_t *, const DevResult *, const double *
 }
 cudaError_t launch_lemma(int32_t, int32_t, int32_t, double, const double *, double *, cudaStream_t) { return cudaSuccess; }
 cudaError_t rho_plan(int32_t, int32_t u_max, RhoPlan *plan) {
-    *plan = {8, 0, 7 * int64_t(u_max)};
+    *plan = {256, 8, 0, 7 * int64_t(u_max)};
     return cudaSuccess;
 }
 cudaError_t launch_rho(const RhoPlan &, int32_t n_u, const int32_t *us, double *out, double *, int32_t, cudaStream_t) {

@@ -141,12 +141,14 @@ def test_rho_to_rounding():
     1.1e-16 each in numerator and denominator."""
     from oracle import analytic as an
     from paper_2508_14544_gb300 import cr_amin_rho
-    us = [1, 2, 3, 10, 33, 100, 512, 513, 1025, 2049, 8193, 20000, 33000, 58500, 58600]
+    us = [1, 2, 3, 10, 31, 32, 33, 127, 128, 129, 512, 513, 1025, 2049, 8193, 20000, 33000, 58500, 58600]
     ref = np.array([an.rho_long(u) for u in us])
     alone = np.array([cr_amin_rho([u])[0] for u in us])
     assert np.all(np.abs(alone - ref) <= 2.2e-14 * ref), (alone - ref) / ref
-    for k in (9, 12, len(us)):
+    for k in (3, 9, 12, 15, len(us)):
         assert np.all(np.abs(cr_amin_rho(us[:k]) - ref[:k]) <= 2.2e-14 * ref[:k])
+    k = us.index(129)  # one warp per value when there are many small ones
+    assert np.all(np.abs(cr_amin_rho(us[:k] * 200).reshape(200, k) - ref[:k]) <= 2.2e-14 * ref[:k])
 
 
 def test_lemma_from_several_threads():
