@@ -3,6 +3,7 @@
 import ctypes
 import shutil
 import subprocess
+from pathlib import Path
 
 import numpy as np
 import pytest
@@ -14,9 +15,11 @@ A_MIN, NOMEM = 1, -6
 
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
-    cxx, cuda = shutil.which("g++"), "/usr/local/cuda/include"
+    from paper_2508_14544_gb300.build import nvcc
+    cxx = shutil.which("g++")
     if not cxx:
         pytest.skip("no host compiler")
+    cuda = Path(nvcc()).resolve().parent.parent / "include"
     so = tmp_path_factory.mktemp("host") / "libhost.so"
     csrc = ROOT / "paper_2508_14544_gb300" / "csrc"
     subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", f"-I{ROOT / 'include'}", f"-I{csrc}",
